@@ -15,9 +15,7 @@
 
 namespace lbib {
 
-constexpr int kPts = 32;          // MLS points per block
-constexpr int kMlsThreads = 256;  // 8 warps, 4 points each
-static_assert(kPts <= 32 && kPts % (kMlsThreads / 32) == 0, "one lane per point in phases 0 and 2");
+constexpr int kMlsThreads = 64;   // MLS points (threads) per block
 constexpr double kAlpha = 0.3;    // Eq. (intKernel)
 constexpr double kRw = 1.3;       // support size r_w (Sec. 2.2)
 constexpr double kProbe = 1.2;    // probe length (Sec. 2.3)
@@ -136,51 +134,7 @@ __global__ void __launch_bounds__(256) k_moments(const S *__restrict__ fin, Latt
     moments_body<S, R>(fin, L, box, box_next, mom, step_inc, blockIdx.x, gridDim.x);
 }
 
-constexpr int kSums = 26;  // A (10 entries), b for rho (4), b for u (12)
-
-// Shared memory of the MLS phases.  The per-point sums are formed through a
-// shared-memory transpose (red) in the MLS kernels, which run alone and are
-// fastest that way, or with kShfl by warp shuffles (the persistent batched
-// step, whose shared memory is taken from the L1 its sweep items need).
-template <typename R, bool kShfl = false>
-struct MlsSmem {
-    // per point, filled in phase 0 (one lane per point)
-    double frac[kPts][3];  // X - base, exact
-    int base[kPts][3];
-    R fracR[kPts][3];
-    R nrm[kPts][3];
-    double vol[kPts];
-    // per point and support node, kept for the transfer weights of markers
-    // (with kShfl the offsets x_k - X are formed again from fracR instead)
-    R W[kPts][27];
-    R d[kShfl ? 1 : kPts][27][3];
-    // per point: A = sum W p p^T, b_f = sum W p (f - f_c) for f = rho - 1, u_x, u_y, u_z
-    R sums[kPts][kSums];
-    R ref[kPts][4];   // the fitted fields at the support's centre node (the fits are of f - ref)
-    R row0[kPts][4];  // first row of A^-1
-    int pid[kPts];    // point of each slot (-1 past the end): slots follow the body's cell order
-    // per warp: transpose buffer of the 26 products of each node (unused with kShfl)
-    R red[kShfl ? 1 : kMlsThreads / 32][kSums][kShfl ? 1 : 33];
-};
-
-// Sums 32 values per lane over the warp (a reduce-scatter butterfly): at
-// offset h each lane keeps the half of its values whose index bit h it
-// holds and receives the partner's partial sums of that half, so that lane
-// q ends with the total of value q (31 shuffles, no shared memory).
-template <typename R>
-__device__ __forceinline__ R warp_reduce_scatter32(R (&v)[32], const int lane) {
-#pragma unroll
-    for (int h = 16; h >= 1; h >>= 1) {
-        const bool up = (lane & h) != 0;
-#pragma unroll
-        for (int i = 0; i < h; ++i) {
-            const R send = up ? v[i] : v[i + h];
-            const R keep = up ? v[i + h] : v[i];
-            v[i] = keep + __shfl_xor_sync(0xffffffffu, send, h);
-        }
-    }
-    return v[0];
-}
+constexpr int kRec = 16;  // R values of a marker's transfer record (BodyView::phi)
 
 // 1/d in FP64 from the FP32 reciprocal refined by two Newton steps
 // (relative error ~1e-7 -> ~1e-14 -> below the double rounding).  d must lie
@@ -204,7 +158,7 @@ __device__ __forceinline__ double recip64(double d) {
 // keep det above ~1e-16; a determinant outside the bounds marks a singular
 // support.
 constexpr double kMinDet = 1e-30, kMaxDet = 1e30;
-__device__ bool spd_inverse4(const double *a, double *inv) {
+__device__ __forceinline__ bool spd_inverse4(const double *a, double *inv) {
     const double m00 = a[0], m01 = a[1], m02 = a[2], m03 = a[3];
     const double m11 = a[4], m12 = a[5], m13 = a[6], m22 = a[7], m23 = a[8], m33 = a[9];
     // rows 0,1 and rows 2,3 (symmetric: m10 = m01, ...)
@@ -243,53 +197,45 @@ __device__ bool spd_inverse4(const double *a, double *inv) {
     return true;
 }
 
-// Inverse of a symmetric positive definite 4x4 matrix (upper triangle as for
-// spd_inverse4) in FP32, by Cholesky: A = L L^T, M = L^-1 by forward
-// substitution, A^-1 = M^T M.  Backward stable, so for moment sums that are
-// themselves FP32 it is as accurate as an FP64 inverse of the same sums
-// (both leave errors of the order of the sums' own rounding in the fits),
-// at FP32 issue rates.  Returns false unless every pivot is positive and
-// finite (a singular support).
-__device__ bool spd_inverse4_chol(const float *a, float *inv) {
-    const float d0 = a[0];
-    if (!(d0 > 0.f && d0 < 1e30f)) return false;
-    const float l00 = sqrtf(d0), r0 = 1.f / l00;
+// The same in FP32 by the root-free Cholesky factors A = L D L^T (L unit
+// lower triangular, M = L^-1): A^-1 = M^T D^-1 M.  Backward stable, so for
+// moment sums that are themselves FP32 it is as accurate as an FP64 inverse
+// of the same sums (both leave errors of the order of the sums' own rounding
+// in the fits), at FP32 issue rates.  Returns false unless every pivot is
+// positive and finite (a singular support).
+__device__ __forceinline__ bool spd_inverse4(const float *a, float *inv) {
+    const float d0 = a[0], r0 = rcp(d0);
     const float l10 = a[1] * r0, l20 = a[2] * r0, l30 = a[3] * r0;
-    const float d1 = a[4] - l10 * l10;
-    if (!(d1 > 0.f)) return false;
-    const float l11 = sqrtf(d1), r1 = 1.f / l11;
-    const float l21 = (a[5] - l20 * l10) * r1, l31 = (a[6] - l30 * l10) * r1;
-    const float d2 = a[7] - l20 * l20 - l21 * l21;
-    if (!(d2 > 0.f)) return false;
-    const float l22 = sqrtf(d2), r2 = 1.f / l22;
-    const float l32 = (a[8] - l30 * l20 - l31 * l21) * r2;
-    const float d3 = a[9] - l30 * l30 - l31 * l31 - l32 * l32;
-    if (!(d3 > 0.f)) return false;
-    const float r3 = 1.f / sqrtf(d3);
-    // M = L^-1 (lower triangular)
-    const float m00 = r0;
-    const float m10 = -l10 * m00 * r1, m11 = r1;
-    const float m20 = -(l20 * m00 + l21 * m10) * r2, m21 = -l21 * m11 * r2, m22 = r2;
-    const float m30 = -(l30 * m00 + l31 * m10 + l32 * m20) * r3, m31 = -(l31 * m11 + l32 * m21) * r3,
-                m32 = -l32 * m22 * r3, m33 = r3;
-    // (M^T M)_ij = sum_{k >= max(i, j)} m_ki m_kj
-    inv[0] = m00 * m00 + m10 * m10 + m20 * m20 + m30 * m30;
-    inv[1] = m10 * m11 + m20 * m21 + m30 * m31;
-    inv[2] = m20 * m22 + m30 * m32;
-    inv[3] = m30 * m33;
-    inv[5] = m11 * m11 + m21 * m21 + m31 * m31;
-    inv[6] = m21 * m22 + m31 * m32;
-    inv[7] = m31 * m33;
-    inv[10] = m22 * m22 + m32 * m32;
-    inv[11] = m32 * m33;
-    inv[15] = m33 * m33;
+    const float d1 = a[4] - l10 * a[1], r1 = rcp(d1);
+    const float t21 = a[5] - l10 * a[2], t31 = a[6] - l10 * a[3];
+    const float l21 = t21 * r1, l31 = t31 * r1;
+    const float d2 = a[7] - l20 * a[2] - l21 * t21, r2 = rcp(d2);
+    const float t32 = a[8] - l20 * a[3] - l21 * t31;
+    const float l32 = t32 * r2;
+    const float d3 = a[9] - l30 * a[3] - l31 * t31 - l32 * t32, r3 = rcp(d3);
+    // M = L^-1
+    const float m10 = -l10, m21 = -l21, m32 = -l32;
+    const float m20 = l21 * l10 - l20;
+    const float m31 = l32 * l21 - l31;
+    const float m30 = -l30 - l31 * m10 - l32 * m20;
+    const float q10 = m10 * r1, q20 = m20 * r2, q21 = m21 * r2, q30 = m30 * r3, q31 = m31 * r3, q32 = m32 * r3;
+    inv[0] = r0 + m10 * q10 + m20 * q20 + m30 * q30;
+    inv[1] = q10 + m20 * q21 + m30 * q31;
+    inv[2] = q20 + m30 * q32;
+    inv[3] = q30;
+    inv[5] = r1 + m21 * q21 + m31 * q31;
+    inv[6] = q21 + m31 * q32;
+    inv[7] = q31;
+    inv[10] = r2 + m32 * q32;
+    inv[11] = q32;
+    inv[15] = r3;
     inv[4] = inv[1];
     inv[8] = inv[2];
     inv[9] = inv[6];
     inv[12] = inv[3];
     inv[13] = inv[7];
     inv[14] = inv[11];
-    return true;
+    return d0 > 0.f && d0 < 1e30f && d1 > 0.f && d2 > 0.f && d3 > 0.f;
 }
 
 // Squared distance with the products and sums rounded one by one in the
@@ -298,301 +244,161 @@ __device__ __forceinline__ double dist2_exact(double a, double b, double c) {
     return __dadd_rn(__dadd_rn(__dmul_rn(a, a), __dmul_rn(b, b)), __dmul_rn(c, c));
 }
 
-// MLS at markers and probes, 32 points per block.  Points 0..nm-1 are the
+// The FP64 decision r_k <= 1 for the support nodes in `near` (bit i + 3 j +
+// 9 k: offsets i - 1, j - 1, k - 1 from the point's base node).
+__device__ __noinline__ unsigned support_exact(unsigned near, double fx, double fy, double fz, double cut) {
+    unsigned in = 0u;
+    while (near) {
+        const int q = __ffs((int)near) - 1;
+        near &= near - 1u;
+        const double e0 = (double)(q % 3 - 1) - fx, e1 = (double)((q / 3) % 3 - 1) - fy, e2 = (double)(q / 9 - 1) - fz;
+        if (dist2_exact(e0, e1, e2) <= cut) in |= 1u << q;
+    }
+    return in;
+}
+
+// One axis of the support weight W = exp(-(r/alpha)^2) of Eq. (intKernel),
+// which is a product over the axes: w[i] = exp(-(d[i]/(r_w alpha))^2) at the
+// offsets d[i] = i - 1 - f.  (Each from its own exponential: opposite offsets
+// then have equal weights, and the sums of a mirrored support mirror exactly.)
+template <typename R>
+__device__ __forceinline__ void axis_weights(R f, R *d, R *w) {
+#pragma unroll
+    for (int i = 0; i < 3; ++i) {
+        d[i] = R(i - 1) - f;
+        const R t = d[i] * R(1.0 / (kRw * kAlpha));
+        w[i] = exp(-(t * t));
+    }
+}
+
+// A node coordinate's image on the lattice; on walled axes bases are clamped
+// so that the support lies inside.
+__device__ __forceinline__ int support_coord(const Lattice &L, int a, int c) {
+    const int n = a == 0 ? L.nx : a == 1 ? L.ny : L.nz;
+    if (L.bc[a] != kPeriodic) return c;
+    if (c < 0)
+        c += n;
+    else if (c >= n)
+        c -= n;
+    return wrap_periodic(c, n);
+}
+
+// Transfer record of marker p: row 0 of A^-1 (4), the offset X - base (3) and
+// the three axes' weights (9), from which every support node's transfer
+// weight phi_k = W_k (A^-1 p_k)_0 follows; base node and the bits of the
+// nodes with r_k <= 1 in node[4 p ..].
+__device__ __forceinline__ void store_record(float *rec, const float *v) {
+#pragma unroll
+    for (int q = 0; q < kRec / 4; ++q)
+        reinterpret_cast<float4 *>(rec)[q] = make_float4(v[4 * q], v[4 * q + 1], v[4 * q + 2], v[4 * q + 3]);
+}
+__device__ __forceinline__ void store_record(double *rec, const double *v) {
+#pragma unroll
+    for (int q = 0; q < kRec / 2; ++q) reinterpret_cast<double2 *>(rec)[q] = make_double2(v[2 * q], v[2 * q + 1]);
+}
+
+// MLS at markers and probes, one thread per point.  Points 0..nm-1 are the
 // markers (the vertices, or the triangle centroids); point nm + 2t + side is
 // the probe of triangle t on the outer (side 0) or inner (side 1) face.  With p_k = (1, x_k - X) the fit of a
 // field f is a = A^-1 b_f, A = sum_k W_k p_k p_k^T, b_f = sum_k W_k p_k f_k
 // (Eq. l2norm), i.e. f(X) = a_0 and grad f = (a_1, a_2, a_3).
-//  phase 0: one lane per point: position (probes: triangle geometry), the
-//           nearest node base = floor(X + 1/2) and the exact offset X - base;
-//  phase 1: one warp per point, one lane per support node: weight
-//           W = exp(-(r/alpha)^2) for r <= 1 (the cut-off decided exactly as
-//           in FP64), node moments less those of the centre node f_c, the
-//           26 products W p p^T and W p (f - f_c), summed over the nodes;
-//  phase 2: one lane per point: inverse of A (FP64 adjugate in the FP64
-//           path, FP32 Cholesky in the FP32 one); markers get
-//           U = (A^-1 b_u)_0 + u_c (Eq. uLag), probes the pressure c_s^2 rho and
-//           the traction rho nu (grad u + grad u^T) . n from the fits;
-//  phase 3: markers keep phi_k = W_k (A^-1 p_k)_0 for spreading.
-template <typename R, bool kCG = false, bool kShfl = false>
+//  positions: the point (probes: triangle geometry), the nearest node base =
+//           floor(X + 1/2) and the exact offset X - base; enclosed volume.
+//           Nothing here reads the moments: with kChain it runs while the
+//           moments kernel ends;
+//  sums:    W is a product over the axes but for its cut-off r_k <= 1 (a bit
+//           per node, decided exactly as in FP64), so the ten sums of A and
+//           the sixteen of b (fields less those of the centre node) are formed
+//           axis by axis: x within each row of three nodes, then y, then z
+//           (about 800 operations a point; 1250 when formed node by node);
+//  solve:   inverse of A (FP64 adjugate in the FP64 path, FP32 L D L^T in
+//           the FP32 one); markers get U = (A^-1 b_u)_0 + u_c (Eq. uLag),
+//           probes the pressure c_s^2 rho and the traction
+//           rho nu (grad u + grad u^T) . n from the fits.
+template <typename R, bool kCG = false, bool kChain = false>
 __device__ __forceinline__ void mls_body(const R *__restrict__ mom, const Lattice &L, const BodyView &B, int *err,
-                                         MlsSmem<R, kShfl> &sm, const int vb, const int nvb) {
+                                         const int vb, const int nvb) {
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     const int nm = B.nm, npts = nm + 2 * B.nt;
-    const int p0 = vb * kPts;
-    const int nxy = L.nx * L.ny;
+    const int slot = vb * blockDim.x + threadIdx.x;
     const int n[3] = {L.nx, L.ny, L.nz};
+    const int p = slot < npts ? (B.perm ? B.perm[slot] : slot) : -1;
 
-    // The lane-per-point phases (0 and 2) run FP64 code; FP64 issues per
-    // warp-instruction on one SM sub-partition, so blocks rotate the warp
-    // that runs them over the four sub-partitions.
-    const int w0 = vb & 3, w2 = (vb + 2) & 3;
-
-    // ---------------- phase 0: one lane per point ----------------
-    if (warp == w0 && lane < kPts) {
-        const int slot = p0 + lane;
-        const int p = slot < npts ? (B.perm ? B.perm[slot] : slot) : -1;
-        sm.pid[lane] = p;
-        sm.vol[lane] = 0.0;
-        if (p >= 0) {
-            double P[3];
-            if (p < nm && B.centroid) {
-                const int *tv = B.tri + 3 * p;
-                for (int a = 0; a < 3; ++a) P[a] = (B.X[3 * tv[0] + a] + B.X[3 * tv[1] + a] + B.X[3 * tv[2] + a]) / 3.0;
-            } else if (p < nm) {
-                P[0] = B.X[3 * p];
-                P[1] = B.X[3 * p + 1];
-                P[2] = B.X[3 * p + 2];
-            } else {
-                // probe X_c +- 1.2 n, with X_c = x_0 + (e1 + e2)/3 and the
-                // triangle's edges and normal from origin-relative positions
-                const int t = (p - nm) >> 1, side = (p - nm) & 1;
-                const int *tv = B.tri + 3 * t;
-                const R *Xr = (const R *)B.Xrel;
-                R r0[3], e1[3], e2[3];
-                for (int a = 0; a < 3; ++a) {
-                    r0[a] = Xr[3 * tv[0] + a];
-                    e1[a] = Xr[3 * tv[1] + a] - r0[a];
-                    e2[a] = Xr[3 * tv[2] + a] - r0[a];
-                }
-                const R N[3] = {e1[1] * e2[2] - e1[2] * e2[1], e1[2] * e2[0] - e1[0] * e2[2],
-                                e1[0] * e2[1] - e1[1] * e2[0]};
-                const R nn = sqrt(N[0] * N[0] + N[1] * N[1] + N[2] * N[2]);
-                const R inn = R(1) / nn, sg = side ? R(-kProbe) : R(kProbe);
-                for (int a = 0; a < 3; ++a) {
-                    const R nr = N[a] * inn, c3 = (e1[a] + e2[a]) / R(3);
-                    sm.nrm[lane][a] = nr;
-                    P[a] = B.X[3 * tv[0] + a] + (double)(c3 + sg * nr);
-                    if (side == 0) {
-                        R *tg = (R *)B.tri_geo + 8 * t;
-                        tg[a] = nr;
-                        tg[4 + a] = r0[a] + c3;
-                    }
-                }
-                if (side == 0) {
-                    ((R *)B.tri_geo)[8 * t + 3] = R(0.5) * nn;
-                    const double v6 = (double)r0[0] * (double)N[0] + (double)r0[1] * (double)N[1] +
-                                      (double)r0[2] * (double)N[2];
-                    B.tri_vol[t] = v6;
-                    sm.vol[lane] = v6;
-                }
-            }
-            bool bad = false, diverged = false;
-            for (int a = 0; a < 3; ++a) {
-                if (!(fabs(P[a]) < kMaxMarkerCoord)) {  // non-finite or runaway: flag, keep indices sane
-                    diverged = true;
-                    P[a] = 0.0;
-                }
-                int b = __double2int_rd(P[a] + 0.5);  // floor(X + 1/2)
-                if (L.bc[a] == kWall && (b - 1 < 1 || b + 1 > n[a] - 2)) {
-                    bad = true;
-                    b = b < 2 ? 2 : (b > n[a] - 3 ? n[a] - 3 : b);
-                }
-                sm.base[lane][a] = b;
-                sm.frac[lane][a] = P[a] - (double)b;
-                sm.fracR[lane][a] = R(sm.frac[lane][a]);
-            }
-            if (diverged)
-                atomicCAS(err, 0, kErrDiverged);
-            else if (bad)
-                atomicCAS(err, 0, kErrBodyWall);
-        }
-    }
-    __syncthreads();
-
-    // ---------------- phase 1: one warp per point, one lane per node ----------------
-    // The gathers of the warp's points are issued together, then each
-    // point's weights and products are reduced in turn.
-    constexpr int kPerWarp = kPts / (kMlsThreads / 32);
-    R gu[kPerWarp][4];
-#pragma unroll
-    for (int j = 0; j < kPerWarp; ++j) {
-        const int lp = warp * kPerWarp + j;
-        const int p = sm.pid[lp];
-        gu[j][0] = gu[j][1] = gu[j][2] = gu[j][3] = R(0);
-        if (p >= 0 && lane < 27) {
-            const int dd[3] = {lane % 3 - 1, (lane / 3) % 3 - 1, lane / 9 - 1};
-            int cw[3];
-            for (int a = 0; a < 3; ++a) {
-                int cc = sm.base[lp][a] + dd[a];
-                if (L.bc[a] == kPeriodic) {
-                    if (cc < 0)
-                        cc += n[a];
-                    else if (cc >= n[a])
-                        cc -= n[a];
-                    if (cc < 0 || cc >= n[a]) cc = ((cc % n[a]) + n[a]) % n[a];
-                }
-                cw[a] = cc;
-            }
-            const int node = cw[0] + L.nx * cw[1] + nxy * cw[2];
-            mom_load<kCG>(mom, node, gu[j]);
-            if (p < nm) {
-                gu[j][0] = R(0);  // markers use the velocity fit only
-                B.node[27 * p + lane] = node;
-            }
-        }
-    }
-#pragma unroll
-    for (int j = 0; j < kPerWarp; ++j) {
-        const int lp = warp * kPerWarp + j;
-        const int p = sm.pid[lp];
-        if (p < 0) break;
-        // fit f - f_c, f_c the moments of the centre node (lane 13, always in
-        // the support): the same fit, since MLS reproduces constants, but
-        // the sums and the solve then carry the field's variation over the
-        // support rather than its size, which the gradients at the probes
-        // (small differences of the fitted values) need
-#pragma unroll
-        for (int c = 0; c < 4; ++c) {
-            const R fc = __shfl_sync(0xffffffffu, gu[j][c], 13);
-            gu[j][c] -= fc;
-            if (lane == 0) sm.ref[lp][c] = fc;
-        }
-        R W = R(0), dk[3] = {R(0), R(0), R(0)};
-        if (lane < 27) {
-            const int dd[3] = {lane % 3 - 1, (lane / 3) % 3 - 1, lane / 9 - 1};
-            // x_k - X = dd - (X - base), one rounding like (base + dd) - X
-            for (int a = 0; a < 3; ++a) dk[a] = R(dd[a]) - sm.fracR[lp][a];
-            // support cut-off r_k <= 1 of Eq. (intKernel), decided on the FP64
-            // squared distance; the FP32 path computes it in FP64 only near
-            // the cut-off, where its own rounding could flip the decision
-            bool inside;
-            R dist2;
-            if (sizeof(R) == 8) {
-                dist2 = R(dist2_exact(double(dk[0]), double(dk[1]), double(dk[2])));
-                inside = double(dist2) <= L.dist2_cut;
-            } else {
-                dist2 = dk[0] * dk[0] + dk[1] * dk[1] + dk[2] * dk[2];
-                if (fabsf(float(dist2) - L.dist2_cut_f) > 1e-4f) {
-                    inside = float(dist2) < L.dist2_cut_f;
-                } else {
-                    const double e0 = (double)dd[0] - sm.frac[lp][0], e1 = (double)dd[1] - sm.frac[lp][1],
-                                 e2 = (double)dd[2] - sm.frac[lp][2];
-                    inside = dist2_exact(e0, e1, e2) <= L.dist2_cut;
-                }
-            }
-            if (inside) {
-                const R r = sqrt(dist2) / R(kRw);
-                W = exp(-(r / R(kAlpha)) * (r / R(kAlpha)));
-            }
-            sm.W[lp][lane] = W;
-            if constexpr (!kShfl)
-                for (int a = 0; a < 3; ++a) sm.d[lp][lane][a] = dk[a];
-        }
-        // the 26 products of this node (zero on lanes 27..31), summed over
-        // the support nodes: lane q forms sum q
-        const R Wd[4] = {W, W * dk[0], W * dk[1], W * dk[2]};
-        if constexpr (kShfl) {
-            R v[32];
-            v[0] = Wd[0];
-            v[1] = Wd[1];
-            v[2] = Wd[2];
-            v[3] = Wd[3];
-            v[4] = Wd[1] * dk[0];
-            v[5] = Wd[1] * dk[1];
-            v[6] = Wd[1] * dk[2];
-            v[7] = Wd[2] * dk[1];
-            v[8] = Wd[2] * dk[2];
-            v[9] = Wd[3] * dk[2];
-#pragma unroll
-            for (int q = 0; q < 4; ++q) {
-                v[10 + q] = Wd[q] * gu[j][0];
-                v[14 + q] = Wd[q] * gu[j][1];
-                v[18 + q] = Wd[q] * gu[j][2];
-                v[22 + q] = Wd[q] * gu[j][3];
-            }
-#pragma unroll
-            for (int q = kSums; q < 32; ++q) v[q] = R(0);
-            const R sum = warp_reduce_scatter32(v, lane);
-            if (lane < kSums) sm.sums[lp][lane] = sum;
+    // ---------------- positions ----------------
+    double vol = 0.0, frac[3] = {0.0, 0.0, 0.0};
+    R nrm[3] = {R(0), R(0), R(0)};
+    int base[3] = {2, 2, 2};
+    if (p >= 0) {
+        double P[3];
+        if (p < nm && B.centroid) {
+            const int *tv = B.tri + 3 * p;
+            for (int a = 0; a < 3; ++a) P[a] = (B.X[3 * tv[0] + a] + B.X[3 * tv[1] + a] + B.X[3 * tv[2] + a]) / 3.0;
+        } else if (p < nm) {
+            P[0] = B.X[3 * p];
+            P[1] = B.X[3 * p + 1];
+            P[2] = B.X[3 * p + 2];
         } else {
-            R(*red)[33] = sm.red[warp];
-            red[0][lane] = Wd[0];
-            red[1][lane] = Wd[1];
-            red[2][lane] = Wd[2];
-            red[3][lane] = Wd[3];
-            red[4][lane] = Wd[1] * dk[0];
-            red[5][lane] = Wd[1] * dk[1];
-            red[6][lane] = Wd[1] * dk[2];
-            red[7][lane] = Wd[2] * dk[1];
-            red[8][lane] = Wd[2] * dk[2];
-            red[9][lane] = Wd[3] * dk[2];
-#pragma unroll
-            for (int q = 0; q < 4; ++q) {
-                red[10 + q][lane] = Wd[q] * gu[j][0];
-                red[14 + q][lane] = Wd[q] * gu[j][1];
-                red[18 + q][lane] = Wd[q] * gu[j][2];
-                red[22 + q][lane] = Wd[q] * gu[j][3];
-            }
-            __syncwarp();
-            if (lane < kSums) {
-                R acc = R(0);
-#pragma unroll
-                for (int k = 0; k < 27; ++k) acc += red[lane][k];
-                sm.sums[lp][lane] = acc;
-            }
-            __syncwarp();
-        }
-    }
-    __syncthreads();
-
-    // ---------------- phase 2: one lane per point ----------------
-    if (warp == w2 && lane < kPts && sm.pid[lane] >= 0) {
-        const int p = sm.pid[lane];
-        const R *S = sm.sums[lane];
-        R Ai[16];
-        if constexpr (sizeof(R) == 8) {
-            double a[10], inv[16];
-            for (int q = 0; q < 10; ++q) a[q] = (double)S[q];
-            if (!spd_inverse4(a, inv)) atomicCAS(err, 0, -1);
-            for (int q = 0; q < 16; ++q) Ai[q] = R(inv[q]);
-        } else {
-            float a[10];
-            for (int q = 0; q < 10; ++q) a[q] = (float)S[q];
-            if (!spd_inverse4_chol(a, (float *)Ai)) atomicCAS(err, 0, -1);
-        }
-        const R *fc = sm.ref[lane];
-        if (p < nm) {
-            for (int q = 0; q < 4; ++q) sm.row0[lane][q] = Ai[q];
-            double *Uo = B.centroid ? B.Uc : B.U;
-            for (int jj = 0; jj < 3; ++jj) {
-                const R *bu = S + 14 + 4 * jj;
-                Uo[3 * p + jj] = (double)(Ai[0] * bu[0] + Ai[1] * bu[1] + Ai[2] * bu[2] + Ai[3] * bu[3] + fc[1 + jj]);
-            }
-        } else {
-            // fits: c_f[i] = sum_m Ai[i][m] b_f[m], plus the centre value for
-            // the value (i = 0)
-            R cr[4], cu[3][4];
-            for (int i = 0; i < 4; ++i) {
-                cr[i] = Ai[4 * i] * S[10] + Ai[4 * i + 1] * S[11] + Ai[4 * i + 2] * S[12] + Ai[4 * i + 3] * S[13];
-                for (int jj = 0; jj < 3; ++jj) {
-                    const R *bu = S + 14 + 4 * jj;
-                    cu[jj][i] = Ai[4 * i] * bu[0] + Ai[4 * i + 1] * bu[1] + Ai[4 * i + 2] * bu[2] + Ai[4 * i + 3] * bu[3];
-                }
-            }
-            cr[0] += fc[0];
-            for (int jj = 0; jj < 3; ++jj) cu[jj][0] += fc[1 + jj];
+            // probe X_c +- 1.2 n, with X_c = x_0 + (e1 + e2)/3 and the
+            // triangle's edges and normal from origin-relative positions
             const int t = (p - nm) >> 1, side = (p - nm) & 1;
-            const R rho = R(1) + cr[0];
-            const R nu = pick<R>(L.nu_d, L.nu_f);
-            R *pr = (R *)B.probe + 8 * t + 4 * side;
-            pr[0] = cr[0] / R(3);  // p - c_s^2 rho0
-            for (int jj = 0; jj < 3; ++jj) {
-                R acc = R(0);
-                for (int m = 0; m < 3; ++m) acc += rho * nu * (cu[jj][1 + m] + cu[m][1 + jj]) * sm.nrm[lane][m];
-                pr[1 + jj] = acc;
+            const int tv[3] = {B.tri[3 * t], B.tri[3 * t + 1], B.tri[3 * t + 2]};
+            const R *Xr = (const R *)B.Xrel;
+            R r0[3], e1[3], e2[3];
+            for (int a = 0; a < 3; ++a) {
+                P[a] = B.X[3 * tv[0] + a];
+                r0[a] = Xr[3 * tv[0] + a];
+                e1[a] = Xr[3 * tv[1] + a] - r0[a];
+                e2[a] = Xr[3 * tv[2] + a] - r0[a];
+            }
+            const R N[3] = {e1[1] * e2[2] - e1[2] * e2[1], e1[2] * e2[0] - e1[0] * e2[2],
+                            e1[0] * e2[1] - e1[1] * e2[0]};
+            const R nn = sqrt(N[0] * N[0] + N[1] * N[1] + N[2] * N[2]);
+            const R inn = R(1) / nn, sg = side ? R(-kProbe) : R(kProbe);
+            R *tg = (R *)B.tri_geo + 8 * t;
+            for (int a = 0; a < 3; ++a) {
+                nrm[a] = N[a] * inn;
+                const R c3 = (e1[a] + e2[a]) / R(3);
+                P[a] += (double)(c3 + sg * nrm[a]);
+                if (side == 0) {
+                    tg[a] = nrm[a];
+                    tg[4 + a] = r0[a] + c3;
+                }
+            }
+            if (side == 0) {
+                tg[3] = R(0.5) * nn;
+                vol = (double)r0[0] * (double)N[0] + (double)r0[1] * (double)N[1] + (double)r0[2] * (double)N[2];
+                B.tri_vol[t] = vol;
             }
         }
+        bool bad = false, diverged = false;
+        for (int a = 0; a < 3; ++a) {
+            if (!(fabs(P[a]) < kMaxMarkerCoord)) {  // non-finite or runaway: flag, keep indices sane
+                diverged = true;
+                P[a] = 0.0;
+            }
+            int b = __double2int_rd(P[a] + 0.5);  // floor(X + 1/2)
+            if (L.bc[a] == kWall && (b - 1 < 1 || b + 1 > n[a] - 2)) {
+                bad = true;
+                b = b < 2 ? 2 : (b > n[a] - 3 ? n[a] - 3 : b);
+            }
+            base[a] = b;
+            frac[a] = P[a] - (double)b;
+        }
+        if (diverged)
+            atomicCAS(err, 0, kErrDiverged);
+        else if (bad)
+            atomicCAS(err, 0, kErrBodyWall);
     }
-    // enclosed volume (membranes): fixed-order partial per block; the last
+    // enclosed volume (membranes): a fixed-order partial per warp; the last
     // block to finish sums the partials with a fixed-shape tree
     // (deterministic whichever block is last)
-    __shared__ int s_last;
     if (!B.rigid) {
-        if (threadIdx.x == 32 * ((w2 + 1) & 3)) {
-            double s = 0.0;
-            for (int k = 0; k < kPts; ++k) s += sm.vol[k];
-            B.vol_part[vb] = s;
+        __shared__ int s_last;
+        const int npart = (npts + 31) / 32, part = slot >> 5;
+        vol = warp_sum(vol);
+        if (lane == 0 && part < npart) B.vol_part[part] = vol;
+        __syncthreads();
+        if (threadIdx.x == 0) {
             __threadfence();
             s_last = atomicAdd(B.vol_count, 1u) == (unsigned)nvb - 1;
         }
@@ -600,51 +406,186 @@ __device__ __forceinline__ void mls_body(const R *__restrict__ mom, const Lattic
         if (s_last) {
             __threadfence();
             double s = 0.0;
-            for (int k = threadIdx.x; k < nvb; k += blockDim.x) s += __ldcg(B.vol_part + k);
+            for (int k = threadIdx.x; k < npart; k += blockDim.x) s += __ldcg(B.vol_part + k);
             s = warp_sum(s);
-            __shared__ double wpart[kMlsThreads / 32];
+            __shared__ double wpart[8];
             if (lane == 0) wpart[warp] = s;
             __syncthreads();
             if (threadIdx.x == 0) {
                 double tot = 0.0;
-                for (int w = 0; w < kMlsThreads / 32; ++w) tot += wpart[w];
+                for (int w = 0; w < (int)blockDim.x / 32; ++w) tot += wpart[w];
                 *B.vol_sum = tot;
                 *B.vol_count = 0u;
             }
         }
     }
-    __syncthreads();
 
-    // ---------------- phase 3: transfer weights of the markers ----------------
-    for (int j = 0; j < kPerWarp; ++j) {
-        const int lp = warp * kPerWarp + j;
-        const int p = sm.pid[lp];
-        if (p < 0) break;
-        if (p >= nm) continue;  // probes keep no transfer weights
-        if (lane < 27) {
-            R dk[3];
-            if constexpr (kShfl) {
-                const int dd[3] = {lane % 3 - 1, (lane / 3) % 3 - 1, lane / 9 - 1};
-                for (int a = 0; a < 3; ++a) dk[a] = R(dd[a]) - sm.fracR[lp][a];  // as in phase 1
-            } else {
-                for (int a = 0; a < 3; ++a) dk[a] = sm.d[lp][lane][a];
+    // weights and the support's nodes (r_k <= 1, Eq. intKernel): FP32 squared
+    // distances, and the FP64 ones of nodes whose decision FP32 rounding
+    // (below 1e-6 here) could flip
+    R d[3][3], w[3][3];
+    unsigned in = 0u, near = 0u;
+    {
+        float sq[3][3];
+        for (int a = 0; a < 3; ++a) {
+            axis_weights(R(frac[a]), d[a], w[a]);
+            const float f = float(frac[a]);
+#pragma unroll
+            for (int i = 0; i < 3; ++i) sq[a][i] = (float(i - 1) - f) * (float(i - 1) - f);
+        }
+#pragma unroll
+        for (int q = 0; q < 27; ++q) {
+            const float t = sq[0][q % 3] + (sq[1][(q / 3) % 3] + sq[2][q / 9]) - L.dist2_cut_f;
+            if (t <= 0.f) in |= 1u << q;
+            if (fabsf(t) <= 1e-5f) near |= 1u << q;
+        }
+        if (near) in = (in & ~near) | support_exact(near, frac[0], frac[1], frac[2], L.dist2_cut);
+    }
+    if constexpr (kChain) chain_wait();
+    if (p < 0) return;
+
+    // ---------------- sums ----------------
+    int ox[3], oy[3], oz[3];
+#pragma unroll
+    for (int i = 0; i < 3; ++i) {
+        ox[i] = support_coord(L, 0, base[0] + i - 1);
+        oy[i] = L.nx * support_coord(L, 1, base[1] + i - 1);
+        oz[i] = L.nx * L.ny * support_coord(L, 2, base[2] + i - 1);
+    }
+    // fit f - f_c, f_c the moments of the centre node (always in the
+    // support): the same fit, since MLS reproduces constants, but the sums
+    // and the solve then carry the field's variation over the support rather
+    // than its size, which the gradients at the probes (small differences of
+    // the fitted values) need
+    R fc[4];
+    mom_load<kCG>(mom, ox[1] + oy[1] + oz[1], fc);
+    // A: 00, 01, 02, 03, 11, 12, 13, 22, 23, 33; b[c]: 1, x, y, z
+    R A[10], b[4][4];
+#pragma unroll
+    for (int q = 0; q < 10; ++q) A[q] = R(0);
+#pragma unroll
+    for (int c = 0; c < 4; ++c)
+#pragma unroll
+        for (int q = 0; q < 4; ++q) b[c][q] = R(0);
+#pragma unroll
+    for (int k = 0; k < 3; ++k) {
+        R T[6], Tf[4][3];  // sums over the plane: 1, x, y, xx, xy, yy; fields: 1, x, y
+#pragma unroll
+        for (int q = 0; q < 6; ++q) T[q] = R(0);
+#pragma unroll
+        for (int c = 0; c < 4; ++c)
+#pragma unroll
+            for (int q = 0; q < 3; ++q) Tf[c][q] = R(0);
+#pragma unroll
+        for (int j = 0; j < 3; ++j) {
+            R S0 = R(0), S1 = R(0), S2 = R(0), F0[4], F1[4];
+#pragma unroll
+            for (int c = 0; c < 4; ++c) F0[c] = F1[c] = R(0);
+#pragma unroll
+            for (int i = 0; i < 3; ++i) {
+                R v[4];
+                mom_load<kCG>(mom, ox[i] + oy[j] + oz[k], v);
+                const R a0 = (in >> (i + 3 * j + 9 * k)) & 1u ? w[0][i] : R(0), a1 = a0 * d[0][i];
+                S0 += a0;
+                S1 += a1;
+                S2 += a1 * d[0][i];
+#pragma unroll
+                for (int c = 0; c < 4; ++c) {
+                    const R f = v[c] - fc[c];
+                    F0[c] += a0 * f;
+                    F1[c] += a1 * f;
+                }
             }
-            const R *r0 = sm.row0[lp];
-            const R phi = sm.W[lp][lane] * (r0[0] + r0[1] * dk[0] + r0[2] * dk[1] + r0[3] * dk[2]);
-            ((R *)B.phi)[27 * p + lane] = phi;
+            const R w1 = w[1][j], w1d = w1 * d[1][j];
+            T[0] += w1 * S0;
+            T[1] += w1 * S1;
+            T[2] += w1d * S0;
+            T[3] += w1 * S2;
+            T[4] += w1d * S1;
+            T[5] += (w1d * d[1][j]) * S0;
+#pragma unroll
+            for (int c = 0; c < 4; ++c) {
+                Tf[c][0] += w1 * F0[c];
+                Tf[c][1] += w1 * F1[c];
+                Tf[c][2] += w1d * F0[c];
+            }
+        }
+        const R w2 = w[2][k], w2d = w2 * d[2][k];
+        A[0] += w2 * T[0];
+        A[1] += w2 * T[1];
+        A[2] += w2 * T[2];
+        A[3] += w2d * T[0];
+        A[4] += w2 * T[3];
+        A[5] += w2 * T[4];
+        A[6] += w2d * T[1];
+        A[7] += w2 * T[5];
+        A[8] += w2d * T[2];
+        A[9] += (w2d * d[2][k]) * T[0];
+#pragma unroll
+        for (int c = 0; c < 4; ++c) {
+            b[c][0] += w2 * Tf[c][0];
+            b[c][1] += w2 * Tf[c][1];
+            b[c][2] += w2 * Tf[c][2];
+            b[c][3] += w2d * Tf[c][0];
+        }
+    }
+
+    // ---------------- solve ----------------
+    R Ai[16];
+    if (!spd_inverse4(A, Ai)) atomicCAS(err, 0, -1);
+    if (p < nm) {
+        double *Uo = B.centroid ? B.Uc : B.U;
+#pragma unroll
+        for (int c = 0; c < 3; ++c) {
+            const R *bu = b[1 + c];
+            Uo[3 * p + c] = (double)(fc[1 + c] + (Ai[3] * bu[3] + Ai[2] * bu[2] + Ai[1] * bu[1] + Ai[0] * bu[0]));
+        }
+        R rec[kRec];
+#pragma unroll
+        for (int q = 0; q < 4; ++q) rec[q] = Ai[q];
+#pragma unroll
+        for (int a = 0; a < 3; ++a) {
+            rec[4 + a] = R(frac[a]);
+#pragma unroll
+            for (int i = 0; i < 3; ++i) rec[7 + 3 * a + i] = w[a][i];
+        }
+        store_record((R *)B.phi + (size_t)kRec * p, rec);
+        reinterpret_cast<int4 *>(B.node)[p] = make_int4(base[0], base[1], base[2], (int)in);
+    } else {
+        // fits: c_f[i] = sum_m Ai[i][m] b_f[m], plus the centre value for
+        // the value (i = 0)
+        const R cr = Ai[0] * b[0][0] + Ai[1] * b[0][1] + Ai[2] * b[0][2] + Ai[3] * b[0][3] + fc[0];
+        R gr[3][3];
+#pragma unroll
+        for (int c = 0; c < 3; ++c)
+#pragma unroll
+            for (int a = 0; a < 3; ++a) {
+                const R *bu = b[1 + c], *row = Ai + 4 * (a + 1);
+                gr[c][a] = row[0] * bu[0] + row[1] * bu[1] + row[2] * bu[2] + row[3] * bu[3];
+            }
+        const int t = (p - nm) >> 1, side = (p - nm) & 1;
+        const R rn = (R(1) + cr) * pick<R>(L.nu_d, L.nu_f);
+        R *pr = (R *)B.probe + 8 * t + 4 * side;
+        pr[0] = cr / R(3);  // p - c_s^2 rho0
+#pragma unroll
+        for (int c = 0; c < 3; ++c) {
+            R acc = R(0);
+#pragma unroll
+            for (int a = 0; a < 3; ++a) acc += (gr[c][a] + gr[a][c]) * nrm[a];
+            pr[1 + c] = rn * acc;
         }
     }
 }
 
-// The blocks take the nvb groups of 32 points in turn (gridDim.x = nvb
-// unless the launch caps the grid).
+// The blocks take the nvb groups of points in turn (gridDim.x = nvb unless
+// the launch caps the grid).
 template <typename R>
 __global__ void __launch_bounds__(kMlsThreads) k_mls(const R *__restrict__ mom, Lattice L, BodyView B,
                                                      int *err, int nvb) {
-    chain_wait();  // launched programmatically after the moments kernel
-    extern __shared__ __align__(16) unsigned char smem_raw[];
     for (int vb = blockIdx.x; vb < nvb; vb += gridDim.x) {
-        mls_body<R>(mom, L, B, err, *reinterpret_cast<MlsSmem<R> *>(smem_raw), vb, nvb);
+        // launched programmatically after the moments kernel, whose results
+        // it waits for inside
+        mls_body<R, false, true>(mom, L, B, err, vb, nvb);
         __syncthreads();  // the next group reuses the shared memory
     }
 }
@@ -659,38 +600,47 @@ __device__ __forceinline__ void tri_hydro(const BodyView &B, int t, R *F) {
     for (int a = 0; a < 3; ++a) F[a] = (-(pp[0] - pm[0]) * tg[a] + (pp[1 + a] - pm[1 + a])) * A;
 }
 
-// Lanes 0..26 of a warp add c phi_k F to the force field at the support
-// nodes of marker v; the lanes of the 8 block corners flag their tiles.
+// What lane k < 27 of a marker's warp needs to spread to support node k: the
+// node (-1: r_k > 1, nothing to add), its transfer weight phi_k, and the
+// tile to flag (the lanes of the 8 block corners; -1 on the others).
 template <typename R>
-__device__ __forceinline__ void spread_warp(const Lattice &L, const BodyView &B, int v, int lane, R c, const R *Fl,
-                                            R *__restrict__ force, uint32_t *stamp, uint32_t step) {
-    if (lane >= 27) return;
-    const long long st = L.stride;
-    const int node = B.node[27 * v + lane];
-    const R w = c * ((const R *)B.phi)[27 * v + lane];
-    atomicAdd(force + node, w * Fl[0]);
-    atomicAdd(force + st + node, w * Fl[1]);
-    atomicAdd(force + 2 * st + node, w * Fl[2]);
-    if (lane == 0 || lane == 2 || lane == 6 || lane == 8 || lane == 18 || lane == 20 || lane == 24 || lane == 26) {
-        const int x = node % L.nx, yz = node / L.nx, y = yz % L.ny, z = yz / L.ny;
-        stamp[(x >> 3) + L.ntx * ((y >> 3) + L.nty * (z >> 3))] = step;
+struct SpreadLane {
+    int node, tile;
+    R phi;
+};
+template <typename R>
+__device__ __forceinline__ SpreadLane<R> spread_load(const Lattice &L, const BodyView &B, int p, int lane) {
+    SpreadLane<R> s;
+    s.node = s.tile = -1;
+    s.phi = R(0);
+    if (lane >= 27) return s;
+    const int i = lane % 3, j = (lane / 3) % 3, k = lane / 9;
+    const R *rec = (const R *)B.phi + (size_t)kRec * p;
+    const int4 bs = reinterpret_cast<const int4 *>(B.node)[p];
+    const int x = support_coord(L, 0, bs.x + i - 1), y = support_coord(L, 1, bs.y + j - 1),
+              z = support_coord(L, 2, bs.z + k - 1);
+    if ((unsigned)bs.w >> lane & 1u) {
+        s.node = x + L.nx * (y + L.ny * z);
+        const R dx = R(i - 1) - rec[4], dy = R(j - 1) - rec[5], dz = R(k - 1) - rec[6];
+        s.phi = (rec[7 + i] * rec[10 + j] * rec[13 + k]) * (rec[0] + rec[1] * dx + rec[2] * dy + rec[3] * dz);
     }
+    if (i != 1 && j != 1 && k != 1) s.tile = (x >> 3) + L.ntx * ((y >> 3) + L.nty * (z >> 3));
+    return s;
 }
 
-// Lane k < 27 of a marker's warp adds w F to the force field at its
-// support node; the lanes of the 8 block corners flag their tiles.
+// Adds c phi_k F to the force field at the lane's support node and flags the
+// lane's tile.
 template <typename R>
-__device__ __forceinline__ void spread_node(const Lattice &L, int lane, int node, R w, const R *Fl,
+__device__ __forceinline__ void spread_lane(const Lattice &L, const SpreadLane<R> &s, R c, const R *Fl,
                                             R *__restrict__ force, uint32_t *stamp, uint32_t step) {
-    if (lane >= 27) return;
-    const long long st = L.stride;
-    atomicAdd(force + node, w * Fl[0]);
-    atomicAdd(force + st + node, w * Fl[1]);
-    atomicAdd(force + 2 * st + node, w * Fl[2]);
-    if (lane == 0 || lane == 2 || lane == 6 || lane == 8 || lane == 18 || lane == 20 || lane == 24 || lane == 26) {
-        const int x = node % L.nx, yz = node / L.nx, y = yz % L.ny, z = yz / L.ny;
-        stamp[(x >> 3) + L.ntx * ((y >> 3) + L.nty * (z >> 3))] = step;
+    if (s.node >= 0) {
+        const long long st = L.stride;
+        const R w = c * s.phi;
+        atomicAdd(force + s.node, w * Fl[0]);
+        atomicAdd(force + st + s.node, w * Fl[1]);
+        atomicAdd(force + 2 * st + s.node, w * Fl[2]);
     }
+    if (s.tile >= 0) stamp[s.tile] = step;
 }
 
 // Node box of level n+1: each block reduces its markers' cells in shared
@@ -736,12 +686,8 @@ __device__ __forceinline__ void membrane_body(const Lattice &L, const BodyView &
     const int v0 = vb * (blockDim.x >> 5);  // first vertex of the block
     const int v = v0 + warp;
     // the spreading lanes fetch their node and weight first
-    int snode = 0;
-    R sphi = R(0);
-    if (!B.centroid && v < B.nv && lane < 27) {
-        snode = B.node[27 * v + lane];
-        sphi = ((const R *)B.phi)[27 * v + lane];
-    }
+    SpreadLane<R> sl{};
+    if (!B.centroid && v < B.nv) sl = spread_load<R>(L, B, v, lane);
     if (threadIdx.x == 0) s_cv = R(B.kv * (1.0 - *B.vol_sum * B.inv_6V0));
     sbox.init();
     __syncthreads();
@@ -886,7 +832,7 @@ __device__ __forceinline__ void membrane_body(const Lattice &L, const BodyView &
     }
     __syncthreads();
     if (!B.centroid && v < B.nv)
-        spread_node<R>(L, lane, snode, s_F[warp][3] * sphi, s_Fl[warp], force, stamp, step);
+        spread_lane<R>(L, sl, s_F[warp][3], s_Fl[warp], force, stamp, step);
     __syncthreads();
     sbox.flush(B.bbox_next);
 }
@@ -1155,6 +1101,8 @@ __device__ __forceinline__ void rigid_markers_body(const Lattice &L, const BodyV
     const int v0 = vb * (blockDim.x >> 5);
     const int v = v0 + warp;
     sbox.init();
+    SpreadLane<R> sl{};
+    if (!B.centroid && v < B.nv) sl = spread_load<R>(L, B, v, lane);
     if (v < B.nv) {
         R Al = R(0);
         double Uv[3] = {0.0, 0.0, 0.0};
@@ -1206,7 +1154,7 @@ __device__ __forceinline__ void rigid_markers_body(const Lattice &L, const BodyV
         s_Fl[j][a] = R(Fla);
     }
     __syncthreads();
-    if (!B.centroid && v < B.nv) spread_warp<R>(L, B, v, lane, s_Al[warp], s_Fl[warp], force, stamp, step);
+    if (!B.centroid && v < B.nv) spread_lane<R>(L, sl, s_Al[warp], s_Fl[warp], force, stamp, step);
     __syncthreads();
     sbox.flush(B.bbox_next);
 }
@@ -1235,12 +1183,8 @@ __device__ __forceinline__ void centroid_body(const Lattice &L, const BodyView &
     __shared__ R s_Fl[8][3];
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     const int t0 = vb * 8, t = t0 + warp;
-    int snode = 0;
-    R sphi = R(0);
-    if (t < B.nt && lane < 27) {
-        snode = B.node[27 * t + lane];
-        sphi = ((const R *)B.phi)[27 * t + lane];
-    }
+    SpreadLane<R> sl{};
+    if (t < B.nt) sl = spread_load<R>(L, B, t, lane);
     if (t < B.nt && lane == 0) s_A[warp] = ((const R *)B.tri_geo)[8 * t + 3];
     // FP64 for the block's 8 markers at once: lane 3 j + a of one warp
     // handles component a of marker j
@@ -1265,7 +1209,7 @@ __device__ __forceinline__ void centroid_body(const Lattice &L, const BodyView &
         s_Fl[j][a] = R(Fla);
     }
     __syncthreads();
-    if (t < B.nt) spread_node<R>(L, lane, snode, s_A[warp] * sphi, s_Fl[warp], force, stamp, step);
+    if (t < B.nt) spread_lane<R>(L, sl, s_A[warp], s_Fl[warp], force, stamp, step);
 }
 
 template <typename R>
@@ -1289,8 +1233,7 @@ __global__ void __launch_bounds__(256) kb_moments(BatchTables T, int phase) {
 }
 
 template <typename R>
-__global__ void __launch_bounds__(kMlsThreads) kb_mls(BatchTables T, int phase) {
-    extern __shared__ __align__(16) unsigned char smem_raw[];
+__global__ void __launch_bounds__(kBatchMlsThreads) kb_mls(BatchTables T, int phase) {
     __shared__ Lattice L;
     __shared__ BodyRef br;
     const int j = __ldg(T.mls_blk + blockIdx.x);
@@ -1298,7 +1241,7 @@ __global__ void __launch_bounds__(kMlsThreads) kb_mls(BatchTables T, int phase) 
     stage_shared(br, T.body + phase * T.nb + j);
     stage_shared(L, T.lat + br.lat);
     const LatRef &F = T.ref[phase * T.nl + br.lat];
-    mls_body<R>((const R *)F.mom, L, br.v, F.err, *reinterpret_cast<MlsSmem<R> *>(smem_raw), vb, nvb);
+    mls_body<R>((const R *)F.mom, L, br.v, F.err, vb, nvb);
 }
 
 template <typename R>
@@ -1405,7 +1348,6 @@ __device__ bool wait_deps(const PersistTables &P, int k, int l, int s) {
 // the launch.
 template <typename S, typename R, bool kOff32>
 __global__ void __launch_bounds__(256, 4) kp_batch(BatchTables T, PersistTables P) {
-    extern __shared__ __align__(16) unsigned char smem_raw[];
     __shared__ Lattice L;
     __shared__ BodyRef br;
     __shared__ unsigned s_t[2];  // this item's ticket and the next one (taken early, double-buffered)
@@ -1460,8 +1402,7 @@ __global__ void __launch_bounds__(256, 4) kp_batch(BatchTables T, PersistTables 
                                          br.inc_step ? F.d_step : nullptr, it.z, it.w);
                 break;
             case kPMls:
-                mls_body<R, true, true>((const R *)F.mom, L, br.v, F.err,
-                                        *reinterpret_cast<MlsSmem<R, true> *>(smem_raw), it.z, it.w);
+                mls_body<R, true>((const R *)F.mom, L, br.v, F.err, it.z, it.w);
                 break;
             case kPMemb: membrane_body<R>(L, br.v, (R *)F.force, F.stamp, F.d_step, it.z); break;
             case kPRf: rigid_forces_body<R>(br.v, it.z, it.w); break;
@@ -1479,9 +1420,9 @@ __global__ void __launch_bounds__(256, 4) kp_batch(BatchTables T, PersistTables 
 template <typename S, typename R>
 static cudaError_t persistent_t(const BatchTables &T, const PersistTables &P, int grid, cudaStream_t s) {
     if (T.sweep_off32)
-        kp_batch<S, R, true><<<grid, 256, sizeof(MlsSmem<R, true>), s>>>(T, P);
+        kp_batch<S, R, true><<<grid, 256, 0, s>>>(T, P);
     else
-        kp_batch<S, R, false><<<grid, 256, sizeof(MlsSmem<R, true>), s>>>(T, P);
+        kp_batch<S, R, false><<<grid, 256, 0, s>>>(T, P);
     return cudaGetLastError();
 }
 
@@ -1495,19 +1436,14 @@ cudaError_t launch_batch_persistent(int prec, const BatchTables &T, const Persis
     }
 }
 
-// Resident blocks per SM of the persistent kernel (its dynamic shared
-// memory set), for the grid size.
+// Resident blocks per SM of the persistent kernel, for the grid size.
 template <typename S, typename R>
 static int persistent_occ(bool off32) {
     int n = 0;
-    const size_t smem = sizeof(MlsSmem<R, true>);
-    if (off32) {
-        cudaFuncSetAttribute(kp_batch<S, R, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-        cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, kp_batch<S, R, true>, 256, smem);
-    } else {
-        cudaFuncSetAttribute(kp_batch<S, R, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-        cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, kp_batch<S, R, false>, 256, smem);
-    }
+    if (off32)
+        cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, kp_batch<S, R, true>, 256, 0);
+    else
+        cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, kp_batch<S, R, false>, 256, 0);
     return n;
 }
 
@@ -1523,7 +1459,7 @@ int batch_persistent_blocks_per_sm(int prec, bool off32) {
 template <typename S, typename R>
 static cudaError_t batch_ib_t(const BatchTables &T, const BatchGrid &G, int phase, cudaStream_t s) {
     if (G.mom > 0) kb_moments<S, R><<<G.mom, 256, 0, s>>>(T, phase);
-    if (G.mls > 0) kb_mls<R><<<G.mls, kMlsThreads, sizeof(MlsSmem<R>), s>>>(T, phase);
+    if (G.mls > 0) kb_mls<R><<<G.mls, kBatchMlsThreads, 0, s>>>(T, phase);
     if (G.memb > 0) kb_membrane<R><<<G.memb, 256, 0, s>>>(T, phase);
     if (G.rf > 0) kb_rigid_forces<R><<<G.rf, 256, 0, s>>>(T, phase);
     if (G.rm > 0) kb_rigid_markers<R><<<G.rm, 256, 0, s>>>(T, phase);
@@ -1541,7 +1477,7 @@ cudaError_t launch_batch_ib(int prec, const BatchTables &T, const BatchGrid &G, 
 }
 
 // ---- launchers ----
-int mls_blocks(const BodyView &B) { return (B.nm + 2 * B.nt + kPts - 1) / kPts; }
+int mls_blocks(const BodyView &B, int threads) { return (B.nm + 2 * B.nt + threads - 1) / threads; }
 
 // Grid of n blocks' work under a cap (0: none).
 static int capped(int n, int cap) { return cap > 0 && cap < n ? cap : n; }
@@ -1555,26 +1491,9 @@ static cudaError_t ib_front_t(const void *fin, const Lattice &L, const BodyView 
     // the MLS kernel is scheduled while the moments kernel ends (measured:
     // about 2 us off the 96^3 capsule step; the same launch for the other
     // kernels of the step made it slower)
-    const int nvb = mls_blocks(B);
-    return launch_chained(k_mls<R>, dim3(capped(nvb, grid_cap)), dim3(kMlsThreads), sizeof(MlsSmem<R>), s,
+    const int nvb = mls_blocks(B, kMlsThreads);
+    return launch_chained(k_mls<R>, dim3(capped(nvb, grid_cap)), dim3(kMlsThreads), 0, s,
                           (const R *)mom, L, B, err, nvb);
-}
-
-// Kernel attributes that must be set before the first launch (and before
-// any stream capture): the MLS kernel's dynamic shared memory.
-cudaError_t prepare_kernels() {
-    cudaError_t e = cudaFuncSetAttribute(k_mls<float>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                         (int)sizeof(MlsSmem<float>));
-    if (e == cudaSuccess)
-        e = cudaFuncSetAttribute(k_mls<double>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                 (int)sizeof(MlsSmem<double>));
-    if (e == cudaSuccess)
-        e = cudaFuncSetAttribute(kb_mls<float>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                 (int)sizeof(MlsSmem<float>));
-    if (e == cudaSuccess)
-        e = cudaFuncSetAttribute(kb_mls<double>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                 (int)sizeof(MlsSmem<double>));
-    return e;
 }
 
 cudaError_t launch_ib_front(int prec, const void *fin, const Lattice &L, const BodyView &B, void *mom, int nsm,

@@ -565,7 +565,6 @@ int lbib_create(const lbib_params *p, void **out) {
     if (e == cudaSuccess) e = cudaMemsetAsync(c->d_sr, 0, 2 * sizeof(uint32_t), c->stream);
     if (e == cudaSuccess) e = cudaMemsetAsync(c->d_tot, 0, sizeof(double) * (size_t)totals_scratch_doubles(), c->stream);
     if (e == cudaSuccess) e = cudaMemsetAsync(c->d_watch, 0, 2 * sizeof(double), c->stream);
-    if (e == cudaSuccess) e = prepare_kernels();
     if (e == cudaSuccess) e = prepare_sweep_kernels();
     if (e == cudaSuccess) e = cudaStreamCreateWithFlags(&c->s_cap, cudaStreamNonBlocking);
     for (int k = 0; k < 6 && e == cudaSuccess; ++k)
@@ -932,9 +931,9 @@ int lbib_add_body(void *h, const double *verts, int nv, const int *tris, int nt,
         tmp.nv = nv;
         tmp.nt = nt;
         tmp.nm = nm;
-        // partial sums: one per MLS block (membrane volume) or six per
+        // partial sums: one per 32 MLS points (membrane volume) or six per
         // force block (rigid force and moment)
-        b.nvol_part = std::max(mls_blocks(tmp), 6 * ((nt + 255) / 256));
+        b.nvol_part = std::max(mls_blocks(tmp, 32), 6 * ((nt + 255) / 256));
         b.vol_part = upload(c, std::vector<double>((size_t)b.nvol_part, 0.0), &rc);
         b.vol_sum = upload(c, std::vector<double>(1, 6.0 * V0), &rc);
         b.vol_count = upload(c, std::vector<unsigned int>(1, 0u), &rc);
@@ -1689,7 +1688,7 @@ int batch_build_persistent(Batch *b, const std::vector<std::pair<int, int>> &bod
         std::array<int, kPKinds> &n = count[q];
         n.fill(0);
         n[kPMom] = std::max(8, d.nv / 16);
-        n[kPMls] = mls_blocks(body[q].v);
+        n[kPMls] = mls_blocks(body[q].v, kPersistThreads);
         n[kPMemb] = d.rigid ? 0 : (d.nv + 7) / 8;
         n[kPRf] = d.rigid ? (d.nt + 255) / 256 : 0;
         n[kPRm] = d.rigid ? (d.nv + 7) / 8 : 0;
@@ -1815,7 +1814,7 @@ int batch_build(Batch *b) {
         d.bcur = bcur0;
         const BodyView &v = body[q].v;
         mom_pre.push_back(mom_pre.back() + std::max(8, d.nv / 16));
-        mls_pre.push_back(mls_pre.back() + mls_blocks(v));
+        mls_pre.push_back(mls_pre.back() + mls_blocks(v, kBatchMlsThreads));
         if (d.rigid) {
             rigid_id.push_back(q);
             rf_pre.push_back(rf_pre.back() + (d.nt + 255) / 256);

@@ -273,8 +273,8 @@ struct BodyView {
     int nm;                 // number of markers: nv or nt
     double *Uc;             // centroid markers [3nt]: interpolated fluid velocity
     double *Flc;            // centroid markers [3nt]: Lagrangian IB force
-    void *phi;              // [27nm] R: MLS transfer weights of level n
-    int *node;              // [27nm] support node indices
+    void *phi;              // [27nm] R: MLS transfer records of level n (16 R per marker)
+    int *node;              // [27nm] base node (x, y, z) and support bits of level n (4 per marker)
     const int *perm;        // [nm + 2nt] MLS points in cell order (markers, probes), or nullptr
     const int *tri;         // [3nt]
     void *tri_geo;          // [8nt] R: unit normal (3), area, centroid - origin (3), unused
@@ -301,7 +301,7 @@ struct BodyView {
     // support region: node box of level n (read) and of level n+1 (built)
     const int *bbox;        // [6]: lo xyz, hi xyz (inclusive node coordinates)
     int *bbox_next;         // [6], reset by the moments kernel, filled by the update kernel
-    double *vol_part;       // [one per MLS block] partial sums of the volume terms
+    double *vol_part;       // [one per 32 MLS points] partial sums of the volume terms
     int nvol_part;
     unsigned int *vol_count; // blocks of the MLS kernel done (reset by the last one)
     double *vol_sum;        // enclosed volume times 6, written by the last MLS block

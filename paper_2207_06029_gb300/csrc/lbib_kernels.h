@@ -55,8 +55,10 @@ cudaError_t launch_fields_out(int prec, const void *fields, const Lattice &L, do
                               cudaStream_t s);
 
 // ib.cu
-int mls_blocks(const BodyView &B);
-cudaError_t prepare_kernels();
+constexpr int kBatchMlsThreads = 128;       // MLS points per block of the batched kernel
+constexpr int kPersistThreads = 256;        // threads per block of the persistent batched kernel
+// blocks of `threads` MLS points (markers and probes) of a body
+int mls_blocks(const BodyView &B, int threads);
 // step_inc: device step counter incremented at the start of the step (first
 // body only), or nullptr.  grid_cap > 0: the MLS, structure and spreading
 // kernels launch at most grid_cap blocks, each taking its share of their
@@ -79,8 +81,7 @@ cudaError_t launch_batch_sweep(int prec, const BatchTables &T, const BatchGrid &
 // launch of `grid` blocks of 256 threads; the counters P.ticket, P.abort and
 // P.done must be zero at launch
 cudaError_t launch_batch_persistent(int prec, const BatchTables &T, const PersistTables &P, int grid, cudaStream_t s);
-// resident blocks per SM of the persistent kernel (sets its shared-memory
-// attribute; call before any capture)
+// resident blocks per SM of the persistent kernel
 int batch_persistent_blocks_per_sm(int prec, bool off32);
 
 }  // namespace lbib

@@ -15,7 +15,7 @@
 
 namespace lbib {
 
-constexpr int kMlsThreads = 64;   // MLS points (threads) per block
+constexpr int kStructThreads = 128;  // threads per block of the structure kernels (16 markers)
 constexpr double kAlpha = 0.3;    // Eq. (intKernel)
 constexpr double kRw = 1.3;       // support size r_w (Sec. 2.2)
 constexpr double kProbe = 1.2;    // probe length (Sec. 2.3)
@@ -297,13 +297,44 @@ __device__ __forceinline__ void store_record(double *rec, const double *v) {
     for (int q = 0; q < kRec / 2; ++q) reinterpret_cast<double2 *>(rec)[q] = make_double2(v[2 * q], v[2 * q + 1]);
 }
 
+// Sums a body takes over its MLS points: the enclosed volume times 6, or a
+// rigid body's force and moment.
+__device__ __forceinline__ int body_sums(const BodyView &B) { return B.rigid ? 6 : 1; }
+
+// Momentum exchange: triangle t's share of minus the IB force of the
+// previous step (sum_l A_l F_l) and of its moment about x_c (arm: X_c - x_c).
+template <typename R>
+__device__ __forceinline__ void exchange_force(const BodyView &B, int t, R area, const R *arm, R *f) {
+    if (B.centroid) {
+        for (int c = 0; c < 3; ++c) f[c] = -area * R(B.Flc[3 * t + c]);
+        f[3] = arm[1] * f[2] - arm[2] * f[1];
+        f[4] = arm[2] * f[0] - arm[0] * f[2];
+        f[5] = arm[0] * f[1] - arm[1] * f[0];
+        return;
+    }
+    // each corner carries a third of the triangle's area
+    const R c = -area / R(3);
+    const R *Xr = (const R *)B.Xrel;
+    R xc[3];
+    for (int a = 0; a < 3; ++a) xc[a] = R(__ldcg(B.rstate + RigidState::XC + a) - B.origin[a]);
+    for (int q = 0; q < 3; ++q) {
+        const int v = B.tri[3 * t + q];
+        const R Fv[3] = {c * R(B.Fl[3 * v]), c * R(B.Fl[3 * v + 1]), c * R(B.Fl[3 * v + 2])};
+        const R r[3] = {Xr[3 * v] - xc[0], Xr[3 * v + 1] - xc[1], Xr[3 * v + 2] - xc[2]};
+        for (int a = 0; a < 3; ++a) f[a] += Fv[a];
+        f[3] += r[1] * Fv[2] - r[2] * Fv[1];
+        f[4] += r[2] * Fv[0] - r[0] * Fv[2];
+        f[5] += r[0] * Fv[1] - r[1] * Fv[0];
+    }
+}
+
 // MLS at markers and probes, one thread per point.  Points 0..nm-1 are the
 // markers (the vertices, or the triangle centroids); point nm + 2t + side is
 // the probe of triangle t on the outer (side 0) or inner (side 1) face.  With p_k = (1, x_k - X) the fit of a
 // field f is a = A^-1 b_f, A = sum_k W_k p_k p_k^T, b_f = sum_k W_k p_k f_k
 // (Eq. l2norm), i.e. f(X) = a_0 and grad f = (a_1, a_2, a_3).
 //  positions: the point (probes: triangle geometry), the nearest node base =
-//           floor(X + 1/2) and the exact offset X - base; enclosed volume.
+//           floor(X + 1/2) and the exact offset X - base.
 //           Nothing here reads the moments: with kChain it runs while the
 //           moments kernel ends;
 //  sums:    W is a product over the axes but for its cut-off r_k <= 1 (a bit
@@ -314,10 +345,11 @@ __device__ __forceinline__ void store_record(double *rec, const double *v) {
 //  solve:   inverse of A (FP64 adjugate in the FP64 path, FP32 L D L^T in
 //           the FP32 one); markers get U = (A^-1 b_u)_0 + u_c (Eq. uLag),
 //           probes the pressure c_s^2 rho and the traction
-//           rho nu (grad u + grad u^T) . n from the fits.
+//           rho nu (grad u + grad u^T) . n from the fits (membranes keep
+//           them per triangle, rigid bodies sum the forces and moments).
 template <typename R, bool kCG = false, bool kChain = false>
 __device__ __forceinline__ void mls_body(const R *__restrict__ mom, const Lattice &L, const BodyView &B, int *err,
-                                         const int vb, const int nvb) {
+                                         const int vb) {
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     const int nm = B.nm, npts = nm + 2 * B.nt;
     const int slot = vb * blockDim.x + threadIdx.x;
@@ -326,7 +358,7 @@ __device__ __forceinline__ void mls_body(const R *__restrict__ mom, const Lattic
 
     // ---------------- positions ----------------
     double vol = 0.0, frac[3] = {0.0, 0.0, 0.0};
-    R nrm[3] = {R(0), R(0), R(0)};
+    R nrm[3] = {R(0), R(0), R(0)}, arm[3] = {R(0), R(0), R(0)}, area = R(0);  // probes: normal, X_c - x_c, area
     int base[3] = {2, 2, 2};
     if (p >= 0) {
         double P[3];
@@ -355,20 +387,24 @@ __device__ __forceinline__ void mls_body(const R *__restrict__ mom, const Lattic
             const R nn = sqrt(N[0] * N[0] + N[1] * N[1] + N[2] * N[2]);
             const R inn = R(1) / nn, sg = side ? R(-kProbe) : R(kProbe);
             R *tg = (R *)B.tri_geo + 8 * t;
+            area = R(0.5) * nn;
             for (int a = 0; a < 3; ++a) {
                 nrm[a] = N[a] * inn;
                 const R c3 = (e1[a] + e2[a]) / R(3);
                 P[a] += (double)(c3 + sg * nrm[a]);
+                arm[a] = r0[a] + c3;
                 if (side == 0) {
                     tg[a] = nrm[a];
-                    tg[4 + a] = r0[a] + c3;
+                    tg[4 + a] = arm[a];
                 }
             }
             if (side == 0) {
-                tg[3] = R(0.5) * nn;
-                vol = (double)r0[0] * (double)N[0] + (double)r0[1] * (double)N[1] + (double)r0[2] * (double)N[2];
-                B.tri_vol[t] = vol;
+                tg[3] = area;
+                if (!B.rigid)
+                    vol = (double)r0[0] * (double)N[0] + (double)r0[1] * (double)N[1] + (double)r0[2] * (double)N[2];
             }
+            if (B.rigid)
+                for (int a = 0; a < 3; ++a) arm[a] -= R(__ldcg(B.rstate + RigidState::XC + a) - B.origin[a]);
         }
         bool bad = false, diverged = false;
         for (int a = 0; a < 3; ++a) {
@@ -389,37 +425,6 @@ __device__ __forceinline__ void mls_body(const R *__restrict__ mom, const Lattic
         else if (bad)
             atomicCAS(err, 0, kErrBodyWall);
     }
-    // enclosed volume (membranes): a fixed-order partial per warp; the last
-    // block to finish sums the partials with a fixed-shape tree
-    // (deterministic whichever block is last)
-    if (!B.rigid) {
-        __shared__ int s_last;
-        const int npart = (npts + 31) / 32, part = slot >> 5;
-        vol = warp_sum(vol);
-        if (lane == 0 && part < npart) B.vol_part[part] = vol;
-        __syncthreads();
-        if (threadIdx.x == 0) {
-            __threadfence();
-            s_last = atomicAdd(B.vol_count, 1u) == (unsigned)nvb - 1;
-        }
-        __syncthreads();
-        if (s_last) {
-            __threadfence();
-            double s = 0.0;
-            for (int k = threadIdx.x; k < npart; k += blockDim.x) s += __ldcg(B.vol_part + k);
-            s = warp_sum(s);
-            __shared__ double wpart[8];
-            if (lane == 0) wpart[warp] = s;
-            __syncthreads();
-            if (threadIdx.x == 0) {
-                double tot = 0.0;
-                for (int w = 0; w < (int)blockDim.x / 32; ++w) tot += wpart[w];
-                *B.vol_sum = tot;
-                *B.vol_count = 0u;
-            }
-        }
-    }
-
     // weights and the support's nodes (r_k <= 1, Eq. intKernel): FP32 squared
     // distances, and the FP64 ones of nodes whose decision FP32 rounding
     // (below 1e-6 here) could flip
@@ -442,8 +447,8 @@ __device__ __forceinline__ void mls_body(const R *__restrict__ mom, const Lattic
         if (near) in = (in & ~near) | support_exact(near, frac[0], frac[1], frac[2], L.dist2_cut);
     }
     if constexpr (kChain) chain_wait();
-    if (p < 0) return;
-
+    R f6[6] = {R(0), R(0), R(0), R(0), R(0), R(0)};  // rigid: the point's share of the force and moment
+    if (p >= 0) {
     // ---------------- sums ----------------
     int ox[3], oy[3], oz[3];
 #pragma unroll
@@ -565,27 +570,64 @@ __device__ __forceinline__ void mls_body(const R *__restrict__ mom, const Lattic
             }
         const int t = (p - nm) >> 1, side = (p - nm) & 1;
         const R rn = (R(1) + cr) * pick<R>(L.nu_d, L.nu_f);
-        R *pr = (R *)B.probe + 8 * t + 4 * side;
-        pr[0] = cr / R(3);  // p - c_s^2 rho0
+        const R pr0 = cr / R(3);  // p - c_s^2 rho0
+        R tr[3];
 #pragma unroll
         for (int c = 0; c < 3; ++c) {
             R acc = R(0);
 #pragma unroll
             for (int a = 0; a < 3; ++a) acc += (gr[c][a] + gr[a][c]) * nrm[a];
-            pr[1 + c] = rn * acc;
+            tr[c] = rn * acc;
         }
+        if (!B.rigid) {
+            R *pr = (R *)B.probe + 8 * t + 4 * side;
+            pr[0] = pr0;
+            for (int c = 0; c < 3; ++c) pr[1 + c] = tr[c];
+        } else if (!B.rigid_force) {
+            // the probe's side of the stress jump (Eqs. hydroForP, hydroForNu):
+            // +-(-p n + tau . n) A and its moment about x_c
+            const R sA = side ? -area : area;
+            for (int c = 0; c < 3; ++c) f6[c] = (tr[c] - pr0 * nrm[c]) * sA;
+            f6[3] = arm[1] * f6[2] - arm[2] * f6[1];
+            f6[4] = arm[2] * f6[0] - arm[0] * f6[2];
+            f6[5] = arm[0] * f6[1] - arm[1] * f6[0];
+        } else if (side == 0) {
+            exchange_force<R>(B, t, area, arm, f6);
+        }
+    }
+    }
+    // the block's partial sums, in a fixed order: enclosed volume (membranes)
+    // or force and moment (rigid bodies)
+    __shared__ double red[6][8];
+    const int nw = blockDim.x >> 5;
+    if (B.rigid) {
+#pragma unroll
+        for (int q = 0; q < 6; ++q) {
+            const R sum = warp_sum(f6[q]);
+            if (lane == 0) red[q][warp] = (double)sum;
+        }
+    } else {
+        vol = warp_sum(vol);
+        if (lane == 0) red[0][warp] = vol;
+    }
+    __syncthreads();
+    if ((int)threadIdx.x < body_sums(B)) {
+        double acc = 0.0;
+        for (int k = 0; k < nw; ++k) acc += red[threadIdx.x][k];
+        B.part[body_sums(B) * vb + threadIdx.x] = acc;
     }
 }
 
 // The blocks take the nvb groups of points in turn (gridDim.x = nvb unless
 // the launch caps the grid).
 template <typename R>
-__global__ void __launch_bounds__(kMlsThreads) k_mls(const R *__restrict__ mom, Lattice L, BodyView B,
+__global__ void __launch_bounds__(mls_threads(sizeof(R) == 8 ? 0 : 1)) k_mls(const R *__restrict__ mom, Lattice L, BodyView B,
                                                      int *err, int nvb) {
+    chain_release();  // the structure kernel may be scheduled beside this one
     for (int vb = blockIdx.x; vb < nvb; vb += gridDim.x) {
         // launched programmatically after the moments kernel, whose results
         // it waits for inside
-        mls_body<R, false, true>(mom, L, B, err, vb, nvb);
+        mls_body<R, false, true>(mom, L, B, err, vb);
         __syncthreads();  // the next group reuses the shared memory
     }
 }
@@ -600,47 +642,74 @@ __device__ __forceinline__ void tri_hydro(const BodyView &B, int t, R *F) {
     for (int a = 0; a < 3; ++a) F[a] = (-(pp[0] - pm[0]) * tg[a] + (pp[1 + a] - pm[1 + a])) * A;
 }
 
-// What lane k < 27 of a marker's warp needs to spread to support node k: the
-// node (-1: r_k > 1, nothing to add), its transfer weight phi_k, and the
-// tile to flag (the lanes of the 8 block corners; -1 on the others).
+// Spreading by the 8 lanes of a marker: c phi_k F added to the force field
+// at the support nodes with r_k <= 1 (the others have phi_k = 0), from the
+// marker's transfer record; the tiles of the block's 8 corners are flagged.
+constexpr int kLanes = 8;  // lanes per marker in the structure kernels
 template <typename R>
-struct SpreadLane {
-    int node, tile;
-    R phi;
-};
-template <typename R>
-__device__ __forceinline__ SpreadLane<R> spread_load(const Lattice &L, const BodyView &B, int p, int lane) {
-    SpreadLane<R> s;
-    s.node = s.tile = -1;
-    s.phi = R(0);
-    if (lane >= 27) return s;
-    const int i = lane % 3, j = (lane / 3) % 3, k = lane / 9;
+__device__ __forceinline__ void spread(const Lattice &L, const BodyView &B, int p, int l8, R c, const R *Fl,
+                                       R *__restrict__ force, uint32_t *stamp, uint32_t step) {
     const R *rec = (const R *)B.phi + (size_t)kRec * p;
     const int4 bs = reinterpret_cast<const int4 *>(B.node)[p];
-    const int x = support_coord(L, 0, bs.x + i - 1), y = support_coord(L, 1, bs.y + j - 1),
-              z = support_coord(L, 2, bs.z + k - 1);
-    if ((unsigned)bs.w >> lane & 1u) {
-        s.node = x + L.nx * (y + L.ny * z);
-        const R dx = R(i - 1) - rec[4], dy = R(j - 1) - rec[5], dz = R(k - 1) - rec[6];
-        s.phi = (rec[7 + i] * rec[10 + j] * rec[13 + k]) * (rec[0] + rec[1] * dx + rec[2] * dy + rec[3] * dz);
+    const R r0 = rec[0], r1 = rec[1], r2 = rec[2], r3 = rec[3], fx = rec[4], fy = rec[5], fz = rec[6];
+    const R F0 = c * Fl[0], F1 = c * Fl[1], F2 = c * Fl[2];
+    const long long st = L.stride;
+#pragma unroll
+    for (int q = l8; q < 27; q += kLanes) {
+        if (!((unsigned)bs.w >> q & 1u)) continue;
+        const int i = q % 3, j = (q / 3) % 3, k = q / 9;
+        const int node = support_coord(L, 0, bs.x + i - 1) +
+                         L.nx * (support_coord(L, 1, bs.y + j - 1) + L.ny * support_coord(L, 2, bs.z + k - 1));
+        const R phi = (rec[7 + i] * rec[10 + j] * rec[13 + k]) *
+                      (r0 + r1 * (R(i - 1) - fx) + r2 * (R(j - 1) - fy) + r3 * (R(k - 1) - fz));
+        atomicAdd(force + node, phi * F0);
+        atomicAdd(force + st + node, phi * F1);
+        atomicAdd(force + 2 * st + node, phi * F2);
     }
-    if (i != 1 && j != 1 && k != 1) s.tile = (x >> 3) + L.ntx * ((y >> 3) + L.nty * (z >> 3));
-    return s;
+    const int x = support_coord(L, 0, bs.x + (l8 & 1 ? 1 : -1)), y = support_coord(L, 1, bs.y + (l8 & 2 ? 1 : -1)),
+              z = support_coord(L, 2, bs.z + (l8 & 4 ? 1 : -1));
+    stamp[(x >> 3) + L.ntx * ((y >> 3) + L.nty * (z >> 3))] = step;
+}
+template <typename T>
+__device__ __forceinline__ T lanes_sum(T v) {  // over the 8 lanes of a marker
+#pragma unroll
+    for (int o = kLanes / 2; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
+    return v;
 }
 
-// Adds c phi_k F to the force field at the lane's support node and flags the
-// lane's tile.
-template <typename R>
-__device__ __forceinline__ void spread_lane(const Lattice &L, const SpreadLane<R> &s, R c, const R *Fl,
-                                            R *__restrict__ force, uint32_t *stamp, uint32_t step) {
-    if (s.node >= 0) {
-        const long long st = L.stride;
-        const R w = c * s.phi;
-        atomicAdd(force + s.node, w * Fl[0]);
-        atomicAdd(force + st + s.node, w * Fl[1]);
-        atomicAdd(force + 2 * st + s.node, w * Fl[2]);
+// A body's sum q over the partials of its MLS blocks (called by whole warps;
+// a fixed order).  Above kDirectParts partials k_body_sums has added them up
+// into the slot behind them.
+constexpr int kDirectParts = 512;
+__device__ __forceinline__ double body_sum(const BodyView &B, int nparts, int q) {
+    const int ns = body_sums(B), lane = threadIdx.x & 31;
+    if (nparts > kDirectParts) return __ldcg(B.part + (size_t)ns * nparts + q);
+    double s = 0.0;
+    for (int k = lane; k < nparts; k += 32) s += __ldcg(B.part + (size_t)ns * k + q);
+    return warp_sum(s);
+}
+__device__ __forceinline__ void body_sums_body(const BodyView &B, int nparts) {
+    const int ns = body_sums(B), lane = threadIdx.x & 31, nw = blockDim.x >> 5;
+    __shared__ double red[6][8];
+    // every warp takes a share of the partials of all sums
+    double s[6] = {0.0, 0.0, 0.0, 0.0, 0.0, 0.0};
+    for (int k = threadIdx.x; k < nparts; k += blockDim.x)
+        for (int q = 0; q < ns; ++q) s[q] += __ldcg(B.part + (size_t)ns * k + q);
+    for (int q = 0; q < ns; ++q) {
+        const double t = warp_sum(s[q]);
+        if (lane == 0) red[q][threadIdx.x >> 5] = t;
     }
-    if (s.tile >= 0) stamp[s.tile] = step;
+    __syncthreads();
+    if ((int)threadIdx.x < ns) {
+        double t = 0.0;
+        for (int w = 0; w < nw; ++w) t += red[threadIdx.x][w];
+        B.part[(size_t)ns * nparts + threadIdx.x] = t;
+    }
+}
+__global__ void __launch_bounds__(256) k_body_sums(BodyView B, int nparts) {
+    chain_release();
+    chain_wait();
+    body_sums_body(B, nparts);
 }
 
 // Node box of level n+1: each block reduces its markers' cells in shared
@@ -652,7 +721,7 @@ struct BlockBox {
         if (threadIdx.x < 6) v[threadIdx.x] = threadIdx.x < 3 ? 0x7fffffff : (int)0x80000000;
     }
     __device__ void add(int a, double x) {
-        const int c = (int)floor(x);
+        const int c = __double2int_rd(x);
         atomicMin(&v[a], c - kBoxLo);
         atomicMax(&v[3 + a], c + kBoxHi);
     }
@@ -664,38 +733,32 @@ struct BlockBox {
     }
 };
 
-// Membrane vertex update, one warp per vertex: spring (Eq. strainFor),
+// Membrane vertex update, 8 lanes per vertex: spring (Eq. strainFor),
 // bending (gradient of k_b[1 - cos(theta - theta0)], reading of Eq. bendFor),
 // volume penalty (restoring reading of Eq. volFor) and element hydrodynamic
 // forces shared 1/3 per vertex (Eq. newtonSoft), with the lanes sharing the
-// incident hinges and triangles; Verlet positions (Eqs. verletPos,
-// verletVel) in FP64, one lane per component; boundary velocity
-// U_b = U + F/m_v dt; the Lagrangian force F_l = U_b - U spread with
-// c_l = A_l (Eq. bodyforce).
+// incident hinges (12 on a regular mesh) and triangles (6); Verlet positions
+// (Eqs. verletPos, verletVel) in FP64, one thread per component; boundary
+// velocity U_b = U + F/m_v dt; the Lagrangian force F_l = U_b - U spread with
+// c_l = A_l (Eq. bodyforce).  The hinges need the positions only: launched
+// programmatically behind the MLS kernel they run beside it, and chain_wait
+// stands before the first use of its results.
 template <typename R>
 __device__ __forceinline__ void membrane_body(const Lattice &L, const BodyView &B, R *__restrict__ force,
                                               uint32_t *__restrict__ stamp, const uint32_t *__restrict__ dstep,
-                                              const int vb) {
-    const uint32_t step = __ldcg(dstep);  // written by the moments kernel of the step
+                                              const int vb, const int nparts) {
     __shared__ R s_cv;
     __shared__ BlockBox sbox;
-    __shared__ R s_F[8][4];   // per vertex warp: total force (3) and vertex area
-    __shared__ R s_Fl[8][3];  // per vertex warp: Lagrangian force
-    __shared__ double s_U[8][3];  // centroid markers: the vertex velocity
-    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-    const int v0 = vb * (blockDim.x >> 5);  // first vertex of the block
-    const int v = v0 + warp;
-    // the spreading lanes fetch their node and weight first
-    SpreadLane<R> sl{};
-    if (!B.centroid && v < B.nv) sl = spread_load<R>(L, B, v, lane);
-    if (threadIdx.x == 0) s_cv = R(B.kv * (1.0 - *B.vol_sum * B.inv_6V0));
+    __shared__ R s_F[32][3];       // per vertex: total force
+    __shared__ R s_Fl[32][3];      // per vertex: Lagrangian force
+    __shared__ double s_U[32][3];  // centroid markers: the vertex velocity
+    const int l8 = threadIdx.x & (kLanes - 1), g = threadIdx.x / kLanes;
+    const int nvpb = blockDim.x / kLanes, v0 = vb * nvpb, v = v0 + g;
+    R F[3] = {R(0), R(0), R(0)};
     sbox.init();
-    __syncthreads();
-    const R cv = s_cv;
     if (v < B.nv) {
     const R *Xr = (const R *)B.Xrel;
-    R F[3] = {R(0), R(0), R(0)};
-    for (int q = B.vh_ptr[v] + lane; q < B.vh_ptr[v + 1]; q += 32) {
+    for (int q = B.vh_ptr[v] + l8; q < B.vh_ptr[v + 1]; q += kLanes) {
         const int role = B.vh_list[q] & 3;
         const int4 H = B.vh_verts[q];
         const R *par = (const R *)B.vh_par + 4 * q;  // k_s, l0, k_b, theta0
@@ -763,53 +826,67 @@ __device__ __forceinline__ void membrane_body(const Lattice &L, const BodyView &
         const R g1 = c1 * le * il1, g2 = c2 * le * il2;  // c / h
         for (int a = 0; a < 3; ++a) F[a] -= dE * (g1 * n1[a] + g2 * n2[a]);
     }
-    // element terms: volume penalty and hydrodynamic force, 1/3 per vertex
-    R Al = R(0);
+    }
+    const int q1 = v < B.nv ? B.vt_ptr[v + 1] : 0, q0 = v < B.nv ? B.vt_ptr[v] + l8 : 0;
+    const int t0 = q0 < q1 ? B.vt_list[q0] / 3 : 0;
+    // components of the block's vertices integrated below: thread 3 j + a
+    const int j = threadIdx.x / 3, a = threadIdx.x % 3, vj = v0 + j;
+    const bool mine = (int)threadIdx.x < 3 * nvpb && vj < B.nv;
+    const double x = mine ? B.X[3 * vj + a] : 0.0, xp = mine ? B.Xprev[3 * vj + a] : 0.0;
+    chain_wait();
+    const uint32_t step = __ldcg(dstep);  // written by the moments kernel of the step
+    const double U0 = mine && !B.centroid ? B.U[3 * vj + a] : 0.0;
+    if ((int)threadIdx.x >= (int)blockDim.x - 32) {
+        const double v6 = body_sum(B, nparts, 0);
+        if ((threadIdx.x & 31) == 0) s_cv = R(B.kv * (1.0 - v6 * B.inv_6V0));
+    }
+    // element terms: volume penalty (G, the vertex's share of sum A n) and
+    // hydrodynamic force, 1/3 per vertex
+    R Al = R(0), G[3] = {R(0), R(0), R(0)};
     double Uv[3] = {0.0, 0.0, 0.0};
-    for (int q = B.vt_ptr[v] + lane; q < B.vt_ptr[v + 1]; q += 32) {
-        const int t = B.vt_list[q] / 3;
+    for (int q = q0; q < q1; q += kLanes) {
+        const int t = q == q0 ? t0 : B.vt_list[q] / 3;
         const R *tg = (const R *)B.tri_geo + 8 * t;
-        Al += tg[3] / R(3);
+        const R A3 = tg[3] / R(3);
+        Al += A3;
         R Fh[3] = {R(0), R(0), R(0)};
         if (!B.kinematic) tri_hydro<R>(B, t, Fh);  // kinematic IB: the fluid's stresses stay in the fluid
-        for (int a = 0; a < 3; ++a) F[a] += (cv * tg[a] * tg[3] + Fh[a]) / R(3);
+        for (int a = 0; a < 3; ++a) {
+            G[a] += tg[a] * A3;
+            F[a] += Fh[a] / R(3);
+        }
         if (B.centroid)
-            for (int a = 0; a < 3; ++a) Uv[a] += (double)(tg[3] / R(3)) * B.Uc[3 * t + a];
+            for (int a = 0; a < 3; ++a) Uv[a] += (double)A3 * B.Uc[3 * t + a];
     }
-    for (int a = 0; a < 3; ++a) F[a] = warp_sum(F[a]);
-    Al = warp_sum(Al);
-    if (lane == 0) {
-        s_F[warp][0] = F[0];
-        s_F[warp][1] = F[1];
-        s_F[warp][2] = F[2];
-        s_F[warp][3] = Al;
-    }
+    for (int a = 0; a < 3; ++a) F[a] = lanes_sum(F[a]);
+    for (int a = 0; a < 3; ++a) G[a] = lanes_sum(G[a]);
+    Al = lanes_sum(Al);
     if (B.centroid) {
         // the vertex moves with the area-weighted mean of its triangles'
         // centroid velocities
-        for (int a = 0; a < 3; ++a) Uv[a] = warp_sum(Uv[a]);
-        if (lane == 0)
-            for (int a = 0; a < 3; ++a) s_U[warp][a] = Uv[a] / (double)Al;
+        for (int a = 0; a < 3; ++a) Uv[a] = lanes_sum(Uv[a]);
+        if (l8 == 0)
+            for (int a = 0; a < 3; ++a) s_U[g][a] = Uv[a] / (double)Al;
     }
+    __syncthreads();
+    if (l8 == 0) {
+        const R cv = s_cv;
+        for (int a = 0; a < 3; ++a) s_F[g][a] = F[a] + cv * G[a];
     }
     __syncthreads();
     // Newton (Eq. newtonSoft) and Verlet (Eqs. verletPos, verletVel), dt = 1,
-    // in FP64 for the block's 8 vertices at once: lane 3 j + a of one warp
-    // integrates component a of vertex j (FP64 issues per warp-instruction;
-    // the warp rotates over the SM sub-partitions from block to block)
-    if (warp == (vb & 7) && lane < 24 && v0 + lane / 3 < B.nv) {
-        const int j = lane / 3, a = lane % 3, vj = v0 + j;
+    // in FP64 for the block's vertices at once: thread 3 j + a integrates
+    // component a of vertex j (FP64 issues per warp-instruction, so the
+    // components fill whole warps)
+    if (mine) {
         const double acc = (double)s_F[j][a] * B.inv_mv;
-        double U;
+        double U = U0;
         if (B.centroid) {
             U = s_U[j][a];
             B.U[3 * vj + a] = U;
-        } else {
-            U = B.U[3 * vj + a];
         }
         const double Ub = U + acc;
         const double Fla = Ub - U;
-        const double x = B.X[3 * vj + a], xp = B.Xprev[3 * vj + a];
         double xn;
         if (B.kinematic) {
             xn = x + U;  // kinematic IB: advected with the interpolated fluid velocity
@@ -831,202 +908,120 @@ __device__ __forceinline__ void membrane_body(const Lattice &L, const BodyView &
         s_Fl[j][a] = R(Fla);
     }
     __syncthreads();
-    if (!B.centroid && v < B.nv)
-        spread_lane<R>(L, sl, s_F[warp][3], s_Fl[warp], force, stamp, step);
-    __syncthreads();
+    if (!B.centroid && v < B.nv) spread<R>(L, B, v, l8, Al, s_Fl[g], force, stamp, step);
     sbox.flush(B.bbox_next);
 }
 
 template <typename R>
-__global__ void __launch_bounds__(256) k_membrane(Lattice L, BodyView B, R *__restrict__ force,
-                                                  uint32_t *__restrict__ stamp, const uint32_t *__restrict__ dstep,
-                                                  int nvb) {
+__global__ void __launch_bounds__(kStructThreads) k_membrane(Lattice L, BodyView B, R *__restrict__ force,
+                                                             uint32_t *__restrict__ stamp,
+                                                             const uint32_t *__restrict__ dstep, int nvb, int nparts) {
+    chain_release();
     for (int vb = blockIdx.x; vb < nvb; vb += gridDim.x) {
-        membrane_body<R>(L, B, force, stamp, dstep, vb);
+        membrane_body<R>(L, B, force, stamp, dstep, vb, nparts);
         __syncthreads();  // the next group of vertices reuses the shared memory
     }
 }
 
-// Rigid body: total force and moment of the element stresses, gravity
-// minus buoyancy, F = m du/dt and M = I dw/dt with I in the world frame,
-// second-order backward velocities (Eqs. linearVelRig, angularVelRig),
-// centre and orientation advanced with the new velocities.
-// One thread per triangle sums force and moment (fixed-shape block
-// reduction, FP64 partial per block); the last block to finish reduces the
-// partials in block order and integrates with lanes 0..8 of one warp
-// working on the components side by side (FP64 issues per
-// warp-instruction, so the update is written across lanes).
-template <typename R>
-__device__ __forceinline__ void rigid_forces_body(const BodyView &B, const int vb, const int nvb) {
-    __shared__ double red[6][8];
-    __shared__ int s_last;
-    __shared__ double sF[6], sR[9], sY[3], sQ[4];
-    double *S = B.rstate;
-    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-    const R xc[3] = {R(S[RigidState::XC] - B.origin[0]), R(S[RigidState::XC + 1] - B.origin[1]),
-                     R(S[RigidState::XC + 2] - B.origin[2])};
-    R f[6] = {R(0), R(0), R(0), R(0), R(0), R(0)};
-    const int t = vb * blockDim.x + threadIdx.x;
-    if (t < B.nt && !B.rigid_force) {
-        R Fh[3];
-        tri_hydro<R>(B, t, Fh);
-        const R *tg = (const R *)B.tri_geo + 8 * t;
-        const R r[3] = {tg[4] - xc[0], tg[5] - xc[1], tg[6] - xc[2]};
-        f[0] = Fh[0];
-        f[1] = Fh[1];
-        f[2] = Fh[2];
-        f[3] = r[1] * Fh[2] - r[2] * Fh[1];
-        f[4] = r[2] * Fh[0] - r[0] * Fh[2];
-        f[5] = r[0] * Fh[1] - r[1] * Fh[0];
-    } else if (t < B.nt && B.centroid) {
-        // momentum exchange, centroid markers: minus the previous step's IB
-        // force of the triangle's marker times its area, about x_c
-        const R *tg = (const R *)B.tri_geo + 8 * t;
-        const R c = -tg[3];
-        const R Fv[3] = {c * R(B.Flc[3 * t]), c * R(B.Flc[3 * t + 1]), c * R(B.Flc[3 * t + 2])};
-        const R r[3] = {tg[4] - xc[0], tg[5] - xc[1], tg[6] - xc[2]};
-        f[0] = Fv[0];
-        f[1] = Fv[1];
-        f[2] = Fv[2];
-        f[3] = r[1] * Fv[2] - r[2] * Fv[1];
-        f[4] = r[2] * Fv[0] - r[0] * Fv[2];
-        f[5] = r[0] * Fv[1] - r[1] * Fv[0];
-    } else if (t < B.nt) {
-        // momentum exchange: minus the IB force of the previous step, each
-        // corner carrying a third of the triangle's area (sum_l A_l F_l)
-        const R *tg = (const R *)B.tri_geo + 8 * t;
-        const R c = -tg[3] / R(3);
-        const R *Xr = (const R *)B.Xrel;
-        for (int q = 0; q < 3; ++q) {
-            const int v = B.tri[3 * t + q];
-            const R Fv[3] = {c * R(B.Fl[3 * v]), c * R(B.Fl[3 * v + 1]), c * R(B.Fl[3 * v + 2])};
-            const R r[3] = {Xr[3 * v] - xc[0], Xr[3 * v + 1] - xc[1], Xr[3 * v + 2] - xc[2]};
-            f[0] += Fv[0];
-            f[1] += Fv[1];
-            f[2] += Fv[2];
-            f[3] += r[1] * Fv[2] - r[2] * Fv[1];
-            f[4] += r[2] * Fv[0] - r[0] * Fv[2];
-            f[5] += r[0] * Fv[1] - r[1] * Fv[0];
-        }
-    }
-    for (int q = 0; q < 6; ++q) {
-        const R w = warp_sum(f[q]);
-        if (lane == 0) red[q][warp] = (double)w;
-    }
-    __syncthreads();
-    if (threadIdx.x < 6) {
-        double acc = 0.0;
-        for (int w = 0; w < 8; ++w) acc += red[threadIdx.x][w];
-        B.vol_part[6 * vb + threadIdx.x] = acc;
-    }
-    __syncthreads();
-    if (threadIdx.x == 0) {
-        __threadfence();
-        s_last = atomicAdd(B.vol_count, 1u) == (unsigned)nvb - 1;
-    }
-    __syncthreads();
-    if (!s_last) return;
-    __threadfence();
-    // totals: warp q < 6 sums partial q over the blocks, lane l taking blocks
-    // l, l + 32, ... and the warp's fixed butterfly adding the lanes
-    // (deterministic whichever block is last)
-    if (warp < 6) {
-        double acc = 0.0;
-        for (int b = lane; b < nvb; b += 32) acc += __ldcg(B.vol_part + 6 * b + warp);
-        acc = warp_sum(acc);
-        if (lane == 0) {
-            if (warp < 3) acc += (S[RigidState::DENS] - 1.0) * S[RigidState::VOL] * S[RigidState::GRAV + warp];
+// Rigid body: F = m du/dt and M = I dw/dt with I in the world frame and F
+// the element stresses (or the momentum exchange) plus gravity minus
+// buoyancy, second-order backward velocities (Eqs. linearVelRig,
+// angularVelRig), centre and orientation advanced with the new velocities.
+//
+// Every block of the marker kernel does this for itself with one warp: FP64
+// is a serial chain here (64 cycles per dependent operation, 16 per
+// independent one, whatever the lanes), so a kernel of its own cost 10 us on
+// 1280 triangles, most of it launch, cross-block reduction and the chain.
+// What does not need the step's force is formed before the MLS kernel ends
+// (rigid_prepare), the velocities follow in five operations
+// (rigid_velocities), and the orientation (rigid_orientation) is advanced
+// while the other warps form the markers' IB force.
+struct RigidBlock {
+    double S[RigidState::SIZE];  // state of level n, then of level n+1
+    double W[9], T[9];           // R I_b^-1 R^T, and I_b^-1 R^T
+    double c[6];                 // 2 v(t) - v(t - dt)/2 of u and w
+    double add[6];               // force and moment besides the element sums
+    double F[6];                 // the element sums
+    double xo[3];                // centre of level n
+    int last;
+};
+__device__ __forceinline__ void rigid_prepare(const BodyView &B, RigidBlock &r, const int lane) {
+    for (int k = lane; k < RigidState::SIZE; k += 32) r.S[k] = __ldcg(B.rstate + k);
+    __syncwarp();
+    const double *S = r.S, *Rm = S + RigidState::ROT, *Ii = S + RigidState::IBINV;
+    const int i = lane / 3, j = lane % 3;
+    if (lane < 9) r.T[lane] = Ii[3 * i] * Rm[3 * j] + Ii[3 * i + 1] * Rm[3 * j + 1] + Ii[3 * i + 2] * Rm[3 * j + 2];
+    if (lane < 6) {
+        const int v = lane < 3 ? RigidState::U : RigidState::W, vp = lane < 3 ? RigidState::UP : RigidState::WP;
+        r.c[lane] = 2.0 * S[v + j] - 0.5 * S[vp + j];
+        double add = 0.0;
+        if (lane < 3) {
+            add = (S[RigidState::DENS] - 1.0) * S[RigidState::VOL] * S[RigidState::GRAV + lane];
             // momentum exchange: the fluid inside moves with the body, rho_f V du/dt
-            if (warp < 3 && B.rigid_force)
-                acc += S[RigidState::VOL] * (S[RigidState::U + warp] - S[RigidState::UP + warp]);
-            sF[warp] = acc;
+            if (B.rigid_force) add += S[RigidState::VOL] * (S[RigidState::U + lane] - S[RigidState::UP + lane]);
+            r.xo[lane] = S[RigidState::XC + lane];
         }
-    }
-    __syncthreads();
-    if (warp != 0) return;
-    if (lane == 0) *B.vol_count = 0u;
-    __syncwarp();
-    const double *q = S + RigidState::Q4;
-    // rotation matrix of q, entry lane < 9
-    if (lane < 9) {
-        const double w = q[0], x = q[1], y = q[2], z = q[3];
-        const int i = lane / 3, j = lane % 3;
-        double v;
-        if (i == j) {
-            const double a2 = i == 0 ? y * y + z * z : i == 1 ? x * x + z * z : x * x + y * y;
-            v = 1.0 - 2.0 * a2;
-        } else {
-            // off-diagonal 2 (u_i u_j -+ w u_k), k the third axis
-            const double ui = i == 0 ? x : i == 1 ? y : z, uj = j == 0 ? x : j == 1 ? y : z;
-            const int k = 3 - i - j;
-            const double uk = k == 0 ? x : k == 1 ? y : z;
-            const bool plus = (i == 0 && j == 2) || (i == 1 && j == 0) || (i == 2 && j == 1);
-            v = 2.0 * (ui * uj + (plus ? w * uk : -w * uk));
-        }
-        sR[lane] = v;
+        r.add[lane] = add;
     }
     __syncwarp();
-    // dw/dt = I_world^-1 M = R I_b^-1 R^T M, lanes 0..2
+    if (lane < 9) r.W[lane] = Rm[3 * i] * r.T[j] + Rm[3 * i + 1] * r.T[3 + j] + Rm[3 * i + 2] * r.T[6 + j];
     if (B.rigid_force) {
-        // and I_f dw/dt = R I_b R^T (w - wp) rho_f / rho_s
-        if (lane < 3) {
-            const double *w = S + RigidState::W, *wp = S + RigidState::WP;
-            sY[lane] = sR[lane] * (w[0] - wp[0]) + sR[3 + lane] * (w[1] - wp[1]) + sR[6 + lane] * (w[2] - wp[2]);
-        }
+        // and I_f dw/dt = R I_b R^T (w - wp) rho_f / rho_s (r.T reused)
+        const double *w = S + RigidState::W, *wp = S + RigidState::WP, *Ib = S + RigidState::IB;
         __syncwarp();
-        double iy = 0.0;
-        if (lane < 3) {
-            const double *Ib = S + RigidState::IB + 3 * lane;
-            iy = Ib[0] * sY[0] + Ib[1] * sY[1] + Ib[2] * sY[2];
-        }
+        if (lane < 3) r.T[lane] = Rm[lane] * (w[0] - wp[0]) + Rm[3 + lane] * (w[1] - wp[1]) + Rm[6 + lane] * (w[2] - wp[2]);
         __syncwarp();
-        if (lane < 3) sY[lane] = iy;
+        if (lane < 3) r.T[3 + lane] = Ib[3 * lane] * r.T[0] + Ib[3 * lane + 1] * r.T[1] + Ib[3 * lane + 2] * r.T[2];
         __syncwarp();
         if (lane < 3)
-            sF[3 + lane] += (sR[3 * lane] * sY[0] + sR[3 * lane + 1] * sY[1] + sR[3 * lane + 2] * sY[2]) /
-                            S[RigidState::DENS];
-        __syncwarp();
-    }
-    if (lane < 3) sY[lane] = sR[lane] * sF[3] + sR[3 + lane] * sF[4] + sR[6 + lane] * sF[5];  // R^T M
-    __syncwarp();
-    double zl = 0.0;
-    if (lane < 3) {
-        const double *Ii = S + RigidState::IBINV + 3 * lane;
-        zl = Ii[0] * sY[0] + Ii[1] * sY[1] + Ii[2] * sY[2];
+            r.add[3 + lane] =
+                (Rm[3 * lane] * r.T[3] + Rm[3 * lane + 1] * r.T[4] + Rm[3 * lane + 2] * r.T[5]) / S[RigidState::DENS];
     }
     __syncwarp();
-    if (lane < 3) sY[lane] = zl;
-    __syncwarp();
-    // lanes 0..2: linear velocity and centre; lanes 3..5: angular velocity
-    double vn = 0.0;
+}
+// The body's sums over the MLS blocks' partials, 16 lanes each.
+__device__ __forceinline__ void rigid_sums(const BodyView &B, RigidBlock &r, const int nparts) {
+    const int h = threadIdx.x >> 4, l = threadIdx.x & 15, nh = blockDim.x >> 4;
+    for (int q0 = 0; q0 < 6; q0 += nh) {
+        const int q = q0 + h;
+        double t = 0.0;
+        if (q < 6) {
+            if (nparts > kDirectParts)
+                t = l == 0 ? __ldcg(B.part + 6 * (size_t)nparts + q) : 0.0;
+            else
+                for (int k = l; k < nparts; k += 16) t += __ldcg(B.part + 6 * (size_t)k + q);
+        }
+#pragma unroll
+        for (int o = 8; o > 0; o >>= 1) t += __shfl_xor_sync(0xffffffffu, t, o);
+        if (q < 6 && l == 0) r.F[q] = t;
+    }
+}
+__device__ __forceinline__ void rigid_velocities(RigidBlock &r, const int lane) {
+    double *S = r.S;
     if (lane < 6) {
         const int a = lane % 3;
-        double vdot, v1, v2;
+        double vdot;
         if (lane < 3) {
-            vdot = sF[a] * S[RigidState::INVM];
-            v1 = S[RigidState::U + a];
-            v2 = S[RigidState::UP + a];
+            vdot = (r.F[a] + r.add[a]) * S[RigidState::INVM];
         } else {
-            vdot = sR[3 * a] * sY[0] + sR[3 * a + 1] * sY[1] + sR[3 * a + 2] * sY[2];
-            v1 = S[RigidState::W + a];
-            v2 = S[RigidState::WP + a];
+            vdot = r.W[3 * a] * (r.F[3] + r.add[3]) + r.W[3 * a + 1] * (r.F[4] + r.add[4]) +
+                   r.W[3 * a + 2] * (r.F[5] + r.add[5]);
         }
-        vn = 2.0 / 3.0 * (2.0 * v1 - 0.5 * v2 + vdot);
+        const double vn = 2.0 / 3.0 * (r.c[lane] + vdot);
+        const int v = lane < 3 ? RigidState::U : RigidState::W, vp = lane < 3 ? RigidState::UP : RigidState::WP;
+        S[vp + a] = S[v + a];
+        S[v + a] = vn;
     }
     __syncwarp();
+}
+__device__ __forceinline__ void rigid_orientation(RigidBlock &r, const int lane) {
+    double *S = r.S;
     if (lane < 3) {
-        const double x0 = S[RigidState::XC + lane];
-        S[RigidState::XC_OLD + lane] = x0;
-        S[RigidState::XC + lane] = x0 + vn;
-        S[RigidState::UP + lane] = S[RigidState::U + lane];
-        S[RigidState::U + lane] = vn;
-    } else if (lane < 6) {
-        S[RigidState::WP + lane - 3] = S[RigidState::W + lane - 3];
-        S[RigidState::W + lane - 3] = vn;
+        S[RigidState::XC_OLD + lane] = r.xo[lane];
+        S[RigidState::XC + lane] = r.xo[lane] + S[RigidState::U + lane];
     }
     // rotation by |w| about w: dq = (cos(|w|/2), sin(|w|/2) w/|w|)
-    const double w0 = __shfl_sync(0xffffffffu, vn, 3), w1 = __shfl_sync(0xffffffffu, vn, 4),
-                 w2 = __shfl_sync(0xffffffffu, vn, 5);
+    const double w0 = S[RigidState::W], w1 = S[RigidState::W + 1], w2 = S[RigidState::W + 2];
     const double th2 = w0 * w0 + w1 * w1 + w2 * w2;
     double c, sth;  // cos(|w|/2) and sin(|w|/2)/|w|
     if (th2 < 1e-6) {
@@ -1040,136 +1035,155 @@ __device__ __forceinline__ void rigid_forces_body(const BodyView &B, const int v
         sincos(0.5 * wl, &sn, &c);
         sth = sn / wl;
     }
-    const double dq[4] = {c, sth * w0, sth * w1, sth * w2};
-    double qn = q[0];
-    if (th2 > 0.0 && lane < 4) {
-        // component lane of dq (x) q
-        if (lane == 0) qn = dq[0] * q[0] - dq[1] * q[1] - dq[2] * q[2] - dq[3] * q[3];
-        if (lane == 1) qn = dq[0] * q[1] + dq[1] * q[0] + dq[2] * q[3] - dq[3] * q[2];
-        if (lane == 2) qn = dq[0] * q[2] - dq[1] * q[3] + dq[2] * q[0] + dq[3] * q[1];
-        if (lane == 3) qn = dq[0] * q[3] + dq[1] * q[2] - dq[2] * q[1] + dq[3] * q[0];
-    } else if (lane < 4) {
-        qn = q[lane];
-    }
-    double qq = lane < 4 ? qn * qn : 0.0;
+    // component l = lane & 3 of dq (x) q: sum over k of +-dq_k q_(l xor k), the
+    // minus signs those of the quaternion product
+    const int l = lane & 3;
+    const double *q = S + RigidState::Q4;
+    auto term = [&](int k, bool minus) { return minus ? -q[l ^ k] : q[l ^ k]; };
+    double qn = c * q[l] + (sth * w0) * term(1, l == 0 || l == 2) + (sth * w1) * term(2, l == 0 || l == 3) +
+                (sth * w2) * term(3, l == 0 || l == 1);
+    if (!(th2 > 0.0)) qn = q[l];
+    double qq = qn * qn;
     qq += __shfl_xor_sync(0xffffffffu, qq, 1);
     qq += __shfl_xor_sync(0xffffffffu, qq, 2);
-    if (lane < 4) {
-        double r = (double)rsqrtf((float)qq);  // 1/sqrt(qq), refined twice
-        r = r * (1.5 - 0.5 * qq * r * r);
-        r = r * (1.5 - 0.5 * qq * r * r);
-        if (th2 > 0.0) qn *= r;
-        sQ[lane] = qn;
-        S[RigidState::Q4 + lane] = qn;
-    }
+    double rs = (double)rsqrtf((float)qq);  // 1/sqrt(qq), refined twice
+    rs = rs * (1.5 - 0.5 * qq * rs * rs);
+    rs = rs * (1.5 - 0.5 * qq * rs * rs);
+    if (th2 > 0.0) qn *= rs;
+    __syncwarp();
+    if (lane < 4) S[RigidState::Q4 + lane] = qn;
     __syncwarp();
     if (lane < 9) {
-        const double w = sQ[0], x = sQ[1], y = sQ[2], z = sQ[3];
+        // entry (i, j): 1 - 2 (a^2 + b^2) of the other two components on the
+        // diagonal, else 2 (u_i u_j -+ w u_k), k the third axis; one form for
+        // both, base - 2 (f0 f1 + f2 f3)
         const int i = lane / 3, j = lane % 3;
-        double v;
-        if (i == j) {
-            const double a2 = i == 0 ? y * y + z * z : i == 1 ? x * x + z * z : x * x + y * y;
-            v = 1.0 - 2.0 * a2;
-        } else {
-            const double ui = i == 0 ? x : i == 1 ? y : z, uj = j == 0 ? x : j == 1 ? y : z;
-            const int k = 3 - i - j;
-            const double uk = k == 0 ? x : k == 1 ? y : z;
-            const bool plus = (i == 0 && j == 2) || (i == 1 && j == 0) || (i == 2 && j == 1);
-            v = 2.0 * (ui * uj + (plus ? w * uk : -w * uk));
-        }
-        S[RigidState::ROT + lane] = v;
+        const int k = i == j ? (i + 2) % 3 : 3 - i - j;
+        const bool plus = (j - i + 3) % 3 == 2;
+        const double w = q[0], ui = q[1 + i], uj = q[1 + j], uk = q[1 + k], a = q[1 + (i + 1) % 3];
+        const double f0 = i == j ? a : -ui, f1 = i == j ? a : uj;
+        const double f2 = i == j ? uk : plus ? -w : w, f3 = uk;
+        S[RigidState::ROT + lane] = (i == j ? 1.0 : 0.0) - 2.0 * (f0 * f1 + f2 * f3);
+    }
+    __syncwarp();
+}
+// After every warp's last read of the old state (a block barrier before):
+// the last block of the kernel to get here writes the new one.
+__device__ __forceinline__ void rigid_commit(const BodyView &B, RigidBlock &r, const int nblocks, const int lane) {
+    if (lane == 0) {
+        __threadfence();
+        r.last = atomicAdd(B.vol_count, 1u) == (unsigned)nblocks - 1;
+    }
+    __syncwarp();
+    if (r.last) {
+        for (int k = lane; k < RigidState::SIZE; k += 32) B.rstate[k] = r.S[k];
+        if (lane == 0) *B.vol_count = 0u;
     }
 }
 
-template <typename R>
-__global__ void __launch_bounds__(256) k_rigid_forces(BodyView B) {
-    rigid_forces_body<R>(B, blockIdx.x, gridDim.x);
-}
-
-// Rigid markers, one warp each: boundary velocity u + w x (X - x_c) of
-// level n, IB force and spreading, then the markers of level n+1.
+// Rigid markers, 8 lanes each: boundary velocity u + w x (X - x_c) of
+// level n, IB force and spreading, then the markers of level n+1.  The
+// block takes the groups vb, vb + stride, ... below nvb; nblocks blocks work
+// on the body.
 template <typename R>
 __device__ __forceinline__ void rigid_markers_body(const Lattice &L, const BodyView &B, R *__restrict__ force,
-                                                   uint32_t *__restrict__ stamp,
-                                                   const uint32_t *__restrict__ dstep, const int vb) {
-    const uint32_t step = __ldcg(dstep);  // written by the moments kernel of the step
+                                                   uint32_t *__restrict__ stamp, const uint32_t *__restrict__ dstep,
+                                                   int vb, const int stride, const int nvb, const int nparts,
+                                                   const int nblocks) {
+    __shared__ RigidBlock r;
     __shared__ BlockBox sbox;
-    __shared__ R s_Al[8];
-    __shared__ R s_Fl[8][3];
-    __shared__ double s_U[8][3];  // centroid markers: the vertex velocity
-    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-    const int v0 = vb * (blockDim.x >> 5);
-    const int v = v0 + warp;
+    __shared__ R s_Fl[32][3];
+    __shared__ double s_U[32][3];  // centroid markers: the vertex velocity
+    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    const int l8 = threadIdx.x & (kLanes - 1), g = threadIdx.x / kLanes, nvpb = blockDim.x / kLanes;
+    // FP64 for the block's markers at once: thread 32 + 3 j + a handles
+    // component a of marker j (warp 0 advances the body meanwhile)
+    const int comp = (int)threadIdx.x - 32, j = comp / 3, a = comp % 3, a1 = (a + 1) % 3, a2 = (a + 2) % 3;
+    if (warp == 0) rigid_prepare(B, r, lane);
     sbox.init();
-    SpreadLane<R> sl{};
-    if (!B.centroid && v < B.nv) sl = spread_load<R>(L, B, v, lane);
-    if (v < B.nv) {
+    for (bool first = true; vb < nvb; vb += stride, first = false) {
+        const int v0 = vb * nvpb, v = v0 + g, vj = v0 + j;
+        const bool mine = comp >= 0 && comp < 3 * nvpb && vj < B.nv;
+        // what the MLS kernel does not write
+        double x[3] = {0.0, 0.0, 0.0}, xb[3] = {0.0, 0.0, 0.0};
+        if (mine)
+            for (int k = 0; k < 3; ++k) {
+                x[k] = B.X[3 * vj + (a + k) % 3];
+                xb[k] = B.Xbody[3 * vj + k];
+            }
+        const int q1 = v < B.nv ? B.vt_ptr[v + 1] : 0, q0 = v < B.nv ? B.vt_ptr[v] + l8 : 0;
+        const int t0 = q0 < q1 ? B.vt_list[q0] / 3 : 0;
+        chain_wait();
+        if (first) rigid_sums(B, r, nparts);
+        const uint32_t step = __ldcg(dstep);  // written by the moments kernel of the step
+        const double U0 = mine && !B.centroid ? B.U[3 * vj + a] : 0.0;
         R Al = R(0);
         double Uv[3] = {0.0, 0.0, 0.0};
-        for (int q = B.vt_ptr[v] + lane; q < B.vt_ptr[v + 1]; q += 32) {
-            const int t = B.vt_list[q] / 3;
+        for (int q = q0; q < q1; q += kLanes) {
+            const int t = q == q0 ? t0 : B.vt_list[q] / 3;
             const R At3 = ((const R *)B.tri_geo)[8 * t + 3] / R(3);
             Al += At3;
             if (B.centroid)
-                for (int a = 0; a < 3; ++a) Uv[a] += (double)At3 * B.Uc[3 * t + a];
+                for (int k = 0; k < 3; ++k) Uv[k] += (double)At3 * B.Uc[3 * t + k];
         }
-        Al = warp_sum(Al);
-        if (lane == 0) s_Al[warp] = Al;
+        Al = lanes_sum(Al);
         if (B.centroid) {
             // the vertex velocity: area-weighted mean of its triangles'
             // centroid velocities
-            for (int a = 0; a < 3; ++a) Uv[a] = warp_sum(Uv[a]);
-            if (lane == 0)
-                for (int a = 0; a < 3; ++a) s_U[warp][a] = Uv[a] / (double)Al;
+            for (int k = 0; k < 3; ++k) Uv[k] = lanes_sum(Uv[k]);
+            if (l8 == 0)
+                for (int k = 0; k < 3; ++k) s_U[g][k] = Uv[k] / (double)Al;
         }
-    }
-    __syncthreads();
-    // FP64 for the block's 8 markers at once: lane 3 j + a of one warp
-    // handles component a of marker j
-    if (warp == (vb & 7) && lane < 24 && v0 + lane / 3 < B.nv) {
-        const int j = lane / 3, a = lane % 3, vj = v0 + j, a1 = (a + 1) % 3, a2 = (a + 2) % 3;
-        const double *S = B.rstate;
-        const double *un = S + RigidState::U, *wn = S + RigidState::W, *xo = S + RigidState::XC_OLD;
-        const double *xc = S + RigidState::XC, *Rn = S + RigidState::ROT;
-        const double r1 = B.X[3 * vj + a1] - xo[a1], r2 = B.X[3 * vj + a2] - xo[a2];
-        const double ub = un[a] + (wn[a1] * r2 - wn[a2] * r1);  // (w x r)_a
-        double U;
-        if (B.centroid) {
-            U = s_U[j][a];
-            B.U[3 * vj + a] = U;
-        } else {
-            U = B.U[3 * vj + a];
+        if (first) {
+            __syncthreads();
+            if (warp == 0) rigid_velocities(r, lane);
         }
-        const double Fla = ub - U;
-        B.Ub[3 * vj + a] = ub;
-        B.Fl[3 * vj + a] = Fla;
-        const double *xb = B.Xbody + 3 * vj;
-        const double xn = xc[a] + Rn[3 * a] * xb[0] + Rn[3 * a + 1] * xb[1] + Rn[3 * a + 2] * xb[2];
-        // a marker moving a lattice unit or more in one step (or a NaN) has
-        // diverged
-        if (!(fabs(xn - B.X[3 * vj + a]) < kMaxMarkerStep)) atomicCAS(B.err, 0, kErrDiverged);
-        B.Xnew[3 * vj + a] = xn;
-        ((R *)B.Xrel_next)[3 * vj + a] = R(xn - B.origin[a]);
-        sbox.add(a, xn);
-        s_Fl[j][a] = R(Fla);
+        __syncthreads();
+        const double *S = r.S;
+        if (mine) {
+            const double *un = S + RigidState::U, *wn = S + RigidState::W;
+            const double r1 = x[1] - r.xo[a1], r2 = x[2] - r.xo[a2];
+            const double ub = un[a] + (wn[a1] * r2 - wn[a2] * r1);  // (w x r)_a
+            double U = U0;
+            if (B.centroid) {
+                U = s_U[j][a];
+                B.U[3 * vj + a] = U;
+            }
+            const double Fla = ub - U;
+            B.Ub[3 * vj + a] = ub;
+            B.Fl[3 * vj + a] = Fla;
+            s_Fl[j][a] = R(Fla);
+        } else if (first && warp == 0) {
+            rigid_orientation(r, lane);
+        }
+        __syncthreads();
+        if (!B.centroid && v < B.nv) spread<R>(L, B, v, l8, Al, s_Fl[g], force, stamp, step);
+        if (mine) {
+            const double *xc = S + RigidState::XC, *Rn = S + RigidState::ROT;
+            const double xn = xc[a] + Rn[3 * a] * xb[0] + Rn[3 * a + 1] * xb[1] + Rn[3 * a + 2] * xb[2];
+            // a marker moving a lattice unit or more in one step (or a NaN)
+            // has diverged
+            if (!(fabs(xn - x[0]) < kMaxMarkerStep)) atomicCAS(B.err, 0, kErrDiverged);
+            B.Xnew[3 * vj + a] = xn;
+            ((R *)B.Xrel_next)[3 * vj + a] = R(xn - B.origin[a]);
+            sbox.add(a, xn);
+        }
+        if (first && warp == 0) rigid_commit(B, r, nblocks, lane);
+        __syncthreads();
     }
-    __syncthreads();
-    if (!B.centroid && v < B.nv) spread_lane<R>(L, sl, s_Al[warp], s_Fl[warp], force, stamp, step);
-    __syncthreads();
     sbox.flush(B.bbox_next);
 }
 
 template <typename R>
-__global__ void __launch_bounds__(256) k_rigid_markers(Lattice L, BodyView B, R *__restrict__ force,
-                                                       uint32_t *__restrict__ stamp, const uint32_t *__restrict__ dstep,
-                                                       int nvb) {
-    for (int vb = blockIdx.x; vb < nvb; vb += gridDim.x) {
-        rigid_markers_body<R>(L, B, force, stamp, dstep, vb);
-        __syncthreads();  // the next group of markers reuses the shared memory
-    }
+__global__ void __launch_bounds__(kStructThreads) k_rigid_markers(Lattice L, BodyView B, R *__restrict__ force,
+                                                                  uint32_t *__restrict__ stamp,
+                                                                  const uint32_t *__restrict__ dstep, int nvb,
+                                                                  int nparts) {
+    chain_release();
+    rigid_markers_body<R>(L, B, force, stamp, dstep, blockIdx.x, gridDim.x, nvb, nparts, gridDim.x);
 }
 
-// IB force of centroid markers, one warp per triangle: the boundary
+// IB force of centroid markers, 8 lanes per triangle: the boundary
 // velocity at the centroid (rigid: u + w x (X_c - x_c) of level n;
 // membrane: the interpolated velocity advanced by the mean Newton
 // acceleration of the triangle's vertices, which the structure kernel left
@@ -1179,17 +1193,13 @@ __device__ __forceinline__ void centroid_body(const Lattice &L, const BodyView &
                                               uint32_t *__restrict__ stamp, const uint32_t *__restrict__ dstep,
                                               const int vb) {
     const uint32_t step = __ldcg(dstep);  // written by the moments kernel of the step
-    __shared__ R s_A[8];
-    __shared__ R s_Fl[8][3];
-    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-    const int t0 = vb * 8, t = t0 + warp;
-    SpreadLane<R> sl{};
-    if (t < B.nt) sl = spread_load<R>(L, B, t, lane);
-    if (t < B.nt && lane == 0) s_A[warp] = ((const R *)B.tri_geo)[8 * t + 3];
-    // FP64 for the block's 8 markers at once: lane 3 j + a of one warp
-    // handles component a of marker j
-    if (warp == (vb & 7) && lane < 24 && t0 + lane / 3 < B.nt) {
-        const int j = lane / 3, a = lane % 3, tj = t0 + j;
+    __shared__ R s_Fl[32][3];
+    const int l8 = threadIdx.x & (kLanes - 1), g = threadIdx.x / kLanes;
+    const int ntpb = blockDim.x / kLanes, t0 = vb * ntpb, t = t0 + g;
+    // FP64 for the block's markers at once: thread 3 j + a handles component
+    // a of marker j
+    if ((int)threadIdx.x < 3 * ntpb && t0 + (int)threadIdx.x / 3 < B.nt) {
+        const int j = threadIdx.x / 3, a = threadIdx.x % 3, tj = t0 + j;
         const int *tv = B.tri + 3 * tj;
         const double uc = B.Uc[3 * tj + a];
         double ub;
@@ -1209,11 +1219,12 @@ __device__ __forceinline__ void centroid_body(const Lattice &L, const BodyView &
         s_Fl[j][a] = R(Fla);
     }
     __syncthreads();
-    if (t < B.nt) spread_lane<R>(L, sl, s_A[warp], s_Fl[warp], force, stamp, step);
+    if (t < B.nt)
+        spread<R>(L, B, t, l8, ((const R *)B.tri_geo)[8 * t + 3], s_Fl[g], force, stamp, step);
 }
 
 template <typename R>
-__global__ void __launch_bounds__(256) k_centroid_spread(Lattice L, BodyView B, R *__restrict__ force,
+__global__ void __launch_bounds__(kStructThreads) k_centroid_spread(Lattice L, BodyView B, R *__restrict__ force,
                                                          uint32_t *__restrict__ stamp,
                                                          const uint32_t *__restrict__ dstep) {
     centroid_body<R>(L, B, force, stamp, dstep, blockIdx.x);
@@ -1241,7 +1252,7 @@ __global__ void __launch_bounds__(kBatchMlsThreads) kb_mls(BatchTables T, int ph
     stage_shared(br, T.body + phase * T.nb + j);
     stage_shared(L, T.lat + br.lat);
     const LatRef &F = T.ref[phase * T.nl + br.lat];
-    mls_body<R>((const R *)F.mom, L, br.v, F.err, vb, nvb);
+    mls_body<R>((const R *)F.mom, L, br.v, F.err, vb);
 }
 
 template <typename R>
@@ -1252,15 +1263,15 @@ __global__ void __launch_bounds__(256) kb_membrane(BatchTables T, int phase) {
     stage_shared(br, T.body + phase * T.nb + __ldg(T.memb_id + m));
     stage_shared(L, T.lat + br.lat);
     const LatRef &F = T.ref[phase * T.nl + br.lat];
-    membrane_body<R>(L, br.v, (R *)F.force, F.stamp, F.d_step, blockIdx.x - __ldg(T.memb_pre + m));
+    membrane_body<R>(L, br.v, (R *)F.force, F.stamp, F.d_step, blockIdx.x - __ldg(T.memb_pre + m),
+                     points_blocks(br.v, kBatchMlsThreads));
 }
 
-template <typename R>
-__global__ void __launch_bounds__(256) kb_rigid_forces(BatchTables T, int phase) {
-    const int m = __ldg(T.rf_blk + blockIdx.x);
-    const BodyRef &br = T.body[phase * T.nb + __ldg(T.rigid_id + m)];
-    const int b0 = __ldg(T.rf_pre + m);
-    rigid_forces_body<R>(br.v, blockIdx.x - b0, __ldg(T.rf_pre + m + 1) - b0);
+// One block per body with more MLS partials than the structure kernels add up
+// by themselves.
+__global__ void __launch_bounds__(256) kb_body_sums(BatchTables T, int phase) {
+    const BodyRef &br = T.body[phase * T.nb + __ldg(T.sums_id + blockIdx.x)];
+    body_sums_body(br.v, points_blocks(br.v, kBatchMlsThreads));
 }
 
 template <typename R>
@@ -1271,7 +1282,9 @@ __global__ void __launch_bounds__(256) kb_rigid_markers(BatchTables T, int phase
     stage_shared(br, T.body + phase * T.nb + __ldg(T.rigid_id + m));
     stage_shared(L, T.lat + br.lat);
     const LatRef &F = T.ref[phase * T.nl + br.lat];
-    rigid_markers_body<R>(L, br.v, (R *)F.force, F.stamp, F.d_step, blockIdx.x - __ldg(T.rm_pre + m));
+    const int b0 = __ldg(T.rm_pre + m), nvb = __ldg(T.rm_pre + m + 1) - b0;
+    rigid_markers_body<R>(L, br.v, (R *)F.force, F.stamp, F.d_step, blockIdx.x - b0, nvb, nvb,
+                          points_blocks(br.v, kBatchMlsThreads), nvb);
 }
 
 template <typename R>
@@ -1327,9 +1340,9 @@ __device__ bool wait_deps(const PersistTables &P, int k, int l, int s) {
     switch (k) {
         case kPMom: return wait_kind(P, l, kPSweep, s - 1, t0);
         case kPMls: return wait_kind(P, l, kPMom, s, t0);
+        case kPSum: return wait_kind(P, l, kPMls, s, t0);
         case kPMemb:
-        case kPRf: return wait_kind(P, l, kPMls, s, t0);
-        case kPRm: return wait_kind(P, l, kPRf, s, t0);
+        case kPRm: return wait_kind(P, l, kPMls, s, t0) && wait_kind(P, l, kPSum, s, t0);
         case kPCen: return wait_kind(P, l, kPMemb, s, t0) && wait_kind(P, l, kPRm, s, t0);
         default:
             for (int j = kPMom; j < kPSweep; ++j)
@@ -1402,11 +1415,16 @@ __global__ void __launch_bounds__(256, 4) kp_batch(BatchTables T, PersistTables 
                                          br.inc_step ? F.d_step : nullptr, it.z, it.w);
                 break;
             case kPMls:
-                mls_body<R, true>((const R *)F.mom, L, br.v, F.err, it.z, it.w);
+                mls_body<R, true>((const R *)F.mom, L, br.v, F.err, it.z);
                 break;
-            case kPMemb: membrane_body<R>(L, br.v, (R *)F.force, F.stamp, F.d_step, it.z); break;
-            case kPRf: rigid_forces_body<R>(br.v, it.z, it.w); break;
-            case kPRm: rigid_markers_body<R>(L, br.v, (R *)F.force, F.stamp, F.d_step, it.z); break;
+            case kPSum: body_sums_body(br.v, points_blocks(br.v, kPersistThreads)); break;
+            case kPMemb:
+                membrane_body<R>(L, br.v, (R *)F.force, F.stamp, F.d_step, it.z, points_blocks(br.v, kPersistThreads));
+                break;
+            case kPRm:
+                rigid_markers_body<R>(L, br.v, (R *)F.force, F.stamp, F.d_step, it.z, it.w, it.w,
+                                      points_blocks(br.v, kPersistThreads), it.w);
+                break;
             default: centroid_body<R>(L, br.v, (R *)F.force, F.stamp, F.d_step, it.z); break;
         }
         __syncthreads();
@@ -1460,8 +1478,8 @@ template <typename S, typename R>
 static cudaError_t batch_ib_t(const BatchTables &T, const BatchGrid &G, int phase, cudaStream_t s) {
     if (G.mom > 0) kb_moments<S, R><<<G.mom, 256, 0, s>>>(T, phase);
     if (G.mls > 0) kb_mls<R><<<G.mls, kBatchMlsThreads, 0, s>>>(T, phase);
+    if (G.sums > 0) kb_body_sums<<<G.sums, 256, 0, s>>>(T, phase);
     if (G.memb > 0) kb_membrane<R><<<G.memb, 256, 0, s>>>(T, phase);
-    if (G.rf > 0) kb_rigid_forces<R><<<G.rf, 256, 0, s>>>(T, phase);
     if (G.rm > 0) kb_rigid_markers<R><<<G.rm, 256, 0, s>>>(T, phase);
     if (G.cen > 0) kb_centroid_spread<R><<<G.cen, 256, 0, s>>>(T, phase);  // after the structure kernels
     return cudaGetLastError();
@@ -1477,7 +1495,8 @@ cudaError_t launch_batch_ib(int prec, const BatchTables &T, const BatchGrid &G, 
 }
 
 // ---- launchers ----
-int mls_blocks(const BodyView &B, int threads) { return (B.nm + 2 * B.nt + threads - 1) / threads; }
+int mls_blocks(const BodyView &B, int threads) { return points_blocks(B, threads); }
+bool needs_body_sums(const BodyView &B, int threads) { return points_blocks(B, threads) > kDirectParts; }
 
 // Grid of n blocks' work under a cap (0: none).
 static int capped(int n, int cap) { return cap > 0 && cap < n ? cap : n; }
@@ -1488,11 +1507,11 @@ static cudaError_t ib_front_t(const void *fin, const Lattice &L, const BodyView 
     k_moments<S, R><<<2 * nsm, 256, 0, s>>>((const S *)fin, L, B.bbox, B.bbox_next, (R *)mom, step_inc);
     cudaError_t e = cudaGetLastError();
     if (e != cudaSuccess) return e;
-    // the MLS kernel is scheduled while the moments kernel ends (measured:
-    // about 2 us off the 96^3 capsule step; the same launch for the other
-    // kernels of the step made it slower)
-    const int nvb = mls_blocks(B, kMlsThreads);
-    return launch_chained(k_mls<R>, dim3(capped(nvb, grid_cap)), dim3(kMlsThreads), 0, s,
+    // the MLS kernel is scheduled while the moments kernel ends, and forms its
+    // points' positions and weights meanwhile
+    constexpr int threads = mls_threads(sizeof(R) == 8 ? 0 : 1);
+    const int nvb = mls_blocks(B, threads);
+    return launch_chained(k_mls<R>, dim3(capped(nvb, grid_cap)), dim3(threads), 0, s,
                           (const R *)mom, L, B, err, nvb);
 }
 
@@ -1508,43 +1527,49 @@ cudaError_t launch_ib_front(int prec, const void *fin, const Lattice &L, const B
 
 static cudaError_t launch_centroid(int prec, const Lattice &L, const BodyView &B, void *force, uint32_t *stamp,
                                    const uint32_t *step, cudaStream_t s) {
-    const unsigned g = (unsigned)((B.nt + 7) / 8);  // 8 warps (triangles) per block
+    const unsigned g = (unsigned)((B.nt + kStructThreads / kLanes - 1) / (kStructThreads / kLanes));
     if (prec == 0)
-        k_centroid_spread<double><<<g, 256, 0, s>>>(L, B, (double *)force, stamp, step);
+        k_centroid_spread<double><<<g, kStructThreads, 0, s>>>(L, B, (double *)force, stamp, step);
     else
-        k_centroid_spread<float><<<g, 256, 0, s>>>(L, B, (float *)force, stamp, step);
+        k_centroid_spread<float><<<g, kStructThreads, 0, s>>>(L, B, (float *)force, stamp, step);
     return cudaGetLastError();
 }
 
-cudaError_t launch_membrane(int prec, const Lattice &L, const BodyView &B, void *force, uint32_t *stamp,
-                            const uint32_t *step, int grid_cap, cudaStream_t s) {
-    const int nvb = (B.nv + 7) / 8;  // 8 warps (vertices) per block
-    const unsigned g = (unsigned)capped(nvb, grid_cap);
-    if (prec == 0)
-        k_membrane<double><<<g, 256, 0, s>>>(L, B, (double *)force, stamp, step, nvb);
-    else
-        k_membrane<float><<<g, 256, 0, s>>>(L, B, (float *)force, stamp, step, nvb);
-    cudaError_t e = cudaGetLastError();
-    if (e != cudaSuccess || !B.centroid) return e;
-    return launch_centroid(prec, L, B, force, stamp, step, s);
+// The structure kernel is launched programmatically behind the MLS kernel:
+// the membrane's hinge forces and the rigid body's preparation run beside
+// it.  Its blocks hold their registers while they wait, on SMs that a
+// far-field sweep could use, so only grids of at most this many blocks per SM
+// are launched so (96^3 capsule, 161 blocks: 45 us a step with, 49 without;
+// 160x160x480 sphere, 641 blocks: 343 with, 310 us without).
+constexpr int kChainPerSm = 2;
+
+template <typename... KArgs, typename... Args>
+static cudaError_t launch_struct(void (*kernel)(KArgs...), bool chained, unsigned grid, unsigned block, cudaStream_t s,
+                                 Args... args) {
+    if (chained) return launch_chained(kernel, dim3(grid), dim3(block), 0, s, args...);
+    kernel<<<grid, block, 0, s>>>(args...);
+    return cudaGetLastError();
 }
 
-cudaError_t launch_rigid(int prec, const Lattice &L, const BodyView &B, void *force, uint32_t *stamp,
-                         const uint32_t *step, int grid_cap, cudaStream_t s) {
-    const unsigned gf = (unsigned)((B.nt + 255) / 256);
-    if (prec == 0)
-        k_rigid_forces<double><<<gf, 256, 0, s>>>(B);
-    else
-        k_rigid_forces<float><<<gf, 256, 0, s>>>(B);
-    cudaError_t e = cudaGetLastError();
+cudaError_t launch_structure(int prec, const Lattice &L, const BodyView &B, void *force, uint32_t *stamp,
+                             const uint32_t *step, int nsm, int grid_cap, bool chained, cudaStream_t s) {
+    const int nparts = points_blocks(B, mls_threads(prec));
+    cudaError_t e = cudaSuccess;
+    if (nparts > kDirectParts) e = launch_struct(k_body_sums, chained, 1, 256, s, B, nparts);
     if (e != cudaSuccess) return e;
-    const int nvb = (B.nv + 7) / 8;
+    const int per = kStructThreads / kLanes, nvb = (B.nv + per - 1) / per;
     const unsigned g = (unsigned)capped(nvb, grid_cap);
-    if (prec == 0)
-        k_rigid_markers<double><<<g, 256, 0, s>>>(L, B, (double *)force, stamp, step, nvb);
+    chained = chained && (int)g <= kChainPerSm * nsm;
+    if (B.rigid)
+        e = prec == 0 ? launch_struct(k_rigid_markers<double>, chained, g, kStructThreads, s, L, B, (double *)force,
+                                      stamp, step, nvb, nparts)
+                      : launch_struct(k_rigid_markers<float>, chained, g, kStructThreads, s, L, B, (float *)force,
+                                      stamp, step, nvb, nparts);
     else
-        k_rigid_markers<float><<<g, 256, 0, s>>>(L, B, (float *)force, stamp, step, nvb);
-    e = cudaGetLastError();
+        e = prec == 0 ? launch_struct(k_membrane<double>, chained, g, kStructThreads, s, L, B, (double *)force, stamp,
+                                      step, nvb, nparts)
+                      : launch_struct(k_membrane<float>, chained, g, kStructThreads, s, L, B, (float *)force, stamp,
+                                      step, nvb, nparts);
     if (e != cudaSuccess || !B.centroid) return e;
     return launch_centroid(prec, L, B, force, stamp, step, s);
 }

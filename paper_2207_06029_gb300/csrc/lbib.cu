@@ -27,7 +27,7 @@ struct DevBody {
     lbib_body_params p{};
     double *X[3] = {nullptr, nullptr, nullptr};  // rotating buffers: prev, cur, next
     int cur = 1;
-    double *U = nullptr, *Ub = nullptr, *Fl = nullptr, *tri_vol = nullptr;
+    double *U = nullptr, *Ub = nullptr, *Fl = nullptr;
     double *Uc = nullptr, *Flc = nullptr;  // centroid markers
     void *phi = nullptr, *tri_geo = nullptr, *probe = nullptr;  // arithmetic precision R
     void *Xrel[2] = {nullptr, nullptr};                          // R: X - origin, current and next
@@ -40,11 +40,10 @@ struct DevBody {
     double *Xbody = nullptr, *rstate = nullptr;
     int *bbox[2] = {nullptr, nullptr};  // support-region node boxes, current and next
     int bcur = 0;
-    double *vol_part = nullptr, *vol_sum = nullptr;
+    double *part = nullptr;  // MLS partial sums (per-step scratch)
     unsigned int *vol_count = nullptr;
     int4 *vh_verts = nullptr;
     void *vh_par = nullptr;
-    int nvol_part = 0;
     double V0 = 0, A0 = 0, mv = 0, origin[3] = {0, 0, 0};
 };
 
@@ -297,7 +296,6 @@ BodyView make_view(Ctx *c, DevBody &b) {
     v.perm = b.perm;
     v.tri = b.tri;
     v.tri_geo = b.tri_geo;
-    v.tri_vol = b.tri_vol;
     v.probe = b.probe;
     v.Xrel = b.Xrel[b.bcur];
     v.Xrel_next = b.Xrel[1 - b.bcur];
@@ -325,14 +323,21 @@ BodyView make_view(Ctx *c, DevBody &b) {
     v.rstate = b.rstate;
     v.bbox = b.bbox[b.bcur];
     v.bbox_next = b.bbox[1 - b.bcur];
-    v.vol_part = b.vol_part;
-    v.nvol_part = b.nvol_part;
+    v.part = b.part;
     v.vol_count = b.vol_count;
-    v.vol_sum = b.vol_sum;
     v.vh_verts = b.vh_verts;
     v.vh_par = b.vh_par;
     v.err = c->d_err;
     return v;
+}
+
+// Blocks of the batched structure kernels (and of the persistent kernel's
+// structure items) for n markers.
+int marker_blocks(int n) { return (n + kMarkersPerBlock - 1) / kMarkersPerBlock; }
+
+// Kernels of a body's structure stage.
+int structure_launches(int prec, const BodyView &v) {
+    return 1 + needs_body_sums(v, mls_threads(prec)) + (v.centroid ? 1 : 0);
 }
 
 int check_device_error(Ctx *c) {
@@ -847,7 +852,9 @@ int lbib_add_body(void *h, const double *verts, int nv, const int *tris, int nt,
         b.perm = upload(c, perm, &rc);
     }
     b.tri_geo = dev_alloc(c, c->relem * 8 * (size_t)nt);
-    b.tri_vol = (double *)dev_alloc(c, sizeof(double) * (size_t)nt);
+    // (space of checkpoints written when the step kept the triangles' volume
+    // terms; the same below for the reductions' partials and sum)
+    double *const old_terms = (double *)dev_alloc(c, sizeof(double) * (size_t)nt);
     b.probe = dev_alloc(c, c->relem * 8 * (size_t)nt);
     b.vh_ptr = upload(c, vh_ptr, &rc);
     b.vh_list = upload(c, vh_list, &rc);
@@ -931,12 +938,13 @@ int lbib_add_body(void *h, const double *verts, int nv, const int *tris, int nt,
         tmp.nv = nv;
         tmp.nt = nt;
         tmp.nm = nm;
-        // partial sums: one per 32 MLS points (membrane volume) or six per
-        // force block (rigid force and moment)
-        b.nvol_part = std::max(mls_blocks(tmp, 32), 6 * ((nt + 255) / 256));
-        b.vol_part = upload(c, std::vector<double>((size_t)b.nvol_part, 0.0), &rc);
-        b.vol_sum = upload(c, std::vector<double>(1, 6.0 * V0), &rc);
+        upload(c, std::vector<double>((size_t)std::max(mls_blocks(tmp, 32), 6 * ((nt + 255) / 256)), 0.0), &rc);
+        upload(c, std::vector<double>(1, 6.0 * V0), &rc);
         b.vol_count = upload(c, std::vector<unsigned int>(1, 0u), &rc);
+        // the MLS blocks' partial sums and, behind them, the sums (of the
+        // one-lattice kernel: the batched ones have fewer)
+        b.part = (double *)dev_alloc(c, sizeof(double) * 6 * (size_t)(mls_blocks(tmp, mls_threads(c->prec)) + 1));
+        if (b.part) c->transient.push_back(b.part);
         // per (vertex, hinge) entry: the hinge's vertices and parameters
         std::vector<int4> hv(vh_list.size());
         std::vector<double> hp(4 * vh_list.size());
@@ -951,7 +959,7 @@ int lbib_add_body(void *h, const double *verts, int nv, const int *tris, int nt,
         b.vh_verts = upload(c, hv, &rc);
         b.vh_par = upload_r(c, hp, &rc);
     }
-    if (rc || !b.phi || !b.node || !b.tri_geo || !b.tri_vol || !b.probe) {
+    if (rc || !b.phi || !b.node || !b.tri_geo || !old_terms || !b.probe || !b.part) {
         c->err = rc ? rc : LBIB_ENOMEM;
         return fail(c, c->err, "body allocation or upload failed");
     }
@@ -1006,14 +1014,11 @@ int enqueue_step(Ctx *c, bool store_fields, cudaEvent_t *ev, bool external, int 
     // structure update and spreading
     for (auto &b : c->bodies) {
         const BodyView v = make_view(c, b);
-        cudaError_t e;
-        if (b.rigid) {
-            e = launch_rigid(c->prec, c->L, v, c->force, c->stamp, c->d_step, c->ib_per_sm * c->nsm, hi);
-            c->launches += 2 + v.centroid;
-        } else {
-            e = launch_membrane(c->prec, c->L, v, c->force, c->stamp, c->d_step, c->ib_per_sm * c->nsm, hi);
-            c->launches += 1 + v.centroid;
-        }
+        // programmatically behind the MLS kernel (or the body before), unless
+        // a timing event stands between them
+        const cudaError_t e = launch_structure(c->prec, c->L, v, c->force, c->stamp, c->d_step, c->nsm,
+                                               c->ib_per_sm * c->nsm, !ev, hi);
+        c->launches += structure_launches(c->prec, v);
         if (e != cudaSuccess) return cuda_fail(c, e, "structure kernel");
     }
     rec(2, hi);
@@ -1107,9 +1112,9 @@ int build_graphs(Ctx *c) {
 }
 
 // launches per step (for the counters when a graph runs the step)
-long long launches_per_step(const Ctx *c) {
+long long launches_per_step(Ctx *c) {
     long long n = 1 + (c->bodies.size() == 1 && c->split_sweep ? 1 : 0);
-    for (auto &b : c->bodies) n += 2 + (b.rigid ? 2 : 1);
+    for (auto &b : c->bodies) n += 2 + structure_launches(c->prec, make_view(c, b));
     return n;
 }
 
@@ -1663,7 +1668,7 @@ void batch_free_tables(Batch *b) {
 }
 
 // Work items of the persistent kernel's six-step launch, in queue order.
-// Per body: support-moment, MLS, membrane, rigid-force, rigid-marker and
+// Per body: support-moment, MLS, partial-sum, membrane, rigid-marker and
 // centroid items (each split into the blocks the separate kernels would
 // launch); per lattice: sweep tiles of sweep_cells cells.  Each lattice's
 // chain of phases (its item kinds in order, step after step) is laid out in
@@ -1689,10 +1694,10 @@ int batch_build_persistent(Batch *b, const std::vector<std::pair<int, int>> &bod
         n.fill(0);
         n[kPMom] = std::max(8, d.nv / 16);
         n[kPMls] = mls_blocks(body[q].v, kPersistThreads);
-        n[kPMemb] = d.rigid ? 0 : (d.nv + 7) / 8;
-        n[kPRf] = d.rigid ? (d.nt + 255) / 256 : 0;
-        n[kPRm] = d.rigid ? (d.nv + 7) / 8 : 0;
-        n[kPCen] = d.p.centroid_markers ? (d.nt + 7) / 8 : 0;
+        n[kPSum] = needs_body_sums(body[q].v, kPersistThreads);
+        n[kPMemb] = d.rigid ? 0 : marker_blocks(d.nv);
+        n[kPRm] = d.rigid ? marker_blocks(d.nv) : 0;
+        n[kPCen] = d.p.centroid_markers ? marker_blocks(d.nt) : 0;
         for (int k = kPMom; k < kPSweep; ++k) need[(size_t)bodies[q].first * kPKinds + k] += (unsigned)n[k];
     }
     std::vector<int> tiles(nl);
@@ -1796,7 +1801,7 @@ int batch_build(Batch *b) {
             r.parity = (int)((c->steps + k) & 1);
         }
     }
-    std::vector<int> mom_pre(1, 0), mls_pre(1, 0), memb_id, memb_pre(1, 0), rigid_id, rf_pre(1, 0), rm_pre(1, 0),
+    std::vector<int> mom_pre(1, 0), mls_pre(1, 0), memb_id, memb_pre(1, 0), rigid_id, rm_pre(1, 0), sums_id,
         cen_id, cen_pre(1, 0);
     for (int q = 0; q < nb; ++q) {
         Ctx *c = b->ctx[bodies[q].first];
@@ -1817,16 +1822,16 @@ int batch_build(Batch *b) {
         mls_pre.push_back(mls_pre.back() + mls_blocks(v, kBatchMlsThreads));
         if (d.rigid) {
             rigid_id.push_back(q);
-            rf_pre.push_back(rf_pre.back() + (d.nt + 255) / 256);
-            rm_pre.push_back(rm_pre.back() + (d.nv + 7) / 8);
+            rm_pre.push_back(rm_pre.back() + marker_blocks(d.nv));
         } else {
             memb_id.push_back(q);
-            memb_pre.push_back(memb_pre.back() + (d.nv + 7) / 8);
+            memb_pre.push_back(memb_pre.back() + marker_blocks(d.nv));
         }
         if (d.p.centroid_markers) {
             cen_id.push_back(q);
-            cen_pre.push_back(cen_pre.back() + (d.nt + 7) / 8);
+            cen_pre.push_back(cen_pre.back() + marker_blocks(d.nt));
         }
+        if (needs_body_sums(v, kBatchMlsThreads)) sums_id.push_back(q);
     }
     // sweep slots: lattices in launch order (0: as given, 1: largest first)
     std::vector<int> order(nl);
@@ -1846,7 +1851,7 @@ int batch_build(Batch *b) {
         return blk;
     };
     const std::vector<int> sweep_blk = blocks_of(sweep_pre), mom_blk = blocks_of(mom_pre),
-                           mls_blk = blocks_of(mls_pre), memb_blk = blocks_of(memb_pre), rf_blk = blocks_of(rf_pre),
+                           mls_blk = blocks_of(mls_pre), memb_blk = blocks_of(memb_pre),
                            rm_blk = blocks_of(rm_pre), cen_blk = blocks_of(cen_pre);
     // one device block for all tables
     size_t off = 0;
@@ -1860,10 +1865,10 @@ int batch_build(Batch *b) {
                  o_spre = place(sizeof(int) * sweep_pre.size()), o_mom = place(sizeof(int) * mom_pre.size()),
                  o_mls = place(sizeof(int) * mls_pre.size()), o_mid = place(sizeof(int) * memb_id.size()),
                  o_mpre = place(sizeof(int) * memb_pre.size()), o_rid = place(sizeof(int) * rigid_id.size()),
-                 o_rf = place(sizeof(int) * rf_pre.size()), o_rm = place(sizeof(int) * rm_pre.size()),
+                 o_sum = place(sizeof(int) * sums_id.size()), o_rm = place(sizeof(int) * rm_pre.size()),
                  o_bs = place(sizeof(int) * sweep_blk.size()), o_bmo = place(sizeof(int) * mom_blk.size()),
                  o_bml = place(sizeof(int) * mls_blk.size()), o_bme = place(sizeof(int) * memb_blk.size()),
-                 o_brf = place(sizeof(int) * rf_blk.size()), o_brm = place(sizeof(int) * rm_blk.size()),
+                 o_brm = place(sizeof(int) * rm_blk.size()),
                  o_cid = place(sizeof(int) * cen_id.size()), o_cpre = place(sizeof(int) * cen_pre.size()),
                  o_bce = place(sizeof(int) * cen_blk.size());
     cudaError_t e = cudaMalloc(&b->dmem, off);
@@ -1885,13 +1890,12 @@ int batch_build(Batch *b) {
     put(o_mid, memb_id.data(), sizeof(int) * memb_id.size());
     put(o_mpre, memb_pre.data(), sizeof(int) * memb_pre.size());
     put(o_rid, rigid_id.data(), sizeof(int) * rigid_id.size());
-    put(o_rf, rf_pre.data(), sizeof(int) * rf_pre.size());
+    put(o_sum, sums_id.data(), sizeof(int) * sums_id.size());
     put(o_rm, rm_pre.data(), sizeof(int) * rm_pre.size());
     put(o_bs, sweep_blk.data(), sizeof(int) * sweep_blk.size());
     put(o_bmo, mom_blk.data(), sizeof(int) * mom_blk.size());
     put(o_bml, mls_blk.data(), sizeof(int) * mls_blk.size());
     put(o_bme, memb_blk.data(), sizeof(int) * memb_blk.size());
-    put(o_brf, rf_blk.data(), sizeof(int) * rf_blk.size());
     put(o_brm, rm_blk.data(), sizeof(int) * rm_blk.size());
     put(o_cid, cen_id.data(), sizeof(int) * cen_id.size());
     put(o_cpre, cen_pre.data(), sizeof(int) * cen_pre.size());
@@ -1915,13 +1919,12 @@ int batch_build(Batch *b) {
     T.memb_id = reinterpret_cast<const int *>(d + o_mid);
     T.memb_pre = reinterpret_cast<const int *>(d + o_mpre);
     T.rigid_id = reinterpret_cast<const int *>(d + o_rid);
-    T.rf_pre = reinterpret_cast<const int *>(d + o_rf);
+    T.sums_id = reinterpret_cast<const int *>(d + o_sum);
     T.rm_pre = reinterpret_cast<const int *>(d + o_rm);
     T.sweep_blk = reinterpret_cast<const int *>(d + o_bs);
     T.mom_blk = reinterpret_cast<const int *>(d + o_bmo);
     T.mls_blk = reinterpret_cast<const int *>(d + o_bml);
     T.memb_blk = reinterpret_cast<const int *>(d + o_bme);
-    T.rf_blk = reinterpret_cast<const int *>(d + o_brf);
     T.rm_blk = reinterpret_cast<const int *>(d + o_brm);
     T.cen_id = reinterpret_cast<const int *>(d + o_cid);
     T.cen_pre = reinterpret_cast<const int *>(d + o_cpre);
@@ -1930,7 +1933,7 @@ int batch_build(Batch *b) {
     T.sweep_cpt = b->sweep_cpt;
     T.sweep_off32 = 1;
     for (const Lattice &Li : lat) T.sweep_off32 &= Li.off32;
-    b->G = BatchGrid{sweep_pre.back(), mom_pre.back(), mls_pre.back(), memb_pre.back(), rf_pre.back(), rm_pre.back(),
+    b->G = BatchGrid{sweep_pre.back(), mom_pre.back(), mls_pre.back(), (int)sums_id.size(), memb_pre.back(), rm_pre.back(),
                      cen_pre.back()};
     if (b->persistent) {
         int rc = batch_build_persistent(b, bodies, body, lat, order);
@@ -1970,7 +1973,7 @@ int batch_enqueue(Batch *b, int phase, bool store, cudaStream_t st) {
 
 int batch_launches_per_step(const Batch *b) {
     int n = 0;
-    for (int v : {b->G.mom, b->G.mls, b->G.memb, b->G.rf, b->G.rm, b->G.cen}) n += v > 0;
+    for (int v : {b->G.mom, b->G.mls, b->G.sums, b->G.memb, b->G.rm, b->G.cen}) n += v > 0;
     return n + (b->sweep_split ? (int)b->lat_h.size() : (b->G.sweep > 0));
 }
 

@@ -278,7 +278,6 @@ struct BodyView {
     const int *perm;        // [nm + 2nt] MLS points in cell order (markers, probes), or nullptr
     const int *tri;         // [3nt]
     void *tri_geo;          // [8nt] R: unit normal (3), area, centroid - origin (3), unused
-    double *tri_vol;        // [nt] volume terms (x_0 - o) . (e1 x e2)
     void *probe;            // [8nt] R per side: pressure - 1/3, traction tau.n (3)
     // membrane topology (CSR over vertices)
     const int *vh_ptr;      // [nv+1]
@@ -301,12 +300,15 @@ struct BodyView {
     // support region: node box of level n (read) and of level n+1 (built)
     const int *bbox;        // [6]: lo xyz, hi xyz (inclusive node coordinates)
     int *bbox_next;         // [6], reset by the moments kernel, filled by the update kernel
-    double *vol_part;       // [one per 32 MLS points] partial sums of the volume terms
-    int nvol_part;
-    unsigned int *vol_count; // blocks of the MLS kernel done (reset by the last one)
-    double *vol_sum;        // enclosed volume times 6, written by the last MLS block
+    double *part;           // per MLS block: partial volume (membranes) or force and moment (rigid, 6); then the sums
+    unsigned int *vol_count; // rigid: blocks of the marker kernel that have read the old state
     int *err;               // device error word of the context (first error wins)
 };
+
+// Blocks of `threads` MLS points (markers, then two probes per triangle).
+__host__ __device__ inline int points_blocks(const BodyView &B, int threads) {
+    return (B.nm + 2 * B.nt + threads - 1) / threads;
+}
 
 // Device error codes (the values of include/lbib.h).
 constexpr int kErrDiverged = -4;   // LBIB_EDIVERGED
@@ -350,13 +352,13 @@ struct BatchTables {
     const int *mom_pre;    // [nb + 1] moments blocks
     const int *mls_pre;    // [nb + 1] MLS blocks
     const int *memb_id;    // [nmemb] membrane bodies
-    const int *memb_pre;   // [nmemb + 1] blocks of 8 vertex warps
+    const int *memb_pre;   // [nmemb + 1] blocks of 32 vertices
     const int *rigid_id;   // [nrigid] rigid bodies
-    const int *rf_pre;     // [nrigid + 1] triangle blocks of the force reduction
-    const int *rm_pre;     // [nrigid + 1] blocks of 8 marker warps
+    const int *sums_id;    // [sums blocks] bodies whose MLS partials are added up by a launch of their own
+    const int *rm_pre;     // [nrigid + 1] blocks of 32 markers
     const int *cen_id;     // [ncen] bodies with centroid markers
-    const int *cen_pre;    // [ncen + 1] blocks of 8 triangle warps
-    const int *sweep_blk, *mom_blk, *mls_blk, *memb_blk, *rf_blk, *rm_blk, *cen_blk;  // item of each block
+    const int *cen_pre;    // [ncen + 1] blocks of 32 triangles
+    const int *sweep_blk, *mom_blk, *mls_blk, *memb_blk, *rm_blk, *cen_blk;  // item of each block
     int sweep_threads;     // threads per sweep block
     int sweep_cpt;         // cells per sweep thread (blocks per lattice = cells / (threads * cpt))
     int sweep_off32;       // 1: every lattice of the batch has off32 set
@@ -369,7 +371,7 @@ struct BatchTables {
 // lattice, and the queue holds those earlier: items are taken in ticket
 // order, so whatever an item waits for was taken earlier by a running
 // block, and the queue cannot deadlock.
-enum PKind { kPMom = 0, kPMls, kPMemb, kPRf, kPRm, kPCen, kPSweep, kPKinds };
+enum PKind { kPMom = 0, kPMls, kPSum, kPMemb, kPRm, kPCen, kPSweep, kPKinds };
 struct PersistTables {
     int nitems;              // items of the launch (all its steps)
     int nsteps;              // steps per launch

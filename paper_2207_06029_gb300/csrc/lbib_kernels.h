@@ -55,24 +55,32 @@ cudaError_t launch_fields_out(int prec, const void *fields, const Lattice &L, do
                               cudaStream_t s);
 
 // ib.cu
+// MLS points per block of the one-lattice kernel.  FP64 (prec 0) issues one
+// warp instruction per 16 cycles on a whole SM, so its warps go to as many
+// SMs as possible: a warp a block.
+constexpr int mls_threads(int prec) { return prec == 0 ? 32 : 64; }
 constexpr int kBatchMlsThreads = 128;       // MLS points per block of the batched kernel
 constexpr int kPersistThreads = 256;        // threads per block of the persistent batched kernel
+constexpr int kMarkersPerBlock = 32;        // markers per block of 256 threads (batched structure kernels)
 // blocks of `threads` MLS points (markers and probes) of a body
 int mls_blocks(const BodyView &B, int threads);
+// whether the MLS partials of blocks of `threads` points are added up by a
+// launch of their own
+bool needs_body_sums(const BodyView &B, int threads);
 // step_inc: device step counter incremented at the start of the step (first
 // body only), or nullptr.  grid_cap > 0: the MLS, structure and spreading
 // kernels launch at most grid_cap blocks, each taking its share of their
 // blocks' work in turn (0: their full grids)
 cudaError_t launch_ib_front(int prec, const void *fin, const Lattice &L, const BodyView &B, void *mom, int nsm,
                             int *err, uint32_t *step_inc, int grid_cap, cudaStream_t s);
-cudaError_t launch_membrane(int prec, const Lattice &L, const BodyView &B, void *force, uint32_t *stamp,
-                            const uint32_t *step, int grid_cap, cudaStream_t s);
-cudaError_t launch_rigid(int prec, const Lattice &L, const BodyView &B, void *force, uint32_t *stamp,
-                         const uint32_t *step, int grid_cap, cudaStream_t s);
+// structure update and spreading; chained: programmatically behind the
+// previous kernel of the stream
+cudaError_t launch_structure(int prec, const Lattice &L, const BodyView &B, void *force, uint32_t *stamp,
+                             const uint32_t *step, int nsm, int grid_cap, bool chained, cudaStream_t s);
 
 // batches (sweep.cu and ib.cu); grid sizes are the totals of the prefix tables
 struct BatchGrid {
-    int sweep, mom, mls, memb, rf, rm, cen;
+    int sweep, mom, mls, sums, memb, rm, cen;
 };
 cudaError_t launch_batch_ib(int prec, const BatchTables &T, const BatchGrid &G, int phase, cudaStream_t s);
 cudaError_t launch_batch_sweep(int prec, const BatchTables &T, const BatchGrid &G, int phase, int store_fields,

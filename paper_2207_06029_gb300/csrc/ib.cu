@@ -127,7 +127,7 @@ __device__ __forceinline__ void moments_body(const S *__restrict__ fin, const La
 }
 
 template <typename S, typename R>
-__global__ void __launch_bounds__(256) k_moments(const S *__restrict__ fin, Lattice L, const int *__restrict__ box,
+__global__ void __launch_bounds__(kNodeThreads) k_moments(const S *__restrict__ fin, Lattice L, const int *__restrict__ box,
                                                  int *__restrict__ box_next, R *__restrict__ mom,
                                                  uint32_t *__restrict__ step_inc) {
     chain_release();  // the MLS kernel may be scheduled beside this one
@@ -1502,9 +1502,10 @@ bool needs_body_sums(const BodyView &B, int threads) { return points_blocks(B, t
 static int capped(int n, int cap) { return cap > 0 && cap < n ? cap : n; }
 
 template <typename S, typename R>
-static cudaError_t ib_front_t(const void *fin, const Lattice &L, const BodyView &B, void *mom, int nsm, int *err,
-                              uint32_t *step_inc, int grid_cap, cudaStream_t s) {
-    k_moments<S, R><<<2 * nsm, 256, 0, s>>>((const S *)fin, L, B.bbox, B.bbox_next, (R *)mom, step_inc);
+static cudaError_t ib_front_t(const void *fin, const Lattice &L, const BodyView &B, void *mom, int nsm,
+                              int box_nodes, int *err, uint32_t *step_inc, int grid_cap, cudaStream_t s) {
+    k_moments<S, R><<<node_blocks(box_nodes, kNodeThreads, nsm), kNodeThreads, 0, s>>>(
+        (const S *)fin, L, B.bbox, B.bbox_next, (R *)mom, step_inc);
     cudaError_t e = cudaGetLastError();
     if (e != cudaSuccess) return e;
     // the MLS kernel is scheduled while the moments kernel ends, and forms its
@@ -1516,12 +1517,12 @@ static cudaError_t ib_front_t(const void *fin, const Lattice &L, const BodyView 
 }
 
 cudaError_t launch_ib_front(int prec, const void *fin, const Lattice &L, const BodyView &B, void *mom, int nsm,
-                            int *err, uint32_t *step_inc, int grid_cap, cudaStream_t s) {
+                            int box_nodes, int *err, uint32_t *step_inc, int grid_cap, cudaStream_t s) {
     switch (prec) {
-        case 0: return ib_front_t<double, double>(fin, L, B, mom, nsm, err, step_inc, grid_cap, s);
-        case 1: return ib_front_t<float, float>(fin, L, B, mom, nsm, err, step_inc, grid_cap, s);
-        case 2: return ib_front_t<__half, float>(fin, L, B, mom, nsm, err, step_inc, grid_cap, s);
-        default: return ib_front_t<__nv_bfloat16, float>(fin, L, B, mom, nsm, err, step_inc, grid_cap, s);
+        case 0: return ib_front_t<double, double>(fin, L, B, mom, nsm, box_nodes, err, step_inc, grid_cap, s);
+        case 1: return ib_front_t<float, float>(fin, L, B, mom, nsm, box_nodes, err, step_inc, grid_cap, s);
+        case 2: return ib_front_t<__half, float>(fin, L, B, mom, nsm, box_nodes, err, step_inc, grid_cap, s);
+        default: return ib_front_t<__nv_bfloat16, float>(fin, L, B, mom, nsm, box_nodes, err, step_inc, grid_cap, s);
     }
 }
 

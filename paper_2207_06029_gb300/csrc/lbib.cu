@@ -40,6 +40,7 @@ struct DevBody {
     double *Xbody = nullptr, *rstate = nullptr;
     int *bbox[2] = {nullptr, nullptr};  // support-region node boxes, current and next
     int bcur = 0;
+    int box_nodes = 0;  // about the nodes of the support box (grid sizes)
     double *part = nullptr;  // MLS partial sums (per-step scratch)
     unsigned int *vol_count = nullptr;
     int4 *vh_verts = nullptr;
@@ -75,11 +76,12 @@ struct Ctx {
     double *d_watch = nullptr;   // divergence watchdog: mass of its first check, mass of its last
     int watch_every = 1000;      // watchdog cadence in steps (0: off)
     double watch_tol = 0.1;      // relative total-mass drift the watchdog tolerates
-    // CUDA graphs of one step, one per phase of the buffer rotation (period 6)
+    // CUDA graphs: one step per phase of the buffer rotation (period 6), and
+    // the six steps from phase 0, each captured when first needed
     cudaStream_t s_cap = nullptr;
-    cudaGraphExec_t gexec[6] = {nullptr, nullptr, nullptr, nullptr, nullptr, nullptr};
-    bool graphs_valid = false, use_graphs = true, graphs_timed = false;
-    long long graph_origin = 0;
+    cudaGraphExec_t gexec[6] = {nullptr, nullptr, nullptr, nullptr, nullptr, nullptr}, gexec6 = nullptr;
+    bool use_graphs = true, graphs_timed = false;
+    long long graph_origin = 0;  // the step count at phase 0
     cudaEvent_t gev[6][6] = {};  // timing events recorded by the graphs
     bool gev_pending[6] = {false, false, false, false, false, false};
     double prof_acc[4] = {0.0, 0.0, 0.0, 0.0};
@@ -599,6 +601,7 @@ void lbib_destroy(void *h) {
     for (cudaStream_t st : {c->s_hi, c->s_lo})
         if (st) cudaStreamSynchronize(st);
     for (auto ev : c->events) cudaEventDestroy(ev);
+    if (c->gexec6) cudaGraphExecDestroy(c->gexec6);
     for (int k = 0; k < 6; ++k) {
         if (c->gexec[k]) cudaGraphExecDestroy(c->gexec[k]);
         for (int j = 0; j < 6; ++j)
@@ -932,6 +935,10 @@ int lbib_add_body(void *h, const double *verts, int nv, const int *tris, int nt,
                 box[a] = std::min(box[a], cc - 3);
                 box[3 + a] = std::max(box[3 + a], cc + 4);
             }
+        const int n3[3] = {c->L.nx, c->L.ny, c->L.nz};
+        double nodes = 1.0;
+        for (int a = 0; a < 3; ++a) nodes *= std::min<double>(n3[a], (double)box[3 + a] - box[a] + 1);
+        b.box_nodes = (int)std::min(nodes, 1e9);
         b.bbox[0] = upload(c, box, &rc);
         b.bbox[1] = upload(c, box, &rc);
         BodyView tmp{};
@@ -993,22 +1000,25 @@ int enqueue_step(Ctx *c, bool store_fields, cudaEvent_t *ev, bool external, int 
     void *fields = store_fields ? c->fields : nullptr;
     const int *box = split ? c->bodies[0].bbox[c->bodies[0].bcur] : nullptr;
     uint32_t *stamp = c->bodies.empty() ? nullptr : c->stamp;
-    if (split) {  // far field on the low-priority stream; it never carries IB force
+    // IB front: support-region moments + MLS at markers and probes
+    for (size_t k = 0; k < c->bodies.size(); ++k) {
+        const BodyView v = make_view(c, c->bodies[k]);
+        cudaError_t e = launch_ib_front(c->prec, c->fA, c->L, v, c->mom, c->nsm, c->bodies[k].box_nodes, c->d_err,
+                                        k == 0 ? c->d_step : nullptr, c->ib_per_sm * c->nsm, hi);
+        c->launches += 2;
+        if (e != cudaSuccess) return cuda_fail(c, e, "MLS kernels");
+    }
+    // the far field on the low-priority stream, behind the IB front in launch
+    // order (the chain of short IB kernels is the longer path on all but the
+    // largest lattices); it never carries IB force
+    if (split) {
         rec(4, lo);
         cudaError_t e = launch_sweep(c->prec, c->fA, c->fB, c->force, nullptr, c->d_step, c->L, fields, 1, box,
-                                     c->d_sr, parity, c->nsm, lo);
+                                     c->d_sr, parity, c->nsm, 0, lo);
         c->launches++;
         if (e != cudaSuccess) return cuda_fail(c, e, "sweep kernel (outside the body box)");
         rec(5, lo);
         cudaEventRecord(c->ev_far, lo);
-    }
-    // IB front: support-region moments + MLS at markers and probes
-    for (size_t k = 0; k < c->bodies.size(); ++k) {
-        const BodyView v = make_view(c, c->bodies[k]);
-        cudaError_t e = launch_ib_front(c->prec, c->fA, c->L, v, c->mom, c->nsm, c->d_err,
-                                        k == 0 ? c->d_step : nullptr, c->ib_per_sm * c->nsm, hi);
-        c->launches += 2;
-        if (e != cudaSuccess) return cuda_fail(c, e, "MLS kernels");
     }
     rec(1, hi);
     // structure update and spreading
@@ -1023,7 +1033,7 @@ int enqueue_step(Ctx *c, bool store_fields, cudaEvent_t *ev, bool external, int 
     }
     rec(2, hi);
     cudaError_t e = launch_sweep(c->prec, c->fA, c->fB, c->force, stamp, c->d_step, c->L, fields, split ? 2 : 0,
-                                 box, c->d_sr, parity, c->nsm, hi);
+                                 box, c->d_sr, parity, c->nsm, split ? c->bodies[0].box_nodes : 0, hi);
     c->launches++;
     if (e != cudaSuccess) return cuda_fail(c, e, "sweep kernel");
     rec(3, hi);
@@ -1075,39 +1085,51 @@ void invalidate_graphs(Ctx *c) {
         if (c->gexec[k]) cudaGraphExecDestroy(c->gexec[k]);
         c->gexec[k] = nullptr;
     }
-    c->graphs_valid = false;
+    if (c->gexec6) cudaGraphExecDestroy(c->gexec6);
+    c->gexec6 = nullptr;
+    c->graph_origin = c->steps;
 }
 
-// Captures one step per phase of the buffer rotation (six steps return the
-// rotation to where it started) as CUDA graphs on the capture stream.
-int build_graphs(Ctx *c) {
-    invalidate_graphs(c);
-    for (int k = 0; k < 6; ++k) {
-        cudaError_t e = cudaStreamBeginCapture(c->s_cap, cudaStreamCaptureModeThreadLocal);
-        if (e != cudaSuccess) return cuda_fail(c, e, "graph capture");
-        cudaEventRecord(c->ev_fork, c->s_cap);
-        cudaStreamWaitEvent(c->s_hi, c->ev_fork, 0);
-        cudaStreamWaitEvent(c->s_lo, c->ev_fork, 0);
-        const long long launches = c->launches;
-        int rc = enqueue_step(c, false, c->profile ? c->gev[k] : nullptr, true, (int)((c->steps + k) & 1));
-        c->launches = launches;
-        cudaEventRecord(c->ev_join, c->s_hi);
-        cudaStreamWaitEvent(c->s_cap, c->ev_join, 0);
-        cudaGraph_t g = nullptr;
-        e = cudaStreamEndCapture(c->s_cap, &g);
-        if (rc) {
-            if (g) cudaGraphDestroy(g);
-            return rc;
-        }
-        if (e != cudaSuccess) return cuda_fail(c, e, "graph capture end");
-        // kernel nodes keep the priority of the stream they were captured from
-        e = cudaGraphInstantiateWithFlags(&c->gexec[k], g, cudaGraphInstantiateFlagUseNodePriority);
-        cudaGraphDestroy(g);
-        if (e != cudaSuccess) return cuda_fail(c, e, "graph instantiate");
+// The host side of n steps' buffer rotation.
+void rotate(Ctx *c, int n) {
+    if (n & 1) std::swap(c->fA, c->fB);
+    for (auto &b : c->bodies) {
+        b.cur = (b.cur + n) % 3;
+        b.bcur ^= n & 1;
     }
-    c->graph_origin = c->steps;
-    c->graphs_timed = c->profile;
-    c->graphs_valid = true;
+}
+
+// Captures the next nsteps steps (1 or 6) as a CUDA graph on the capture
+// stream; the host state is left as it was.  k: the phase (timing events).
+int build_graph(Ctx *c, int nsteps, int k, cudaGraphExec_t *out) {
+    cudaError_t e = cudaStreamBeginCapture(c->s_cap, cudaStreamCaptureModeThreadLocal);
+    if (e != cudaSuccess) return cuda_fail(c, e, "graph capture");
+    cudaEventRecord(c->ev_fork, c->s_cap);
+    cudaStreamWaitEvent(c->s_hi, c->ev_fork, 0);
+    cudaStreamWaitEvent(c->s_lo, c->ev_fork, 0);
+    const long long launches = c->launches;
+    int rc = LBIB_OK, done = 0;
+    for (; done < nsteps && rc == LBIB_OK; ++done)
+        rc = enqueue_step(c, false, c->profile ? c->gev[k] : nullptr, true, (int)((c->steps + done) & 1));
+    if (rc) --done;                      // a failed step has not rotated
+    rotate(c, (6 - done % 6) % 6);       // six steps return the rotation to where it started
+    c->launches = launches;
+    cudaEventRecord(c->ev_join, c->s_hi);
+    cudaStreamWaitEvent(c->s_cap, c->ev_join, 0);
+    cudaGraph_t g = nullptr;
+    e = cudaStreamEndCapture(c->s_cap, &g);
+    if (rc) {
+        if (g) cudaGraphDestroy(g);
+        return rc;
+    }
+    if (e != cudaSuccess) return cuda_fail(c, e, "graph capture end");
+    // kernel nodes keep the priority of the stream they were captured from
+    e = cudaGraphInstantiateWithFlags(out, g, cudaGraphInstantiateFlagUseNodePriority);
+    cudaGraphDestroy(g);
+    if (e != cudaSuccess) {
+        *out = nullptr;
+        return cuda_fail(c, e, "graph instantiate");
+    }
     return LBIB_OK;
 }
 
@@ -1115,6 +1137,22 @@ int build_graphs(Ctx *c) {
 long long launches_per_step(Ctx *c) {
     long long n = 1 + (c->bodies.size() == 1 && c->split_sweep ? 1 : 0);
     for (auto &b : c->bodies) n += 2 + structure_launches(c->prec, make_view(c, b));
+    return n;
+}
+
+// How many of the next n steps of a call, from the one about to be taken (its
+// step count is c->steps + 1, and step_host is already its own), follow one
+// another with nothing but steps between them: no stored fields, no watchdog
+// check before the last, no restart of the step counter.
+int plain_steps(const Ctx *c, int n, bool end_of_call) {
+    if (c->fields_every == 0 && end_of_call) --n;
+    n = std::min(n, 6);
+    for (int j = 0; j < n; ++j) {
+        const long long s = c->steps + 1 + j;
+        if (c->fields_every > 0 && s % c->fields_every == 0) return j;
+        if (j > 0 && c->watch_every > 0 && (s - 1) % c->watch_every == 0) return j;
+        if (!c->bodies.empty() && (uint64_t)c->step_host + (uint64_t)j >= 0xFFFFFFFEull) return j;
+    }
     return n;
 }
 
@@ -1139,22 +1177,33 @@ int step_steps(Ctx *c, int nsteps, bool end_of_call) {
         const bool store = c->fields_every == 0 ? (end_of_call && it == nsteps - 1)
                                                 : (c->fields_every > 0 && (c->steps + 1) % c->fields_every == 0);
         if (c->use_graphs && !store) {
-            if (!c->graphs_valid || c->graphs_timed != c->profile) {
-                int rc = build_graphs(c);
-                if (rc) return rc;
+            if (c->graphs_timed != c->profile) {
+                invalidate_graphs(c);
+                c->graphs_timed = c->profile;
             }
             const int k = (int)(((c->steps - c->graph_origin) % 6 + 6) % 6);
+            // six steps at once where none of them stores the fields, is
+            // timed, restarts the step counter or (but for the last) precedes
+            // a watchdog check: the gap between two graph launches (4 to 5 us)
+            // is paid once for the six
+            const bool six = k == 0 && !c->profile && plain_steps(c, nsteps - it, end_of_call) >= 6;
+            cudaGraphExec_t *g = six ? &c->gexec6 : &c->gexec[k];
+            if (!*g) {
+                int rc = build_graph(c, six ? 6 : 1, k, g);
+                if (rc) return rc;
+            }
             harvest_graph_events(c, k);
-            cudaError_t e = cudaGraphLaunch(c->gexec[k], c->stream);
+            cudaError_t e = cudaGraphLaunch(*g, c->stream);
             if (e != cudaSuccess) return cuda_fail(c, e, "graph launch");
             if (c->profile) c->gev_pending[k] = true;
-            // the graph performs the buffer rotation of its step: mirror it
-            std::swap(c->fA, c->fB);
-            for (auto &b : c->bodies) {
-                b.cur = (b.cur + 1) % 3;
-                b.bcur ^= 1;
+            if (six) {
+                if (!c->bodies.empty()) c->step_host += 5;
+                c->steps += 5;
+                it += 5;
+            } else {
+                rotate(c, 1);  // mirror the graph's buffer rotation
             }
-            c->launches += launches_per_step(c);
+            c->launches += (six ? 6 : 1) * launches_per_step(c);
         } else {
             cudaEvent_t *ev = nullptr;
             if (c->profile) {
@@ -1960,7 +2009,7 @@ int batch_enqueue(Batch *b, int phase, bool store, cudaStream_t st) {
             const int i = b->order_h[q];
             const LatRef &r = b->ref_h[(size_t)phase * nl + i];
             e = launch_sweep(b->prec, r.fin, r.fout, r.force, r.stamp, r.d_step, b->lat_h[i], store ? r.fields : nullptr,
-                             0, nullptr, r.sr, r.parity, b->nsm, b->side[q % ns]);
+                             0, nullptr, r.sr, r.parity, b->nsm, 0, b->side[q % ns]);
         }
         for (int k = 0; k < ns && e == cudaSuccess; ++k) {
             e = cudaEventRecord(b->side_ev[1 + k], b->side[k]);
@@ -2007,11 +2056,7 @@ int batch_capture6(Batch *b) {
 // The contexts' host-side state after n batch steps.
 void batch_advance_contexts(Batch *b, int n) {
     for (Ctx *c : b->ctx) {
-        if (n % 2) std::swap(c->fA, c->fB);
-        for (auto &d : c->bodies) {
-            d.cur = (d.cur + n) % 3;
-            d.bcur ^= (n & 1);
-        }
+        rotate(c, n);
         c->steps += n;
         if (!c->bodies.empty()) c->step_host += (uint32_t)n;
     }

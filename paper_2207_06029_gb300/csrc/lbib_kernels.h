@@ -28,13 +28,25 @@ inline cudaError_t launch_chained(void (*kernel)(KArgs...), dim3 grid, dim3 bloc
     return cudaLaunchKernelEx(&cfg, kernel, args...);
 }
 
+constexpr int kNodeThreads = 64;            // threads per block of the support-box kernels (spread over the SMs)
+// MLS points per block of the one-lattice kernel.  FP64 (prec 0) issues one
+// warp instruction per 16 cycles on a whole SM, so its warps go to as many
+// SMs as possible: a warp a block.
+constexpr int mls_threads(int prec) { return prec == 0 ? 32 : 64; }
+
 // sweep.cu
 // part: 0 the whole lattice, 1 the nodes outside box, 2 the nodes inside box
 // stamp == nullptr: no IB force is read; step points to the device step counter
-// sr: the lattice's two-word rounding-seed counter, parity: the step's parity
+// sr: the lattice's two-word rounding-seed counter, parity: the step's parity;
+// box_nodes: about the nodes of the box (part 2)
 cudaError_t launch_sweep(int prec, const void *fin, void *fout, void *force, const uint32_t *stamp,
                          const uint32_t *step, const Lattice &L, void *fields, int part, const int *box,
-                         uint32_t *sr, int parity, int nsm, cudaStream_t s);
+                         uint32_t *sr, int parity, int nsm, int box_nodes, cudaStream_t s);
+// blocks of `threads` for a grid-stride loop over about `nodes` nodes
+inline int node_blocks(int nodes, int threads, int nsm) {
+    const long long g = ((long long)nodes + threads - 1) / threads;
+    return (int)(g < 1 ? 1 : g > 8LL * nsm ? 8LL * nsm : g);
+}
 cudaError_t prepare_sweep_kernels();
 // global mass and momentum (FP64): part holds totals_scratch_doubles() doubles,
 // count one word that starts (and is left) at zero, out 4 doubles
@@ -55,10 +67,6 @@ cudaError_t launch_fields_out(int prec, const void *fields, const Lattice &L, do
                               cudaStream_t s);
 
 // ib.cu
-// MLS points per block of the one-lattice kernel.  FP64 (prec 0) issues one
-// warp instruction per 16 cycles on a whole SM, so its warps go to as many
-// SMs as possible: a warp a block.
-constexpr int mls_threads(int prec) { return prec == 0 ? 32 : 64; }
 constexpr int kBatchMlsThreads = 128;       // MLS points per block of the batched kernel
 constexpr int kPersistThreads = 256;        // threads per block of the persistent batched kernel
 constexpr int kMarkersPerBlock = 32;        // markers per block of 256 threads (batched structure kernels)
@@ -72,7 +80,7 @@ bool needs_body_sums(const BodyView &B, int threads);
 // kernels launch at most grid_cap blocks, each taking its share of their
 // blocks' work in turn (0: their full grids)
 cudaError_t launch_ib_front(int prec, const void *fin, const Lattice &L, const BodyView &B, void *mom, int nsm,
-                            int *err, uint32_t *step_inc, int grid_cap, cudaStream_t s);
+                            int box_nodes, int *err, uint32_t *step_inc, int grid_cap, cudaStream_t s);
 // structure update and spreading; chained: programmatically behind the
 // previous kernel of the stream
 cudaError_t launch_structure(int prec, const Lattice &L, const BodyView &B, void *force, uint32_t *stamp,

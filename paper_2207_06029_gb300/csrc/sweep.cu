@@ -212,7 +212,7 @@ __global__ void __launch_bounds__(512) k_sweep_tile(const S *__restrict__ fin, S
 
 // The nodes inside the box (grid-stride; periodic coordinates wrap).
 template <typename S, typename R, bool kOff32>
-__global__ void __launch_bounds__(256) k_sweep_box(const S *__restrict__ fin, S *__restrict__ fout,
+__global__ void __launch_bounds__(kNodeThreads) k_sweep_box(const S *__restrict__ fin, S *__restrict__ fout,
                                                    R *__restrict__ force, const uint32_t *__restrict__ stamp,
                                                    const uint32_t *__restrict__ dstep, Lattice L,
                                                    R *__restrict__ fields, const int *__restrict__ box,
@@ -359,10 +359,10 @@ static void sweep_shape(const Lattice &L, dim3 &grid, dim3 &block) {
 template <typename S, typename R, bool kOff32>
 static cudaError_t sweep_t(const void *fin, void *fout, void *force, const uint32_t *stamp, const uint32_t *step,
                            const Lattice &L, void *fields, int part, const int *box, uint32_t *sr, int parity,
-                           int nsm, cudaStream_t s) {
+                           int nsm, int box_nodes, cudaStream_t s) {
     if (part == 2) {
-        k_sweep_box<S, R, kOff32><<<4 * nsm, 256, 0, s>>>((const S *)fin, (S *)fout, (R *)force, stamp, step, L,
-                                                  (R *)fields, box, sr, parity);
+        k_sweep_box<S, R, kOff32><<<node_blocks(box_nodes, kNodeThreads, nsm), kNodeThreads, 0, s>>>(
+            (const S *)fin, (S *)fout, (R *)force, stamp, step, L, (R *)fields, box, sr, parity);
     } else if (const int rows = tile_rows<S>(L)) {
         const dim3 grid((L.ny + rows - 1) / rows, L.nz);
         const size_t smem = (size_t)Q * rows * L.nx * sizeof(S);
@@ -387,22 +387,22 @@ static cudaError_t sweep_t(const void *fin, void *fout, void *force, const uint3
 template <typename S, typename R>
 static cudaError_t sweep_any(const void *fin, void *fout, void *force, const uint32_t *stamp, const uint32_t *step,
                              const Lattice &L, void *fields, int part, const int *box, uint32_t *sr, int parity,
-                             int nsm, cudaStream_t s) {
+                             int nsm, int box_nodes, cudaStream_t s) {
     if (L.off32)
-        return sweep_t<S, R, true>(fin, fout, force, stamp, step, L, fields, part, box, sr, parity, nsm, s);
-    return sweep_t<S, R, false>(fin, fout, force, stamp, step, L, fields, part, box, sr, parity, nsm, s);
+        return sweep_t<S, R, true>(fin, fout, force, stamp, step, L, fields, part, box, sr, parity, nsm, box_nodes, s);
+    return sweep_t<S, R, false>(fin, fout, force, stamp, step, L, fields, part, box, sr, parity, nsm, box_nodes, s);
 }
 
 cudaError_t launch_sweep(int prec, const void *fin, void *fout, void *force, const uint32_t *stamp,
                          const uint32_t *step, const Lattice &L, void *fields, int part, const int *box,
-                         uint32_t *sr, int parity, int nsm, cudaStream_t s) {
+                         uint32_t *sr, int parity, int nsm, int box_nodes, cudaStream_t s) {
     switch (prec) {
-        case 0: return sweep_any<double, double>(fin, fout, force, stamp, step, L, fields, part, box, sr, parity, nsm, s);
-        case 1: return sweep_any<float, float>(fin, fout, force, stamp, step, L, fields, part, box, sr, parity, nsm, s);
-        case 2: return sweep_any<__half, float>(fin, fout, force, stamp, step, L, fields, part, box, sr, parity, nsm, s);
+        case 0: return sweep_any<double, double>(fin, fout, force, stamp, step, L, fields, part, box, sr, parity, nsm, box_nodes, s);
+        case 1: return sweep_any<float, float>(fin, fout, force, stamp, step, L, fields, part, box, sr, parity, nsm, box_nodes, s);
+        case 2: return sweep_any<__half, float>(fin, fout, force, stamp, step, L, fields, part, box, sr, parity, nsm, box_nodes, s);
         default:
             return sweep_any<__nv_bfloat16, float>(fin, fout, force, stamp, step, L, fields, part, box, sr, parity,
-                                                   nsm, s);
+                                                   nsm, box_nodes, s);
     }
 }
 

@@ -171,7 +171,9 @@ __global__ void __launch_bounds__(512) k_sweep_tile(const S *__restrict__ fin, S
         }
         const long long idx = x + (long long)y * nx + (long long)z * nxy;
         R rho, ux, uy, uz;
-        collide_node<R, Pop<S, R>::kScaleLog2>(g, force, stamp, step, L, x, y, z, idx, rho, ux, uy, uz);
+        R fib[3];
+        fetch_force(force, stamp && tile_flag<false>(stamp, L, x, y, z) == step, st, idx, fib);
+        collide_node<R, Pop<S, R>::kScaleLog2>(g, fib, L, x, y, z, rho, ux, uy, uz);
         if (fields) {
             fields[idx] = rho;
             fields[st + idx] = ux;

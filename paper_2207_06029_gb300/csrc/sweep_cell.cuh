@@ -79,6 +79,33 @@ __device__ __forceinline__ void wall_corner(R (&g)[Q], unsigned unknown, const R
     }
 }
 
+// The step that last flagged the tile of node (x, y, z).
+template <bool kCG>
+__device__ __forceinline__ uint32_t tile_flag(const uint32_t *stamp, const Lattice &L, int x, int y, int z) {
+    return ld_ro<kCG>(stamp + ((x >> 3) + L.ntx * ((y >> 3) + L.nty * (z >> 3))));
+}
+
+// Consumes the IB force of a node in a flagged tile (flag == step).  The
+// callers load the flag before and fetch the force right behind the node's
+// population loads, so that the latencies run side by side.  Zeros are
+// written only over forces: most nodes of a flagged tile carry none, and
+// reading and rewriting all of them cost a third of the sweep (64 capsule
+// lattices in one launch, 36 M nodes: 1.55 ms a step so, 1.15 now, 1.12 with
+// the force left out; rewriting without reading, or reading without
+// rewriting, 1.14 and 1.16).
+template <typename R>
+__device__ __forceinline__ void fetch_force(R *__restrict__ force, bool flagged, long long st, long long idx,
+                                            R (&fib)[3]) {
+    fib[0] = fib[1] = fib[2] = R(0);
+    if (flagged) {
+#pragma unroll
+        for (int a = 0; a < 3; ++a) fib[a] = force[a * st + idx];
+        if (fib[0] != R(0) || fib[1] != R(0) || fib[2] != R(0))
+#pragma unroll
+            for (int a = 0; a < 3; ++a) force[a * st + idx] = R(0);
+    }
+}
+
 // Walls, moments, body force and BGK/Guo collision of node (x, y, z) whose
 // streamed populations are g (Eqs. evoleq, eqfunc, forcing; Zou-He walls);
 // on return g holds the post-collision populations and rho, u the moments
@@ -87,13 +114,12 @@ __device__ __forceinline__ void wall_corner(R (&g)[Q], unsigned unknown, const R
 // scaling by a power of two commutes with every rounding, so the update runs
 // on the scaled values (the four moments and the equilibrium weights carry
 // the factor) and gives exactly the scaled result.
-template <typename R, int kLog2S = 0, bool kCG = false>
-__device__ __forceinline__ void collide_node(R (&g)[Q], R *__restrict__ force, const uint32_t *__restrict__ stamp,
-                                             uint32_t step, const Lattice &L, int x, int y, int z, long long idx,
+// fib: the node's IB force (fetch_force).
+template <typename R, int kLog2S = 0>
+__device__ __forceinline__ void collide_node(R (&g)[Q], const R (&fib)[3], const Lattice &L, int x, int y, int z,
                                              R &rho_o, R &ux_o, R &uy_o, R &uz_o) {
     constexpr R kS = R(1 << kLog2S), kInvS = R(1) / R(1 << kLog2S);  // exact powers of two
     const int nx = L.nx, ny = L.ny, nz = L.nz;
-    const long long st = L.stride;
     // walls (faces -x,+x,-y,+y,-z,+z; the index-0 face has inward normal +)
     int nf = 0, fa = 0, fs = 0, code[3] = {0, 0, 0};
     unsigned unknown = 0;
@@ -156,25 +182,12 @@ __device__ __forceinline__ void collide_node(R (&g)[Q], R *__restrict__ force, c
     }
     const R rho = R(1) + dr;
 
-    // body force f_lb = g_ext + f_ib (none on wall nodes); consume the IB
-    // force of flagged tiles
+    // body force f_lb = g_ext + f_ib (none on wall nodes)
     R F0 = R(0), F1 = R(0), F2 = R(0);
     if (nf == 0) {
-        F0 = pick<R>(L.gext_d[0], L.gext_f[0]);
-        F1 = pick<R>(L.gext_d[1], L.gext_f[1]);
-        F2 = pick<R>(L.gext_d[2], L.gext_f[2]);
-    }
-    const int tile = (x >> 3) + L.ntx * ((y >> 3) + L.nty * (z >> 3));
-    if (stamp && ld_ro<kCG>(stamp + tile) == step) {
-        const R fx = force[idx], fy = force[st + idx], fz = force[2 * st + idx];
-        force[idx] = R(0);
-        force[st + idx] = R(0);
-        force[2 * st + idx] = R(0);
-        if (nf == 0) {
-            F0 += fx;
-            F1 += fy;
-            F2 += fz;
-        }
+        F0 = pick<R>(L.gext_d[0], L.gext_f[0]) + fib[0];
+        F1 = pick<R>(L.gext_d[1], L.gext_f[1]) + fib[1];
+        F2 = pick<R>(L.gext_d[2], L.gext_f[2]) + fib[2];
     }
 
     // BGK collision with the Guo term, u = (sum f e + f_lb/2)/rho = j'/rho.
@@ -281,23 +294,29 @@ __device__ __forceinline__ void sweep_cell(const S *__restrict__ fin, S *__restr
     if (yp >= ny) yp = py ? 0 : ny - 1;
     if (zm < 0) zm = pz ? nz - 1 : 0;
     if (zp >= nz) zp = pz ? 0 : nz - 1;
+    const uint32_t flag = stamp ? tile_flag<kCG>(stamp, L, x, y, z) : 0u;
     const int nxy = nx * ny;
     const int oy_m = ym * nx, oy_0 = y * nx, oy_p = yp * nx;
     const int oz_m = zm * nxy, oz_0 = z * nxy, oz_p = zp * nxy;
     const long long st = L.stride;
 
     // pull: f_i(x) = f*_i(x - e_i)
-    R g[Q];
+    S raw[Q];
 #pragma unroll
     for (int i = 0; i < Q; ++i) {
         const int sx = ex(i) > 0 ? xm : ex(i) < 0 ? xp : x;
         const int sy = ey(i) > 0 ? oy_m : ey(i) < 0 ? oy_p : oy_0;
         const int sz = ez(i) > 0 ? oz_m : ez(i) < 0 ? oz_p : oz_0;
-        g[i] = Pop<S, R>::from_raw(ld_ro<kCG>(plane_ptr<kOff32>(fin, L, i, sx + sy + sz)));
+        raw[i] = ld_ro<kCG>(plane_ptr<kOff32>(fin, L, i, sx + sy + sz));
     }
+    R fib[3];
+    fetch_force(force, stamp && flag == step, st, idx, fib);
+    R g[Q];
+#pragma unroll
+    for (int i = 0; i < Q; ++i) g[i] = Pop<S, R>::from_raw(raw[i]);
 
     R rho, ux, uy, uz;
-    collide_node<R, Pop<S, R>::kScaleLog2, kCG>(g, force, stamp, step, L, x, y, z, idx, rho, ux, uy, uz);
+    collide_node<R, Pop<S, R>::kScaleLog2>(g, fib, L, x, y, z, rho, ux, uy, uz);
     // bfloat16 storage rounds stochastically (8-bit mantissa: nearest
     // rounding of a smooth flow repeats the same error at every node of a
     // plane and step, a bias); the other formats round to nearest

@@ -45,8 +45,14 @@ struct DevBody {
     unsigned int *vol_count = nullptr;
     int4 *vh_verts = nullptr;
     void *vh_par = nullptr;
+    std::vector<int> tri_h;  // host copy of tri (lbib_get_body)
     double V0 = 0, A0 = 0, mv = 0, origin[3] = {0, 0, 0};
 };
+
+// Size of a context's page-locked block: allocating one takes about 115 us
+// whatever its size up to 1 MiB, which holds the markers of a body of 14 500
+// vertices.
+constexpr size_t kPinBytes = 1 << 20, kPinHead = 64;
 
 struct Ctx {
     lbib_params p{};
@@ -59,6 +65,9 @@ struct Ctx {
     uint32_t *stamp = nullptr;
     int ntiles = 0;
     int *d_err = nullptr;
+    // page-locked host block: the error word read back (h_err, its first
+    // word) and, from kPinHead on, the markers and state of one body
+    unsigned char *h_pin = nullptr;
     int *h_err = nullptr;
     double *scratch = nullptr;
     size_t scratch_bytes = 0;
@@ -80,6 +89,10 @@ struct Ctx {
     // the six steps from phase 0, each captured when first needed
     cudaStream_t s_cap = nullptr;
     cudaGraphExec_t gexec[6] = {nullptr, nullptr, nullptr, nullptr, nullptr, nullptr}, gexec6 = nullptr;
+    // a step that stores the fields, per phase: enqueued kernel by kernel the
+    // first time, captured when the phase comes to store again
+    cudaGraphExec_t gstore[6] = {nullptr, nullptr, nullptr, nullptr, nullptr, nullptr};
+    bool stored[6] = {false, false, false, false, false, false};
     bool use_graphs = true, graphs_timed = false;
     long long graph_origin = 0;  // the step count at phase 0
     cudaEvent_t gev[6][6] = {};  // timing events recorded by the graphs
@@ -557,13 +570,14 @@ int lbib_create(const lbib_params *p, void **out) {
         lbib_destroy(c);
         return LBIB_ENOMEM;
     }
-    if (cudaMallocHost(&c->h_err, sizeof(int)) != cudaSuccess) {
+    if (cudaMallocHost(&c->h_pin, kPinBytes) != cudaSuccess) {
         cudaGetLastError();
         g_create_error = "pinned host allocation failed";
-        c->h_err = nullptr;
+        c->h_pin = nullptr;
         lbib_destroy(c);
         return LBIB_ENOMEM;
     }
+    c->h_err = reinterpret_cast<int *>(c->h_pin);
     *c->h_err = 0;
     e = cudaMemsetAsync(c->force, 0, 3 * (size_t)L.stride * c->relem, c->stream);
     if (e == cudaSuccess) e = cudaMemsetAsync(c->stamp, 0, sizeof(uint32_t) * (size_t)c->ntiles, c->stream);
@@ -604,6 +618,7 @@ void lbib_destroy(void *h) {
     if (c->gexec6) cudaGraphExecDestroy(c->gexec6);
     for (int k = 0; k < 6; ++k) {
         if (c->gexec[k]) cudaGraphExecDestroy(c->gexec[k]);
+        if (c->gstore[k]) cudaGraphExecDestroy(c->gstore[k]);
         for (int j = 0; j < 6; ++j)
             if (c->gev[k][j]) cudaEventDestroy(c->gev[k][j]);
     }
@@ -613,7 +628,7 @@ void lbib_destroy(void *h) {
     for (cudaStream_t st : {c->s_hi, c->s_lo})
         if (st) cudaStreamDestroy(st);
     dev_free_all(c);
-    if (c->h_err) cudaFreeHost(c->h_err);
+    if (c->h_pin) cudaFreeHost(c->h_pin);
     if (c->own_stream && c->stream) cudaStreamDestroy(c->stream);
     delete c;
 }
@@ -973,7 +988,8 @@ int lbib_add_body(void *h, const double *verts, int nv, const int *tris, int nt,
     cudaError_t e = cudaStreamSynchronize(c->stream);  // host vectors are released on return
     if (e != cudaSuccess) return cuda_fail(c, e, "add_body upload");
     invalidate_graphs(c);
-    c->bodies.push_back(b);
+    b.tri_h = std::move(T);
+    c->bodies.push_back(std::move(b));
     if (body_id) *body_id = (int)c->bodies.size() - 1;
     return LBIB_OK;
 }
@@ -1083,7 +1099,9 @@ void invalidate_graphs(Ctx *c) {
     for (int k = 0; k < 6; ++k) {
         harvest_graph_events(c, k);
         if (c->gexec[k]) cudaGraphExecDestroy(c->gexec[k]);
-        c->gexec[k] = nullptr;
+        if (c->gstore[k]) cudaGraphExecDestroy(c->gstore[k]);
+        c->gexec[k] = c->gstore[k] = nullptr;
+        c->stored[k] = false;
     }
     if (c->gexec6) cudaGraphExecDestroy(c->gexec6);
     c->gexec6 = nullptr;
@@ -1100,8 +1118,9 @@ void rotate(Ctx *c, int n) {
 }
 
 // Captures the next nsteps steps (1 or 6) as a CUDA graph on the capture
-// stream; the host state is left as it was.  k: the phase (timing events).
-int build_graph(Ctx *c, int nsteps, int k, cudaGraphExec_t *out) {
+// stream; the host state is left as it was.  store: the step stores the
+// fields; k: the phase (timing events).
+int build_graph(Ctx *c, int nsteps, bool store, int k, cudaGraphExec_t *out) {
     cudaError_t e = cudaStreamBeginCapture(c->s_cap, cudaStreamCaptureModeThreadLocal);
     if (e != cudaSuccess) return cuda_fail(c, e, "graph capture");
     cudaEventRecord(c->ev_fork, c->s_cap);
@@ -1110,7 +1129,7 @@ int build_graph(Ctx *c, int nsteps, int k, cudaGraphExec_t *out) {
     const long long launches = c->launches;
     int rc = LBIB_OK, done = 0;
     for (; done < nsteps && rc == LBIB_OK; ++done)
-        rc = enqueue_step(c, false, c->profile ? c->gev[k] : nullptr, true, (int)((c->steps + done) & 1));
+        rc = enqueue_step(c, store, c->profile ? c->gev[k] : nullptr, true, (int)((c->steps + done) & 1));
     if (rc) --done;                      // a failed step has not rotated
     rotate(c, (6 - done % 6) % 6);       // six steps return the rotation to where it started
     c->launches = launches;
@@ -1176,20 +1195,20 @@ int step_steps(Ctx *c, int nsteps, bool end_of_call) {
         }
         const bool store = c->fields_every == 0 ? (end_of_call && it == nsteps - 1)
                                                 : (c->fields_every > 0 && (c->steps + 1) % c->fields_every == 0);
-        if (c->use_graphs && !store) {
-            if (c->graphs_timed != c->profile) {
-                invalidate_graphs(c);
-                c->graphs_timed = c->profile;
-            }
-            const int k = (int)(((c->steps - c->graph_origin) % 6 + 6) % 6);
+        if (c->use_graphs && c->graphs_timed != c->profile) {
+            invalidate_graphs(c);
+            c->graphs_timed = c->profile;
+        }
+        const int k = (int)(((c->steps - c->graph_origin) % 6 + 6) % 6);
+        if (c->use_graphs && (!store || (c->stored[k] && !c->profile))) {
             // six steps at once where none of them stores the fields, is
             // timed, restarts the step counter or (but for the last) precedes
             // a watchdog check: the gap between two graph launches (4 to 5 us)
             // is paid once for the six
-            const bool six = k == 0 && !c->profile && plain_steps(c, nsteps - it, end_of_call) >= 6;
-            cudaGraphExec_t *g = six ? &c->gexec6 : &c->gexec[k];
+            const bool six = k == 0 && !store && !c->profile && plain_steps(c, nsteps - it, end_of_call) >= 6;
+            cudaGraphExec_t *g = six ? &c->gexec6 : store ? &c->gstore[k] : &c->gexec[k];
             if (!*g) {
-                int rc = build_graph(c, six ? 6 : 1, k, g);
+                int rc = build_graph(c, six ? 6 : 1, store, k, g);
                 if (rc) return rc;
             }
             harvest_graph_events(c, k);
@@ -1221,6 +1240,7 @@ int step_steps(Ctx *c, int nsteps, bool end_of_call) {
             cudaStreamWaitEvent(c->s_lo, c->ev_fork, 0);
             int rc = enqueue_step(c, store, ev, false, (int)(c->steps & 1));
             if (rc) return rc;
+            if (store && c->use_graphs) c->stored[k] = true;
             cudaEventRecord(c->ev_join, c->s_hi);
             cudaStreamWaitEvent(c->stream, c->ev_join, 0);
         }
@@ -1266,8 +1286,7 @@ int lbib_sync(void *h) {
 int lbib_get_fields(void *h, double *rho, double *u, int on_device) {
     Ctx *c = as_ctx(h);
     if (!c) return LBIB_EINVAL;
-    int rc = sync_ctx(c);
-    if (rc && !readable_error(rc)) return rc;
+    if (c->err && !readable_error(c->err)) return c->err;
     const size_t n = (size_t)c->L.ncell;
     double *drho = rho, *du = u;
     if (!on_device) {
@@ -1276,7 +1295,9 @@ int lbib_get_fields(void *h, double *rho, double *u, int on_device) {
         drho = rho ? tmp : nullptr;
         du = u ? tmp + n : nullptr;
     }
-    cudaError_t e = launch_fields_out(c->prec, c->fields, c->L, drho, du, c->stream);
+    // the kernel behind the queued steps also brings the error word: one
+    // synchronisation for both
+    cudaError_t e = launch_fields_out(c->prec, c->fields, c->L, drho, du, c->d_err, c->h_err, c->stream);
     c->launches++;
     if (e != cudaSuccess) return cuda_fail(c, e, "fields kernel");
     if (!on_device) {
@@ -1286,7 +1307,7 @@ int lbib_get_fields(void *h, double *rho, double *u, int on_device) {
     }
     e = cudaStreamSynchronize(c->stream);
     if (e != cudaSuccess) return cuda_fail(c, e, "fields sync");
-    return rc;
+    return check_device_error(c);
 }
 
 int lbib_get_totals(void *h, double *out) {
@@ -1400,26 +1421,112 @@ int lbib_step_markers(void *h, int nsteps, int body, double *X, double *V, doubl
     return LBIB_OK;
 }
 
+// The markers (and a rigid body's state) and the error word into the
+// context's page-locked block, behind the work already queued.
+__global__ void k_read_back(const double *__restrict__ X, const double *__restrict__ Ub,
+                            const double *__restrict__ Fl, const double *__restrict__ state, const int *err, int n3,
+                            double *__restrict__ out, int *__restrict__ err_out) {
+    const int i0 = blockIdx.x * blockDim.x + threadIdx.x, stride = gridDim.x * blockDim.x;
+    if (i0 == 0) *err_out = *err;
+    for (int i = i0; i < n3; i += stride) {
+        if (X) out[i] = X[i];
+        if (Ub) out[n3 + i] = Ub[i];
+        if (Fl) out[2 * n3 + i] = Fl[i];
+    }
+    if (state)
+        for (int i = i0; i < RigidState::SIZE; i += stride) out[3 * n3 + i] = state[i];
+}
+
+}  // extern "C"
+
+namespace {
+
+// X, U_b and F_l of a body (the wanted ones; device order x, y, z per vertex)
+// and, for a rigid body, its state: pointers into the page-locked block after
+// a synchronisation, or null if the body is too large for it.  One kernel
+// and one synchronisation instead of a staged copy per array.
+double *read_back(Ctx *c, const DevBody &b, bool X, bool V, bool F, bool state, int *rc) {
+    const size_t n3 = 3 * (size_t)b.nv;
+    *rc = LBIB_OK;
+    if (kPinHead + (3 * n3 + RigidState::SIZE) * sizeof(double) > kPinBytes) return nullptr;
+    double *out = reinterpret_cast<double *>(c->h_pin + kPinHead);
+    k_read_back<<<(unsigned)std::min<size_t>((n3 + 255) / 256, 64), 256, 0, c->stream>>>(
+        X ? b.X[b.cur] : nullptr, V ? b.Ub : nullptr, F ? b.Fl : nullptr, state && b.rigid ? b.rstate : nullptr, c->d_err,
+        (int)n3, out, c->h_err);
+    c->launches++;
+    cudaError_t e = cudaGetLastError();
+    if (e == cudaSuccess) e = cudaStreamSynchronize(c->stream);
+    *rc = e == cudaSuccess ? check_device_error(c) : cuda_fail(c, e, "markers read-back");
+    return out;
+}
+
+// Whether p may be written by the host (not device memory).
+bool host_pointer(const void *p) {
+    if (!p) return true;
+    cudaPointerAttributes at{};
+    if (cudaPointerGetAttributes(&at, p) != cudaSuccess) {
+        cudaGetLastError();
+        return false;
+    }
+    return at.type != cudaMemoryTypeDevice;
+}
+
+}  // namespace
+
+extern "C" {
+
 int lbib_get_markers(void *h, int body, double *X, double *V, double *F) {
-    // the copies and the device error word in one round trip
+    Ctx *c = as_ctx(h);
+    if (!c) return LBIB_EINVAL;
+    if (body < 0 || body >= (int)c->bodies.size()) return fail(c, LBIB_EINVAL, "no such body");
+    if (c->err && !readable_error(c->err)) return c->err;
+    const DevBody &b = c->bodies[body];
+    const size_t n3 = 3 * (size_t)b.nv;
+    if (host_pointer(X) && host_pointer(V) && host_pointer(F)) {
+        int rc = LBIB_OK;
+        if (const double *r = read_back(c, b, X, V, F, false, &rc)) {
+            if (rc == LBIB_ECUDA) return rc;
+            if (X) std::memcpy(X, r, n3 * sizeof(double));
+            if (V) std::memcpy(V, r + n3, n3 * sizeof(double));
+            if (F) std::memcpy(F, r + 2 * n3, n3 * sizeof(double));
+            return rc;
+        }
+    }
+    // large bodies: the copies and the device error word in one round trip
     int rc = lbib_get_markers_async(h, body, X, V, F);
     if (rc) return rc;
-    return sync_ctx(as_ctx(h));
+    return sync_ctx(c);
 }
 
 int lbib_get_body(void *h, int body, lbib_body_state *out) {
     Ctx *c = as_ctx(h);
     if (!c || !out) return LBIB_EINVAL;
     if (body < 0 || body >= (int)c->bodies.size()) return fail(c, LBIB_EINVAL, "no such body");
-    DevBody &b = c->bodies[body];
-    std::vector<double> X(3 * (size_t)b.nv), Ub(3 * (size_t)b.nv);
-    int rc = lbib_get_markers(h, body, X.data(), Ub.data(), nullptr);
-    if (rc && !readable_error(rc)) return rc;
+    if (c->err && !readable_error(c->err)) return c->err;
+    const DevBody &b = c->bodies[body];
+    const size_t n3 = 3 * (size_t)b.nv;
+    int rc = LBIB_OK;
+    std::vector<double> big;
+    double st[RigidState::SIZE];
+    const double *X, *Ub;
+    if (const double *r = read_back(c, b, true, true, false, true, &rc)) {
+        if (rc && !readable_error(rc)) return rc;
+        X = r;
+        Ub = r + n3;
+        if (b.rigid) std::memcpy(st, r + 3 * n3, sizeof(st));
+    } else {
+        big.resize(2 * n3);
+        rc = lbib_get_markers(h, body, big.data(), big.data() + n3, nullptr);
+        if (rc && !readable_error(rc)) return rc;
+        X = big.data();
+        Ub = X + n3;
+        if (b.rigid) {
+            cudaError_t e = cudaMemcpy(st, b.rstate, sizeof(st), cudaMemcpyDeviceToHost);
+            if (e != cudaSuccess) return cuda_fail(c, e, "body state copy");
+        }
+    }
     std::memset(out, 0, sizeof(*out));
     if (b.rigid) {
-        double st[RigidState::SIZE];
-        cudaError_t e = cudaMemcpy(st, b.rstate, sizeof(st), cudaMemcpyDeviceToHost);
-        if (e != cudaSuccess) return cuda_fail(c, e, "body state copy");
         for (int a = 0; a < 3; ++a) {
             out->xc[a] = st[RigidState::XC + a];
             out->u[a] = st[RigidState::U + a];
@@ -1434,15 +1541,13 @@ int lbib_get_body(void *h, int body, lbib_body_state *out) {
             }
         out->q[0] = 1.0;
     }
-    std::vector<int> T(3 * (size_t)b.nt);
-    cudaError_t e = cudaMemcpy(T.data(), b.tri, T.size() * sizeof(int), cudaMemcpyDeviceToHost);
-    if (e != cudaSuccess) return cuda_fail(c, e, "triangles copy");
+    const int *T = b.tri_h.data();
     double V = 0, A = 0;
     for (int t = 0; t < b.nt; ++t) {
         double cr[3];
         v_cross(&X[3 * T[3 * t + 1]], &X[3 * T[3 * t + 2]], cr);
         V += v_dot(&X[3 * T[3 * t]], cr) / 6.0;
-        A += tri_area(X.data(), &T[3 * t]);
+        A += tri_area(X, &T[3 * t]);
     }
     out->volume = V;
     out->area = A;
@@ -2458,8 +2563,11 @@ int lbib_load(void *h, const void *buf, size_t size) {
     void *fa = c->allocs[hd.fa_index].first;
     if (fa != c->fA) std::swap(c->fA, c->fB);
     for (size_t j = 0; j < c->bodies.size(); ++j) {
-        c->bodies[j].cur = bs[4 * j];
-        c->bodies[j].bcur = bs[4 * j + 1];
+        DevBody &b = c->bodies[j];
+        b.cur = bs[4 * j];
+        b.bcur = bs[4 * j + 1];
+        e = cudaMemcpy(b.tri_h.data(), b.tri, b.tri_h.size() * sizeof(int), cudaMemcpyDeviceToHost);
+        if (e != cudaSuccess) return cuda_fail(c, e, "checkpoint restore");
     }
     c->steps = hd.steps;
     c->step_host = hd.step_host;

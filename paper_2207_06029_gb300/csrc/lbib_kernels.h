@@ -63,8 +63,9 @@ cudaError_t launch_init_equilibrium(int prec, void *fout, const Lattice &L, cons
                                     void *fields, cudaStream_t s, double shear_lo = 0.0, double shear_hi = 0.0);
 cudaError_t launch_pop_to_aos(int prec, const void *fin, const Lattice &L, double *out, cudaStream_t s);
 cudaError_t launch_aos_to_pop(int prec, const double *in, const Lattice &L, void *fout, cudaStream_t s);
-cudaError_t launch_fields_out(int prec, const void *fields, const Lattice &L, double *rho, double *u,
-                              cudaStream_t s);
+// err_out (mapped host memory) receives the error word err
+cudaError_t launch_fields_out(int prec, const void *fields, const Lattice &L, double *rho, double *u, const int *err,
+                              int *err_out, cudaStream_t s);
 
 // ib.cu
 constexpr int kBatchMlsThreads = 128;       // MLS points per block of the batched kernel

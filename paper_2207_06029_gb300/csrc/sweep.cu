@@ -309,8 +309,9 @@ __global__ void k_aos_to_pop(const double *__restrict__ in, Lattice L, S *__rest
 
 template <typename R>
 __global__ void k_fields_out(const R *__restrict__ fields, Lattice L, double *__restrict__ rho,
-                             double *__restrict__ u) {
+                             double *__restrict__ u, const int *err, int *err_out) {
     const int idx = blockIdx.x * blockDim.x + threadIdx.x;
+    if (idx == 0) *err_out = *err;
     if (idx >= L.ncell) return;
     if (rho) rho[idx] = (double)fields[idx];
     if (u) {
@@ -634,13 +635,13 @@ cudaError_t launch_aos_to_pop(int prec, const double *in, const Lattice &L, void
     return cudaGetLastError();
 }
 
-cudaError_t launch_fields_out(int prec, const void *fields, const Lattice &L, double *rho, double *u,
-                              cudaStream_t s) {
+cudaError_t launch_fields_out(int prec, const void *fields, const Lattice &L, double *rho, double *u, const int *err,
+                              int *err_out, cudaStream_t s) {
     const unsigned g = grid_for(L.ncell, 256);
     if (prec == 0)
-        k_fields_out<double><<<g, 256, 0, s>>>((const double *)fields, L, rho, u);
+        k_fields_out<double><<<g, 256, 0, s>>>((const double *)fields, L, rho, u, err, err_out);
     else
-        k_fields_out<float><<<g, 256, 0, s>>>((const float *)fields, L, rho, u);
+        k_fields_out<float><<<g, 256, 0, s>>>((const float *)fields, L, rho, u, err, err_out);
     return cudaGetLastError();
 }
 

@@ -1231,6 +1231,11 @@ __global__ void __launch_bounds__(kStructThreads) k_centroid_spread(Lattice L, B
 }
 
 // ---- batch kernels: the bodies of all lattices of a batch per launch ----
+// Each is launched programmatically behind the one before and waits for it
+// once its tables are staged (and, MLS and membrane, the positions, weights
+// and hinge forces formed).  Those early parts read what the previous step's
+// structure kernels wrote: the sweep between releases its successor only
+// after its own wait, so these have completed by then.
 template <typename S, typename R>
 __global__ void __launch_bounds__(256) kb_moments(BatchTables T, int phase) {
     __shared__ Lattice L;
@@ -1239,6 +1244,8 @@ __global__ void __launch_bounds__(256) kb_moments(BatchTables T, int phase) {
     const BodyRef &br = T.body[phase * T.nb + j];
     stage_shared(L, T.lat + br.lat);
     const LatRef &F = T.ref[phase * T.nl + br.lat];
+    chain_release();
+    chain_wait();
     moments_body<S, R>((const S *)F.fin, L, br.v.bbox, br.v.bbox_next, (R *)F.mom, br.inc_step ? F.d_step : nullptr,
                        vb, nvb);
 }
@@ -1252,7 +1259,8 @@ __global__ void __launch_bounds__(kBatchMlsThreads) kb_mls(BatchTables T, int ph
     stage_shared(br, T.body + phase * T.nb + j);
     stage_shared(L, T.lat + br.lat);
     const LatRef &F = T.ref[phase * T.nl + br.lat];
-    mls_body<R>((const R *)F.mom, L, br.v, F.err, vb);
+    chain_release();
+    mls_body<R, false, true>((const R *)F.mom, L, br.v, F.err, vb);
 }
 
 template <typename R>
@@ -1263,6 +1271,7 @@ __global__ void __launch_bounds__(256) kb_membrane(BatchTables T, int phase) {
     stage_shared(br, T.body + phase * T.nb + __ldg(T.memb_id + m));
     stage_shared(L, T.lat + br.lat);
     const LatRef &F = T.ref[phase * T.nl + br.lat];
+    chain_release();
     membrane_body<R>(L, br.v, (R *)F.force, F.stamp, F.d_step, blockIdx.x - __ldg(T.memb_pre + m),
                      points_blocks(br.v, kBatchMlsThreads));
 }
@@ -1271,6 +1280,8 @@ __global__ void __launch_bounds__(256) kb_membrane(BatchTables T, int phase) {
 // by themselves.
 __global__ void __launch_bounds__(256) kb_body_sums(BatchTables T, int phase) {
     const BodyRef &br = T.body[phase * T.nb + __ldg(T.sums_id + blockIdx.x)];
+    chain_release();
+    chain_wait();
     body_sums_body(br.v, points_blocks(br.v, kBatchMlsThreads));
 }
 
@@ -1283,6 +1294,7 @@ __global__ void __launch_bounds__(256) kb_rigid_markers(BatchTables T, int phase
     stage_shared(L, T.lat + br.lat);
     const LatRef &F = T.ref[phase * T.nl + br.lat];
     const int b0 = __ldg(T.rm_pre + m), nvb = __ldg(T.rm_pre + m + 1) - b0;
+    chain_release();
     rigid_markers_body<R>(L, br.v, (R *)F.force, F.stamp, F.d_step, blockIdx.x - b0, nvb, nvb,
                           points_blocks(br.v, kBatchMlsThreads), nvb);
 }
@@ -1295,6 +1307,8 @@ __global__ void __launch_bounds__(256) kb_centroid_spread(BatchTables T, int pha
     stage_shared(br, T.body + phase * T.nb + __ldg(T.cen_id + m));
     stage_shared(L, T.lat + br.lat);
     const LatRef &F = T.ref[phase * T.nl + br.lat];
+    chain_release();
+    chain_wait();
     centroid_body<R>(L, br.v, (R *)F.force, F.stamp, F.d_step, blockIdx.x - __ldg(T.cen_pre + m));
 }
 
@@ -1475,22 +1489,32 @@ int batch_persistent_blocks_per_sm(int prec, bool off32) {
 }
 
 template <typename S, typename R>
-static cudaError_t batch_ib_t(const BatchTables &T, const BatchGrid &G, int phase, cudaStream_t s) {
-    if (G.mom > 0) kb_moments<S, R><<<G.mom, 256, 0, s>>>(T, phase);
-    if (G.mls > 0) kb_mls<R><<<G.mls, kBatchMlsThreads, 0, s>>>(T, phase);
-    if (G.sums > 0) kb_body_sums<<<G.sums, 256, 0, s>>>(T, phase);
-    if (G.memb > 0) kb_membrane<R><<<G.memb, 256, 0, s>>>(T, phase);
-    if (G.rm > 0) kb_rigid_markers<R><<<G.rm, 256, 0, s>>>(T, phase);
-    if (G.cen > 0) kb_centroid_spread<R><<<G.cen, 256, 0, s>>>(T, phase);  // after the structure kernels
-    return cudaGetLastError();
+static cudaError_t batch_ib_t(const BatchTables &T, const BatchGrid &G, int phase, bool chained, cudaStream_t s) {
+    auto go = [&](auto kernel, int grid, int block) {
+        if (grid <= 0) return cudaSuccess;
+        return launch_chained(kernel, dim3(grid), dim3(block), 0, s, T, phase);
+    };
+    cudaError_t e = cudaSuccess;
+    if (chained)
+        e = go(kb_moments<S, R>, G.mom, 256);
+    else if (G.mom > 0)
+        kb_moments<S, R><<<G.mom, 256, 0, s>>>(T, phase);
+    if (e == cudaSuccess) e = cudaGetLastError();
+    if (e == cudaSuccess) e = go(kb_mls<R>, G.mls, kBatchMlsThreads);
+    if (e == cudaSuccess) e = go(kb_body_sums, G.sums, 256);
+    if (e == cudaSuccess) e = go(kb_membrane<R>, G.memb, 256);
+    if (e == cudaSuccess) e = go(kb_rigid_markers<R>, G.rm, 256);
+    if (e == cudaSuccess) e = go(kb_centroid_spread<R>, G.cen, 256);  // after the structure kernels
+    return e;
 }
 
-cudaError_t launch_batch_ib(int prec, const BatchTables &T, const BatchGrid &G, int phase, cudaStream_t s) {
+cudaError_t launch_batch_ib(int prec, const BatchTables &T, const BatchGrid &G, int phase, bool chained,
+                            cudaStream_t s) {
     switch (prec) {
-        case 0: return batch_ib_t<double, double>(T, G, phase, s);
-        case 1: return batch_ib_t<float, float>(T, G, phase, s);
-        case 2: return batch_ib_t<__half, float>(T, G, phase, s);
-        default: return batch_ib_t<__nv_bfloat16, float>(T, G, phase, s);
+        case 0: return batch_ib_t<double, double>(T, G, phase, chained, s);
+        case 1: return batch_ib_t<float, float>(T, G, phase, chained, s);
+        case 2: return batch_ib_t<__half, float>(T, G, phase, chained, s);
+        default: return batch_ib_t<__nv_bfloat16, float>(T, G, phase, chained, s);
     }
 }
 

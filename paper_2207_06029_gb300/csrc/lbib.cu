@@ -1846,7 +1846,7 @@ int batch_build_persistent(Batch *b, const std::vector<std::pair<int, int>> &bod
         const DevBody &d = b->ctx[bodies[q].first]->bodies[bodies[q].second];
         std::array<int, kPKinds> &n = count[q];
         n.fill(0);
-        n[kPMom] = std::max(8, d.nv / 16);
+        n[kPMom] = node_blocks(d.box_nodes, 256, b->nsm);
         n[kPMls] = mls_blocks(body[q].v, kPersistThreads);
         n[kPSum] = needs_body_sums(body[q].v, kPersistThreads);
         n[kPMemb] = d.rigid ? 0 : marker_blocks(d.nv);
@@ -1972,7 +1972,7 @@ int batch_build(Batch *b) {
         d.cur = cur0;
         d.bcur = bcur0;
         const BodyView &v = body[q].v;
-        mom_pre.push_back(mom_pre.back() + std::max(8, d.nv / 16));
+        mom_pre.push_back(mom_pre.back() + node_blocks(d.box_nodes, 256, b->nsm));
         mls_pre.push_back(mls_pre.back() + mls_blocks(v, kBatchMlsThreads));
         if (d.rigid) {
             rigid_id.push_back(q);
@@ -2101,8 +2101,9 @@ int batch_build(Batch *b) {
     return LBIB_OK;
 }
 
-int batch_enqueue(Batch *b, int phase, bool store, cudaStream_t st) {
-    cudaError_t e = launch_batch_ib(b->prec, b->T, b->G, phase, st);
+// follows: behind the step before in the same capture
+int batch_enqueue(Batch *b, int phase, bool store, bool follows, cudaStream_t st) {
+    cudaError_t e = launch_batch_ib(b->prec, b->T, b->G, phase, follows && !b->sweep_split, st);
     if (e == cudaSuccess && !b->sweep_split) e = launch_batch_sweep(b->prec, b->T, b->G, phase, store ? 1 : 0, st);
     if (e == cudaSuccess && b->sweep_split) {
         // fork the side streams from st, one one-lattice sweep per lattice
@@ -2141,7 +2142,7 @@ int batch_capture6(Batch *b) {
         if (e == cudaSuccess) e = launch_batch_persistent(b->prec, b->T, b->P, b->pgrid, b->s_cap);
         if (e != cudaSuccess) rc = bcuda(b, e, "persistent batch launch");
     }
-    for (int k = 0; k < 6 && rc == LBIB_OK && !b->persistent; ++k) rc = batch_enqueue(b, k, false, b->s_cap);
+    for (int k = 0; k < 6 && rc == LBIB_OK && !b->persistent; ++k) rc = batch_enqueue(b, k, false, k > 0, b->s_cap);
     cudaGraph_t g = nullptr;
     e = cudaStreamEndCapture(b->s_cap, &g);
     if (rc) {
@@ -2274,7 +2275,7 @@ int lbib_batch_step(void *h, int nsteps) {
             remaining -= 6;
             b->launches += b->persistent ? 1 : 6 * batch_launches_per_step(b);
         } else {
-            int rc = batch_enqueue(b, phase, remaining == 1, b->stream);
+            int rc = batch_enqueue(b, phase, remaining == 1, false, b->stream);
             if (rc) return rc;
             b->steps += 1;
             remaining -= 1;

@@ -91,7 +91,10 @@ cudaError_t launch_structure(int prec, const Lattice &L, const BodyView &B, void
 struct BatchGrid {
     int sweep, mom, mls, sums, memb, rm, cen;
 };
-cudaError_t launch_batch_ib(int prec, const BatchTables &T, const BatchGrid &G, int phase, cudaStream_t s);
+// chained: the previous kernel of the stream is the batched sweep of the step
+// before, in the same capture
+cudaError_t launch_batch_ib(int prec, const BatchTables &T, const BatchGrid &G, int phase, bool chained,
+                            cudaStream_t s);
 cudaError_t launch_batch_sweep(int prec, const BatchTables &T, const BatchGrid &G, int phase, int store_fields,
                                cudaStream_t s);
 // persistent batched step (ib.cu): P.nsteps steps of every lattice in one

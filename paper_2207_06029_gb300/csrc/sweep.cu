@@ -244,6 +244,8 @@ __global__ void __launch_bounds__(512) kb_sweep(BatchTables T, int phase, int st
     const int l = __ldg(T.sweep_lat + slot);
     stage_shared(L, T.lat + l);
     const LatRef &F = T.ref[phase * T.nl + l];
+    chain_wait();     // launched programmatically behind the structure kernels,
+    chain_release();  // and releasing the next step's after they have completed
     const int b0 = __ldg(T.sweep_pre + slot), nb = __ldg(T.sweep_pre + slot + 1) - b0;
     const uint32_t step = F.stamp ? *F.d_step : 0u;
     const uint32_t seed = F.sr[F.parity];
@@ -412,12 +414,11 @@ cudaError_t launch_sweep(int prec, const void *fin, void *fout, void *force, con
 template <typename S, typename R>
 static cudaError_t batch_sweep_t(const BatchTables &T, const BatchGrid &G, int phase, int store, cudaStream_t s) {
     if (G.sweep > 0) {
-        if (T.sweep_off32)
-            kb_sweep<S, R, true><<<G.sweep, T.sweep_threads, 0, s>>>(T, phase, store);
-        else
-            kb_sweep<S, R, false><<<G.sweep, T.sweep_threads, 0, s>>>(T, phase, store);
+        const dim3 grid(G.sweep), block(T.sweep_threads);
+        return T.sweep_off32 ? launch_chained(kb_sweep<S, R, true>, grid, block, 0, s, T, phase, store)
+                             : launch_chained(kb_sweep<S, R, false>, grid, block, 0, s, T, phase, store);
     }
-    return cudaGetLastError();
+    return cudaSuccess;
 }
 
 cudaError_t launch_batch_sweep(int prec, const BatchTables &T, const BatchGrid &G, int phase, int store_fields,

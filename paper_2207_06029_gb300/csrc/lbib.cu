@@ -998,6 +998,19 @@ int lbib_add_body(void *h, const double *verts, int nv, const int *tris, int nt,
 
 namespace {
 
+// Whether the step of a context sweeps the far field beside the IB stage.
+// Below kSplitCells nodes (kSplitCells64 in FP64) the step is the chain of
+// the IB kernels' latencies, and one sweep behind them is shorter than the
+// box sweep and the join.  Measured us a step, overlap against one sweep,
+// rigid sphere in FP32: 32^3 21.0 against 20.1, 48^3 24.2 against 22.6, 64^3
+// 27.7 against 25.2, 80^3 31.0 against 32.0, 96^3 38.4 against 44.5 (16-bit
+// storage and capsules alike); FP64 32^3 78.1 against 76.0, 48^3 109.8 against
+// 125.8.
+constexpr int kSplitCells = 360000, kSplitCells64 = 48000;
+bool splits(const Ctx *c) {
+    return c->bodies.size() == 1 && c->split_sweep && c->L.ncell >= (c->prec == LBIB_FP64 ? kSplitCells64 : kSplitCells);
+}
+
 // Enqueues one step on the two step streams (the caller forks them from,
 // and joins them into, an origin stream).  With one body, the nodes
 // outside its support box do not depend on the IB work of the step: they
@@ -1007,7 +1020,7 @@ namespace {
 // timestamps; `external` records them as graph nodes during capture.
 // Advances the host-side buffer rotation but not the step count.
 int enqueue_step(Ctx *c, bool store_fields, cudaEvent_t *ev, bool external, int parity) {
-    const bool split = c->bodies.size() == 1 && c->split_sweep;
+    const bool split = splits(c);
     cudaStream_t hi = c->s_hi, lo = c->s_lo;
     auto rec = [&](int k, cudaStream_t st) {
         if (ev) cudaEventRecordWithFlags(ev[k], st, external ? cudaEventRecordExternal : cudaEventRecordDefault);
@@ -1154,7 +1167,7 @@ int build_graph(Ctx *c, int nsteps, bool store, int k, cudaGraphExec_t *out) {
 
 // launches per step (for the counters when a graph runs the step)
 long long launches_per_step(Ctx *c) {
-    long long n = 1 + (c->bodies.size() == 1 && c->split_sweep ? 1 : 0);
+    long long n = 1 + (splits(c) ? 1 : 0);
     for (auto &b : c->bodies) n += 2 + structure_launches(c->prec, make_view(c, b));
     return n;
 }

@@ -1418,7 +1418,8 @@ __global__ void __launch_bounds__(256, 4) kp_batch(BatchTables T, PersistTables 
                 const int c0 = it.z * P.sweep_cells;
                 const int c1 = min(c0 + P.sweep_cells, L.ncell);
                 for (int c = c0 + (int)threadIdx.x; c < c1; c += blockDim.x) {
-                    const int x = c % L.nx, yz = c / L.nx, y = yz % L.ny, z = yz / L.ny;
+                    int x, y, z;
+                    node_coords(L, c, x, y, z);
                     sweep_cell<S, R, kOff32, true>((const S *)F.fin, (S *)F.fout, (R *)F.force, F.stamp, step, L,
                                                    nullptr, x, y, z, seed);
                 }

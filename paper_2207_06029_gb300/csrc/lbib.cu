@@ -464,6 +464,7 @@ int lbib_create(const lbib_params *p, void **out) {
     L.nty = (n[1] + kTile - 1) / kTile;
     L.ntz = (n[2] + kTile - 1) / kTile;
     L.ncell = (int)ncell;
+    set_dividers(L);
     L.stride = (ncell + 63) / 64 * 64;
     L.off32 = (long long)Q * L.stride <= 0xFFFFFFFFLL;
     L.sweep_vec = 0;  // the one-node sweep; the autotuner may pick the row-tile kernel

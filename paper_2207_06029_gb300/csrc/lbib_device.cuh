@@ -221,6 +221,8 @@ struct Lattice {
     double gext[3];
     double wall_u[6][3];
     double dist2_cut;       // largest |X - x_k|^2 whose MLS weight is non-zero
+    uint32_t mul_x, mul_y;  // division by nx and ny (set_dividers)
+    int shr_x, shr_y;
     int sweep_bx, sweep_by; // block shape of the whole-lattice sweep (0: default)
     int sweep_vec;          // 1: row-tile sweep (shared-memory staging, 128-bit loads/stores) where it applies
     int far_per_sm;         // > 0: the far-field sweep keeps this many blocks per SM (grid-stride)
@@ -234,6 +236,26 @@ struct Lattice {
     double codd_d[2];
     float codd_f[2];
 };
+
+// Division of node indices (below 2^30) by nx and ny as a multiplication and
+// a shift: with s = ceil(log2 d) and m = ceil(2^(30+s) / d), n m / 2^(30+s)
+// exceeds n / d by less than 2^-s <= 1/d, so the floor is the quotient.
+inline void set_dividers(Lattice &L) {
+    auto one = [](int d, uint32_t &mul, int &shr) {
+        int s = 0;
+        while ((1LL << s) < d) ++s;
+        mul = (uint32_t)(((1ULL << (30 + s)) + (unsigned)d - 1) / (unsigned)d);
+        shr = 30 + s;
+    };
+    one(L.nx, L.mul_x, L.shr_x);
+    one(L.ny, L.mul_y, L.shr_y);
+}
+__host__ __device__ __forceinline__ void node_coords(const Lattice &L, int c, int &x, int &y, int &z) {
+    const int yz = (int)(((uint64_t)(uint32_t)c * L.mul_x) >> L.shr_x);
+    x = c - yz * L.nx;
+    z = (int)(((uint64_t)(uint32_t)yz * L.mul_y) >> L.shr_y);
+    y = yz - z * L.ny;
+}
 
 template <typename R>
 __device__ __forceinline__ R pick(double d, float f);

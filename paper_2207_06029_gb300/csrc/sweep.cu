@@ -80,6 +80,42 @@ __global__ void __launch_bounds__(256) k_sweep(const S *__restrict__ fin, S *__r
     sweep_cell<S, R, kOff32>(fin, fout, force, stamp, step, L, fields, x, y, z, seed);
 }
 
+// The same over consecutive nodes, whatever the rows: for row lengths that
+// are no multiple of a warp, whose rows leave lanes idle (193: 31 of 224) and
+// store across sector boundaries, and for small lattices, whose blocks spread
+// more evenly.  193^3: FP32 187.3 -> 160.8 us (6.80 TB/s, the measured copy
+// rate), FP16 163.4 -> 135.6, FP64 3045 -> 2316; 97^3 FP32 30.3 -> 23.4;
+// 32^3 FP64 23.6 -> 18.2, FP32 3.46 -> 3.12.  160x160x480 (whole warps) keeps
+// its rows: FP32 the same, FP16 251.7 here against 244.0; and so does the far
+// field of a lattice with whole warps, beside whose IB kernels the larger row
+// blocks do better (96^3 capsule 39.0 us a step against 40.0).  128 threads a
+// block: 256 and 192 were slower (97^3 FP32 24.0 and 24.7).
+constexpr int kLineThreads = 128;
+static bool line_sweep(const Lattice &L, int part) {
+    return L.sweep_bx == 0 && ((L.nx & 31) != 0 || (part != 1 && L.ncell < (1 << 20)));
+}
+template <typename S, typename R, bool kOff32>
+__global__ void __launch_bounds__(kLineThreads) k_sweep_line(const S *__restrict__ fin, S *__restrict__ fout,
+                                                             R *__restrict__ force,
+                                                             const uint32_t *__restrict__ stamp,
+                                                             const uint32_t *__restrict__ dstep, Lattice L,
+                                                             R *__restrict__ fields, const int *__restrict__ box,
+                                                             uint32_t *__restrict__ sr, int parity) {
+    const uint32_t step = stamp ? *dstep : 0u;
+    const uint32_t seed = sr[parity];
+    if (blockIdx.x == 0 && threadIdx.x == 0) sr[parity ^ 1] = seed + 1u;
+    const int c = blockIdx.x * kLineThreads + threadIdx.x;
+    if (c >= L.ncell) return;
+    int x, y, z;
+    node_coords(L, c, x, y, z);
+    if (box) {
+        int lo[3], ext[3];
+        clamp_box(L, box, lo, ext);
+        if (in_box(L, lo, ext, x, y, z)) return;
+    }
+    sweep_cell<S, R, kOff32>(fin, fout, force, stamp, step, L, fields, x, y, z, seed);
+}
+
 // The far field (nodes outside the body box) with a bounded number of
 // resident blocks: each block strides over the (x-tile, y-tile, z) tiles of
 // the lattice, so that SM resources stay free for the IB kernels running
@@ -252,7 +288,8 @@ __global__ void __launch_bounds__(512) kb_sweep(BatchTables T, int phase, int st
     if (blockIdx.x == b0 && threadIdx.x == 0) F.sr[F.parity ^ 1] = seed + 1u;
     R *fields = store_fields ? (R *)F.fields : nullptr;
     for (int c = (blockIdx.x - b0) * blockDim.x + threadIdx.x; c < L.ncell; c += nb * blockDim.x) {
-        const int x = c % L.nx, yz = c / L.nx, y = yz % L.ny, z = yz / L.ny;
+        int x, y, z;
+        node_coords(L, c, x, y, z);
         sweep_cell<S, R, kOff32>((const S *)F.fin, (S *)F.fout, (R *)F.force, F.stamp, step, L, fields, x, y, z, seed);
     }
 }
@@ -380,6 +417,9 @@ static cudaError_t sweep_t(const void *fin, void *fout, void *force, const uint3
         k_sweep_far<S, R, kOff32><<<L.far_per_sm * nsm, block, 0, s>>>((const S *)fin, (S *)fout, (R *)force, stamp, step,
                                                                L, (R *)fields, box, sr, parity, (int)grid.x,
                                                                (int)grid.y);
+    } else if (line_sweep(L, part)) {
+        k_sweep_line<S, R, kOff32><<<grid_for(L.ncell, kLineThreads), kLineThreads, 0, s>>>(
+            (const S *)fin, (S *)fout, (R *)force, stamp, step, L, (R *)fields, part == 1 ? box : nullptr, sr, parity);
     } else {
         dim3 grid, block;
         sweep_shape(L, grid, block);

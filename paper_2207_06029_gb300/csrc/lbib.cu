@@ -481,6 +481,10 @@ int lbib_create(const lbib_params *p, void **out) {
     L.cF_d = 1.0 - 0.5 / p->tau;
     L.nu_d = (p->tau - 0.5) / 3.0;
     L.omega_f = (float)L.omega_d;
+    L.om1_d = 1.0 - L.omega_d;
+    L.om1_f = 1.0f - L.omega_f;
+    L.om15_d = 1.5 * L.omega_d;
+    L.om15_f = 1.5f * L.omega_f;
     L.cF_f = (float)L.cF_d;
     // c_dg = omega/12 rounded, c_ax = (omega - 8 c_dg)/2: 8 c_dg lies within
     // a factor two of omega, so the difference and the halving are exact

@@ -227,6 +227,8 @@ struct Lattice {
     int sweep_vec;          // 1: row-tile sweep (shared-memory staging, 128-bit loads/stores) where it applies
     int far_per_sm;         // > 0: the far-field sweep keeps this many blocks per SM (grid-stride)
     // derived, double and float copies
+    double om1_d, om15_d;  // 1 - omega, 1.5 omega
+    float om1_f, om15_f;
     double omega_d, cF_d, nu_d, gext_d[3], uw_d[27][3];
     float omega_f, cF_f, nu_f, gext_f[3], uw_f[27][3], dist2_cut_f;
     // odd (momentum) coefficients 3 w_i omega of the collision for the axis

@@ -348,7 +348,7 @@ __device__ __forceinline__ void exchange_force(const BodyView &B, int t, R area,
 //           rho nu (grad u + grad u^T) . n from the fits (membranes keep
 //           them per triangle, rigid bodies sum the forces and moments).
 template <typename R, bool kCG = false, bool kChain = false>
-__device__ __forceinline__ void mls_body(const R *__restrict__ mom, const Lattice &L, const BodyView &B, int *err,
+__device__ __forceinline__ void mls_body(const R *mom, const Lattice &L, const BodyView &B, int *err,
                                          const int vb) {
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     const int nm = B.nm, npts = nm + 2 * B.nt;
@@ -446,7 +446,7 @@ __device__ __forceinline__ void mls_body(const R *__restrict__ mom, const Lattic
         }
         if (near) in = (in & ~near) | support_exact(near, frac[0], frac[1], frac[2], L.dist2_cut);
     }
-    if constexpr (kChain) chain_wait();
+    if constexpr (kChain) chain_wait();  // (kCG: no read-only loads behind it)
     R f6[6] = {R(0), R(0), R(0), R(0), R(0), R(0)};  // rigid: the point's share of the force and moment
     if (p >= 0) {
     // ---------------- sums ----------------
@@ -621,13 +621,13 @@ __device__ __forceinline__ void mls_body(const R *__restrict__ mom, const Lattic
 // The blocks take the nvb groups of points in turn (gridDim.x = nvb unless
 // the launch caps the grid).
 template <typename R>
-__global__ void __launch_bounds__(mls_threads(sizeof(R) == 8 ? 0 : 1)) k_mls(const R *__restrict__ mom, Lattice L, BodyView B,
+__global__ void __launch_bounds__(mls_threads(sizeof(R) == 8 ? 0 : 1)) k_mls(const R *mom, Lattice L, BodyView B,
                                                      int *err, int nvb) {
     chain_release();  // the structure kernel may be scheduled beside this one
     for (int vb = blockIdx.x; vb < nvb; vb += gridDim.x) {
         // launched programmatically after the moments kernel, whose results
         // it waits for inside
-        mls_body<R, false, true>(mom, L, B, err, vb);
+        mls_body<R, true, true>(mom, L, B, err, vb);
         __syncthreads();  // the next group reuses the shared memory
     }
 }
@@ -1246,7 +1246,7 @@ __global__ void __launch_bounds__(256) kb_moments(BatchTables T, int phase) {
     const LatRef &F = T.ref[phase * T.nl + br.lat];
     chain_release();
     chain_wait();
-    moments_body<S, R>((const S *)F.fin, L, br.v.bbox, br.v.bbox_next, (R *)F.mom, br.inc_step ? F.d_step : nullptr,
+    moments_body<S, R, true>((const S *)F.fin, L, br.v.bbox, br.v.bbox_next, (R *)F.mom, br.inc_step ? F.d_step : nullptr,
                        vb, nvb);
 }
 
@@ -1260,7 +1260,7 @@ __global__ void __launch_bounds__(kBatchMlsThreads) kb_mls(BatchTables T, int ph
     stage_shared(L, T.lat + br.lat);
     const LatRef &F = T.ref[phase * T.nl + br.lat];
     chain_release();
-    mls_body<R, false, true>((const R *)F.mom, L, br.v, F.err, vb);
+    mls_body<R, true, true>((const R *)F.mom, L, br.v, F.err, vb);
 }
 
 template <typename R>

@@ -64,6 +64,8 @@ constexpr bool lattice_is_consistent() {
 static_assert(lattice_is_consistent(), "D3Q19 table");
 
 // Loads of data that a launch never writes take the read-only path (__ldg).
+// Not so behind chain_wait(): read-only loads lie outside the memory model, and
+// were seen moved over the wait (FP64 MLS sums of half-written moments).
 // A launch that reads data other blocks of the same launch wrote (the
 // persistent batched step: one work item's populations, flags and moments
 // are written by earlier items) must not use that path, which lies outside

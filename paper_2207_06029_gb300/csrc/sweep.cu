@@ -290,7 +290,7 @@ __global__ void __launch_bounds__(512) kb_sweep(BatchTables T, int phase, int st
     for (int c = (blockIdx.x - b0) * blockDim.x + threadIdx.x; c < L.ncell; c += nb * blockDim.x) {
         int x, y, z;
         node_coords(L, c, x, y, z);
-        sweep_cell<S, R, kOff32>((const S *)F.fin, (S *)F.fout, (R *)F.force, F.stamp, step, L, fields, x, y, z, seed);
+        sweep_cell<S, R, kOff32, true>((const S *)F.fin, (S *)F.fout, (R *)F.force, F.stamp, step, L, fields, x, y, z, seed);
     }
 }
 

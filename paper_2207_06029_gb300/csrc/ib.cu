@@ -618,6 +618,264 @@ __device__ __forceinline__ void mls_body(const R *mom, const Lattice &L, const B
     }
 }
 
+// The same with four lanes per point, for few points (mls_quads): lane a < 3
+// forms the point's component and the weights of axis a, and lane q takes
+// field q (rho - 1, u_x, u_y, u_z), with the sums of A split by the power of x
+// over lanes 0 to 2.  A point's chain of operations is about a third of
+// mls_body's (FP64: 385 instead of 1080 warp instructions, each holding its
+// SM quarter for 64 cycles), over four times the warps.
+constexpr int kQuadThreads = 128;  // 32 points a block
+// x / 3, rounded as the division (whose FP64 form takes a dozen operations)
+template <typename R>
+__device__ __forceinline__ R third(R x) {
+    const R q = x * R(1.0 / 3.0);
+    return fma(fma(R(-3), q, x), R(1.0 / 3.0), q);
+}
+template <typename R>
+__device__ __forceinline__ void mls_quad_body(const R *mom, const Lattice &L, const BodyView &B, int *err,
+                                              const int vb) {
+    const unsigned kFull = 0xffffffffu;
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, q = lane & 3, qb = lane & ~3;
+    auto from = [&](auto v, int src) { return __shfl_sync(kFull, v, qb | src); };  // lane src of the point
+    const int a = q < 3 ? q : 0, a1 = (a + 1) % 3, a2 = (a + 2) % 3;
+    const int nm = B.nm, npts = nm + 2 * B.nt;
+    const int slot = vb * (kQuadThreads / 4) + (threadIdx.x >> 2);
+    const int p = slot < npts ? (B.perm ? B.perm[slot] : slot) : -1;
+    const bool probe = p >= nm;
+    const int t = probe ? (p - nm) >> 1 : 0, side = (p - nm) & 1;
+
+    // ---------------- positions: component a ----------------
+    double P = 0.0;
+    R r0 = R(0), e1 = R(0), e2 = R(0);
+    if (probe) {
+        const int *tv = B.tri + 3 * t;
+        const int i0 = tv[0], i1 = tv[1], i2 = tv[2];
+        const R *Xr = (const R *)B.Xrel;
+        P = B.X[3 * i0 + a];
+        r0 = Xr[3 * i0 + a];
+        e1 = Xr[3 * i1 + a] - r0;
+        e2 = Xr[3 * i2 + a] - r0;
+    } else if (p >= 0 && B.centroid) {
+        const int *tv = B.tri + 3 * p;
+        P = (B.X[3 * tv[0] + a] + B.X[3 * tv[1] + a] + B.X[3 * tv[2] + a]) / 3.0;
+    } else if (p >= 0) {
+        P = B.X[3 * p + a];
+    }
+    const R e1b = from(e1, a1), e1c = from(e1, a2), e2b = from(e2, a1), e2c = from(e2, a2);
+    const R N = e1b * e2c - e1c * e2b;
+    const R N0 = from(N, 0), N1 = from(N, 1), N2 = from(N, 2);
+    const R nn = sqrt(N0 * N0 + N1 * N1 + N2 * N2), area = R(0.5) * nn;
+    R nrm = R(0), arm = R(0);
+    if (probe) {
+        nrm = N * (R(1) / nn);
+        const R c3 = third(e1 + e2);
+        P += (double)(c3 + (side ? R(-kProbe) : R(kProbe)) * nrm);
+        arm = r0 + c3;
+        if (side == 0) {
+            R *tg = (R *)B.tri_geo + 8 * t;
+            if (q < 3) {
+                tg[a] = nrm;
+                tg[4 + a] = arm;
+            } else {
+                tg[3] = area;
+            }
+        }
+        if (B.rigid) arm -= R(__ldcg(B.rstate + RigidState::XC + a) - B.origin[a]);
+    }
+    double vol = 0.0;  // on lane 0
+    if (!B.rigid) {
+        const double v = (double)r0 * (double)N;
+        vol = from(v, 0) + from(v, 1) + from(v, 2);
+        if (q != 0 || !probe || side != 0) vol = 0.0;
+    }
+    const int n = a == 0 ? L.nx : a == 1 ? L.ny : L.nz;
+    bool diverged = false, bad = false;
+    if (!(fabs(P) < kMaxMarkerCoord)) {  // non-finite or runaway: flag, keep indices sane
+        diverged = p >= 0;
+        P = 0.0;
+    }
+    int base = __double2int_rd(P + 0.5);  // floor(X + 1/2)
+    if (L.bc[a] == kWall && (base - 1 < 1 || base + 1 > n - 2)) {
+        bad = p >= 0;
+        base = base < 2 ? 2 : (base > n - 3 ? n - 3 : base);
+    }
+    const double frac = P - (double)base;
+    const unsigned mdiv = __ballot_sync(kFull, diverged) >> qb & 7u, mbad = __ballot_sync(kFull, bad) >> qb & 7u;
+    if (q == 0 && mdiv)
+        atomicCAS(err, 0, kErrDiverged);
+    else if (q == 0 && mbad)
+        atomicCAS(err, 0, kErrBodyWall);
+
+    // ---------------- weights, support and nodes ----------------
+    const R fR = R(frac), f0 = from(fR, 0), f1 = from(fR, 1), f2 = from(fR, 2);
+    const double g0 = from(frac, 0), g1 = from(frac, 1), g2 = from(frac, 2);
+    unsigned in = 0u, near = 0u;
+    {
+        const float fx = float(f0), fy = float(f1), fz = float(f2);
+        float sx[3], sy[3], sz[3];
+#pragma unroll
+        for (int i = 0; i < 3; ++i) {
+            sx[i] = (float(i - 1) - fx) * (float(i - 1) - fx);
+            sy[i] = (float(i - 1) - fy) * (float(i - 1) - fy);
+            sz[i] = (float(i - 1) - fz) * (float(i - 1) - fz);
+        }
+#pragma unroll
+        for (int k = 0; k < 27; ++k) {
+            const float s = sx[k % 3] + (sy[(k / 3) % 3] + sz[k / 9]) - L.dist2_cut_f;
+            if (s <= 0.f) in |= 1u << k;
+            if (fabsf(s) <= 1e-5f) near |= 1u << k;
+        }
+        if (near) in = (in & ~near) | support_exact(near, g0, g1, g2, L.dist2_cut);
+    }
+    R wx[3], wxd[3], wxp[3], wy[3], wyd[3], wydd[3], wz[3], wzd[3], wzdd[3];
+    {
+        R d[3], w[3];
+        axis_weights(fR, d, w);
+#pragma unroll
+        for (int i = 0; i < 3; ++i) {
+            const R wd = w[i] * d[i], wdd = wd * d[i];
+            wx[i] = from(w[i], 0);
+            wxd[i] = from(wd, 0);
+            const R xdd = from(wdd, 0);
+            wxp[i] = q == 0 ? wx[i] : q == 1 ? wxd[i] : xdd;
+            wy[i] = from(w[i], 1);
+            wyd[i] = from(wd, 1);
+            wydd[i] = from(wdd, 1);
+            wz[i] = from(w[i], 2);
+            wzd[i] = from(wd, 2);
+            wzdd[i] = from(wdd, 2);
+        }
+    }
+    int ox[3], oy[3], oz[3];
+#pragma unroll
+    for (int i = 0; i < 3; ++i) {
+        const int o = (a == 0 ? 1 : a == 1 ? L.nx : L.nx * L.ny) * support_coord(L, a, base + i - 1);
+        ox[i] = from(o, 0);
+        oy[i] = from(o, 1);
+        oz[i] = from(o, 2);
+    }
+    chain_wait();
+
+    // ---------------- sums: field q, and A by the power of x ----------------
+    const R *mq = mom + q;
+    const R fc = ld_ca(mq + 4 * (size_t)(ox[1] + oy[1] + oz[1]));
+    R b[4] = {R(0), R(0), R(0), R(0)};
+    R C00 = R(0), C10 = R(0), C20 = R(0), C01 = R(0), C11 = R(0), C02 = R(0);  // y and z powers
+#pragma unroll
+    for (int k = 0; k < 3; ++k) {
+        R T0 = R(0), T1 = R(0), T2 = R(0), U0 = R(0), U1 = R(0), U2 = R(0);
+#pragma unroll
+        for (int j = 0; j < 3; ++j) {
+            R F0 = R(0), F1 = R(0), S = R(0);
+#pragma unroll
+            for (int i = 0; i < 3; ++i) {
+                const R f = ld_ca(mq + 4 * (size_t)(ox[i] + oy[j] + oz[k])) - fc;
+                const bool on = (in >> (i + 3 * j + 9 * k)) & 1u;
+                F0 += (on ? wx[i] : R(0)) * f;
+                F1 += (on ? wxd[i] : R(0)) * f;
+                S += on ? wxp[i] : R(0);
+            }
+            T0 += wy[j] * F0;
+            T1 += wy[j] * F1;
+            T2 += wyd[j] * F0;
+            U0 += wy[j] * S;
+            U1 += wyd[j] * S;
+            U2 += wydd[j] * S;
+        }
+        b[0] += wz[k] * T0;
+        b[1] += wz[k] * T1;
+        b[2] += wz[k] * T2;
+        b[3] += wzd[k] * T0;
+        C00 += wz[k] * U0;
+        C10 += wz[k] * U1;
+        C20 += wz[k] * U2;
+        C01 += wzd[k] * U0;
+        C11 += wzd[k] * U1;
+        C02 += wzdd[k] * U0;
+    }
+    const R A[10] = {from(C00, 0), from(C00, 1), from(C10, 0), from(C01, 0), from(C00, 2),
+                     from(C10, 1), from(C01, 1), from(C20, 0), from(C11, 0), from(C02, 0)};
+
+    // ---------------- solve ----------------
+    R Ai[16];
+    if (!spd_inverse4(A, Ai) && p >= 0) atomicCAS(err, 0, -1);
+    const R val = fc + (Ai[3] * b[3] + Ai[2] * b[2] + Ai[1] * b[1] + Ai[0] * b[0]);
+    const int b0 = from(base, 0), b1 = from(base, 1), b2 = from(base, 2);
+    const R x0 = wx[0], x1 = wx[1], x2 = wx[2], y0 = wy[0], y1 = wy[1], y2 = wy[2], z0 = wz[0], z1 = wz[1], z2 = wz[2];
+    if (p >= 0 && !probe) {
+        double *Uo = B.centroid ? B.Uc : B.U;
+        if (q > 0) Uo[3 * p + q - 1] = (double)val;
+        // the transfer record, four values a lane
+        R *rec = (R *)B.phi + (size_t)kRec * p + 4 * q;
+        rec[0] = q == 0 ? Ai[0] : q == 1 ? f0 : q == 2 ? x1 : y2;
+        rec[1] = q == 0 ? Ai[1] : q == 1 ? f1 : q == 2 ? x2 : z0;
+        rec[2] = q == 0 ? Ai[2] : q == 1 ? f2 : q == 2 ? y0 : z1;
+        rec[3] = q == 0 ? Ai[3] : q == 1 ? x0 : q == 2 ? y1 : z2;
+        if (q == 0) reinterpret_cast<int4 *>(B.node)[p] = make_int4(b0, b1, b2, (int)in);
+    }
+    // probes: lane q > 0 has the gradient of velocity component q - 1
+    R g[3];
+#pragma unroll
+    for (int c = 0; c < 3; ++c) {
+        const R *row = Ai + 4 * (c + 1);
+        g[c] = row[0] * b[0] + row[1] * b[1] + row[2] * b[2] + row[3] * b[3];
+    }
+    const R cr = from(val, 0), n0 = from(nrm, 0), n1 = from(nrm, 1), n2 = from(nrm, 2);
+    R acc = g[0] * n0 + g[1] * n1 + g[2] * n2;  // row of the gradient, and below its column
+#pragma unroll
+    for (int c = 0; c < 3; ++c) {
+        const R col = from(g[c], 1) * n0 + from(g[c], 2) * n1 + from(g[c], 3) * n2;
+        if (q == c + 1) acc += col;
+    }
+    const R tr = (R(1) + cr) * pick<R>(L.nu_d, L.nu_f) * acc, pr0 = third(cr);  // p - c_s^2 rho0
+    if (probe && !B.rigid) ((R *)B.probe + 8 * t + 4 * side)[q] = q == 0 ? pr0 : tr;
+    __shared__ double red[6][kQuadThreads / 32];
+    if (B.rigid) {
+        // the probe's side of the stress jump, or the momentum exchange:
+        // component q - 1 of force and moment on lane q > 0
+        const R ar[3] = {from(arm, 0), from(arm, 1), from(arm, 2)};
+        R F = R(0), M = R(0);
+        if (B.rigid_force) {
+            R f6[6] = {R(0), R(0), R(0), R(0), R(0), R(0)};
+            if (probe && side == 0 && q == 0) exchange_force<R>(B, t, area, ar, f6);
+#pragma unroll
+            for (int c = 0; c < 3; ++c) {
+                const R Fc = from(f6[c], 0), Mc = from(f6[3 + c], 0);
+                if (q == c + 1) {
+                    F = Fc;
+                    M = Mc;
+                }
+            }
+        } else {
+            const R nq = q == 1 ? n0 : q == 2 ? n1 : n2;
+            if (probe && q > 0) F = (tr - pr0 * nq) * (side ? -area : area);
+            const R F0 = from(F, 1), F1 = from(F, 2), F2 = from(F, 3);
+            if (q == 1) M = ar[1] * F2 - ar[2] * F1;
+            if (q == 2) M = ar[2] * F0 - ar[0] * F2;
+            if (q == 3) M = ar[0] * F1 - ar[1] * F0;
+        }
+#pragma unroll
+        for (int o = 16; o >= 4; o >>= 1) {
+            F += __shfl_xor_sync(kFull, F, o);
+            M += __shfl_xor_sync(kFull, M, o);
+        }
+        if (lane > 0 && lane < 4) {
+            red[lane - 1][warp] = (double)F;
+            red[lane + 2][warp] = (double)M;
+        }
+    } else {
+#pragma unroll
+        for (int o = 16; o >= 4; o >>= 1) vol += __shfl_xor_sync(kFull, vol, o);
+        if (lane == 0) red[0][warp] = vol;
+    }
+    __syncthreads();
+    if ((int)threadIdx.x < body_sums(B)) {
+        double s = 0.0;
+        for (int k = 0; k < kQuadThreads / 32; ++k) s += red[threadIdx.x][k];
+        B.part[body_sums(B) * vb + threadIdx.x] = s;
+    }
+}
+
 // The blocks take the nvb groups of points in turn (gridDim.x = nvb unless
 // the launch caps the grid).
 template <typename R>
@@ -628,6 +886,16 @@ __global__ void __launch_bounds__(mls_threads(sizeof(R) == 8 ? 0 : 1)) k_mls(con
         // launched programmatically after the moments kernel, whose results
         // it waits for inside
         mls_body<R, true, true>(mom, L, B, err, vb);
+        __syncthreads();  // the next group reuses the shared memory
+    }
+}
+
+template <typename R>
+__global__ void __launch_bounds__(kQuadThreads) k_mls_quad(const R *mom, Lattice L, BodyView B, int *err,
+                                                           int nvb) {
+    chain_release();  // the structure kernel may be scheduled beside this one
+    for (int vb = blockIdx.x; vb < nvb; vb += gridDim.x) {
+        mls_quad_body<R>(mom, L, B, err, vb);
         __syncthreads();  // the next group reuses the shared memory
     }
 }
@@ -683,9 +951,10 @@ __device__ __forceinline__ T lanes_sum(T v) {  // over the 8 lanes of a marker
 constexpr int kDirectParts = 512;
 __device__ __forceinline__ double body_sum(const BodyView &B, int nparts, int q) {
     const int ns = body_sums(B), lane = threadIdx.x & 31;
-    if (nparts > kDirectParts) return __ldcg(B.part + (size_t)ns * nparts + q);
+    const double *part = B.part;
+    if (nparts > kDirectParts) return __ldcg(part + (size_t)ns * nparts + q);
     double s = 0.0;
-    for (int k = lane; k < nparts; k += 32) s += __ldcg(B.part + (size_t)ns * k + q);
+    for (int k = lane; k < nparts; k += 32) s += __ldcg(part + (size_t)ns * k + q);
     return warp_sum(s);
 }
 __device__ __forceinline__ void body_sums_body(const BodyView &B, int nparts) {
@@ -693,8 +962,9 @@ __device__ __forceinline__ void body_sums_body(const BodyView &B, int nparts) {
     __shared__ double red[6][8];
     // every warp takes a share of the partials of all sums
     double s[6] = {0.0, 0.0, 0.0, 0.0, 0.0, 0.0};
+    const double *part = B.part;
     for (int k = threadIdx.x; k < nparts; k += blockDim.x)
-        for (int q = 0; q < ns; ++q) s[q] += __ldcg(B.part + (size_t)ns * k + q);
+        for (int q = 0; q < ns; ++q) s[q] += __ldcg(part + (size_t)ns * k + q);
     for (int q = 0; q < ns; ++q) {
         const double t = warp_sum(s[q]);
         if (lane == 0) red[q][threadIdx.x >> 5] = t;
@@ -982,14 +1252,15 @@ __device__ __forceinline__ void rigid_prepare(const BodyView &B, RigidBlock &r, 
 // The body's sums over the MLS blocks' partials, 16 lanes each.
 __device__ __forceinline__ void rigid_sums(const BodyView &B, RigidBlock &r, const int nparts) {
     const int h = threadIdx.x >> 4, l = threadIdx.x & 15, nh = blockDim.x >> 4;
+    const double *part = B.part;
     for (int q0 = 0; q0 < 6; q0 += nh) {
         const int q = q0 + h;
         double t = 0.0;
         if (q < 6) {
             if (nparts > kDirectParts)
-                t = l == 0 ? __ldcg(B.part + 6 * (size_t)nparts + q) : 0.0;
+                t = l == 0 ? __ldcg(part + 6 * (size_t)nparts + q) : 0.0;
             else
-                for (int k = l; k < nparts; k += 16) t += __ldcg(B.part + 6 * (size_t)k + q);
+                for (int k = l; k < nparts; k += 16) t += __ldcg(part + 6 * (size_t)k + q);
         }
 #pragma unroll
         for (int o = 8; o > 0; o >>= 1) t += __shfl_xor_sync(0xffffffffu, t, o);
@@ -1535,10 +1806,11 @@ static cudaError_t ib_front_t(const void *fin, const Lattice &L, const BodyView 
     if (e != cudaSuccess) return e;
     // the MLS kernel is scheduled while the moments kernel ends, and forms its
     // points' positions and weights meanwhile
-    constexpr int threads = mls_threads(sizeof(R) == 8 ? 0 : 1);
-    const int nvb = mls_blocks(B, threads);
-    return launch_chained(k_mls<R>, dim3(capped(nvb, grid_cap)), dim3(threads), 0, s,
-                          (const R *)mom, L, B, err, nvb);
+    const int prec = sizeof(R) == 8 ? 0 : 1, nvb = mls_blocks(B, mls_points(prec, B));
+    const dim3 g(capped(nvb, grid_cap));
+    if (mls_quads(prec, B))
+        return launch_chained(k_mls_quad<R>, g, dim3(kQuadThreads), 0, s, (const R *)mom, L, B, err, nvb);
+    return launch_chained(k_mls<R>, g, dim3(mls_threads(prec)), 0, s, (const R *)mom, L, B, err, nvb);
 }
 
 cudaError_t launch_ib_front(int prec, const void *fin, const Lattice &L, const BodyView &B, void *mom, int nsm,
@@ -1579,7 +1851,7 @@ static cudaError_t launch_struct(void (*kernel)(KArgs...), bool chained, unsigne
 
 cudaError_t launch_structure(int prec, const Lattice &L, const BodyView &B, void *force, uint32_t *stamp,
                              const uint32_t *step, int nsm, int grid_cap, bool chained, cudaStream_t s) {
-    const int nparts = points_blocks(B, mls_threads(prec));
+    const int nparts = points_blocks(B, mls_points(prec, B));
     cudaError_t e = cudaSuccess;
     if (nparts > kDirectParts) e = launch_struct(k_body_sums, chained, 1, 256, s, B, nparts);
     if (e != cudaSuccess) return e;

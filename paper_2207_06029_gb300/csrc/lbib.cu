@@ -352,7 +352,7 @@ int marker_blocks(int n) { return (n + kMarkersPerBlock - 1) / kMarkersPerBlock;
 
 // Kernels of a body's structure stage.
 int structure_launches(int prec, const BodyView &v) {
-    return 1 + needs_body_sums(v, mls_threads(prec)) + (v.centroid ? 1 : 0);
+    return 1 + needs_body_sums(v, mls_points(prec, v)) + (v.centroid ? 1 : 0);
 }
 
 int check_device_error(Ctx *c) {
@@ -968,9 +968,9 @@ int lbib_add_body(void *h, const double *verts, int nv, const int *tris, int nt,
         upload(c, std::vector<double>((size_t)std::max(mls_blocks(tmp, 32), 6 * ((nt + 255) / 256)), 0.0), &rc);
         upload(c, std::vector<double>(1, 6.0 * V0), &rc);
         b.vol_count = upload(c, std::vector<unsigned int>(1, 0u), &rc);
-        // the MLS blocks' partial sums and, behind them, the sums (of the
-        // one-lattice kernel: the batched ones have fewer)
-        b.part = (double *)dev_alloc(c, sizeof(double) * 6 * (size_t)(mls_blocks(tmp, mls_threads(c->prec)) + 1));
+        // the MLS blocks' partial sums and, behind them, the sums (32
+        // points a block at least)
+        b.part = (double *)dev_alloc(c, sizeof(double) * 6 * (size_t)(mls_blocks(tmp, 32) + 1));
         if (b.part) c->transient.push_back(b.part);
         // per (vertex, hinge) entry: the hinge's vertices and parameters
         std::vector<int4> hv(vh_list.size());

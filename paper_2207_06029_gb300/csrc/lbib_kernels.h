@@ -29,10 +29,19 @@ inline cudaError_t launch_chained(void (*kernel)(KArgs...), dim3 grid, dim3 bloc
 }
 
 constexpr int kNodeThreads = 64;            // threads per block of the support-box kernels (spread over the SMs)
-// MLS points per block of the one-lattice kernel.  FP64 (prec 0) issues one
-// warp instruction per 16 cycles on a whole SM, so its warps go to as many
-// SMs as possible: a warp a block.
+// The one-lattice MLS kernel: four lanes per point, 32 points a block, for few
+// points, else a thread per point.  Four lanes shorten a point's chain of
+// operations but add to their number; in FP64, of which an SM quarter issues
+// a warp instruction per 64 cycles, they pay up to about a warp per quarter
+// (8 points x 608), in FP32 until the warps fill the GPU.  Us a step, four
+// lanes against one: 3 202 points FP64 52.6 against 76.0, FP32 19.3 against 22.0;
+// 12 802 points FP64 295 against 285, FP32 32.8 against 33.6; 51 202 points FP32
+// 309.3 against 303.5.
+inline bool mls_quads(int prec, const BodyView &B) { return B.nm + 2 * B.nt <= (prec == 0 ? 6000 : 20000); }
+// points per block; a thread per point, FP64 takes blocks of one warp, which
+// spread over more SMs
 constexpr int mls_threads(int prec) { return prec == 0 ? 32 : 64; }
+inline int mls_points(int prec, const BodyView &B) { return mls_quads(prec, B) ? 32 : mls_threads(prec); }
 
 // sweep.cu
 // part: 0 the whole lattice, 1 the nodes outside box, 2 the nodes inside box

@@ -1,7 +1,9 @@
-"""MLS points (one thread per marker or probe) against the FP64 oracle where
-the kernel's index arithmetic and support cut-off can go wrong: point counts
-around a warp and a block of 64, bodies across a periodic boundary, and
-markers with support nodes exactly at the cut-off r_k = 1.
+"""MLS points against the FP64 oracle where the kernels' index arithmetic and
+support cut-off can go wrong: point counts around a warp and a block, bodies
+across a periodic boundary, and markers with support nodes exactly at the
+cut-off r_k = 1; in both kernels, four lanes a point (a context alone) and a
+thread a point (a batch).  And the read-back of markers, through the
+page-locked block and, for a body too large for it, by copies.
 
 The tolerances are those of the other parity tests: FP64 1e-12 relative
 (velocities against the flow's scale, at least 1e-2), FP32 1e-5 on
@@ -45,11 +47,12 @@ PLACES = {"inside": (0.13, -0.27, 0.41), "across": (9.6, -10.2, 0.37), "outside"
           "cutoff": (0.3, 0.3, 0.3)}
 
 
+@pytest.mark.parametrize("batched", [False, True])
 @pytest.mark.parametrize("prec", [W.PREC_FP64, W.PREC_FP32])
 @pytest.mark.parametrize("centroid", [0, 1])
 @pytest.mark.parametrize("place", sorted(PLACES))
 @pytest.mark.parametrize("mesh", ["cube", "ico0", "ico1", "ico2"])
-def test_points_match_oracle(lbib, mesh, place, centroid, prec):
+def test_points_match_oracle(lbib, mesh, place, centroid, prec, batched):
     n = (20, 19, 22)
     v, f = meshes()[mesh]
     v = v + (np.array([10.0, 9.0, 11.0]) + np.array(PLACES[place]))[None, :]
@@ -67,7 +70,13 @@ def test_points_match_oracle(lbib, mesh, place, centroid, prec):
                   rho0=rho.ravel(), u0=u.reshape(-1, 3))
     steps = 3
     ctx = lbib.Context.from_case(case)
-    ctx.step(steps)
+    if batched:
+        b = lbib.Batch([ctx])
+        b.step(steps)
+        b.sync()
+        b.close()
+    else:
+        ctx.step(steps)
     s = oracle.Sim(case.n, case.tau, gext=case.gext, bc=case.bc, wall_u=case.wall_u.ravel())
     s.set_fields(*case.initial_fields())
     s.add_body(v, f, **body.kwargs())
@@ -85,3 +94,28 @@ def test_points_match_oracle(lbib, mesh, place, centroid, prec):
         tol = 1e-5 * 1e-2
     for a, b in ((Vg, Vo), (Fg, Fo), (ug, uo), (bg["u"], bo["u"])):
         assert np.abs(np.asarray(a) - np.asarray(b)).max() < tol
+
+
+@pytest.mark.parametrize("level", [2, 6])  # 162 and 40 962 vertices: the block holds 14 500
+def test_read_back_by_block_and_by_copies(lbib, level):
+    """lbib_get_markers and lbib_get_body give the arrays that
+    lbib_get_markers_async queues (the same device memory: equal bits), and
+    the volume and area of those positions."""
+    v, f = W.icosphere(level, 6.0, (12.2, 11.7, 12.4))
+    ctx = lbib.Context((24, 24, 24), 0.8, bc=(0, 0, 1), wall_u=W.shear_walls(0.01))
+    ctx.add_body(v, f, rigid=True, density_ratio=1.1, ref_radius=6.0)
+    ctx.step(3)
+    X, V, F = ctx.markers(0)
+    ref = [np.zeros_like(v) for _ in range(3)]
+    lbib.lbib_get_markers_async(ctx.h, 0, *ref)
+    ctx.sync()
+    for a, b in zip((X, V, F), ref):
+        assert np.array_equal(a, b)
+    only = np.zeros_like(v)
+    lbib.lbib_get_markers(ctx.h, 0, None, only, None)
+    assert np.array_equal(only, V)
+    st = ctx.body(0)
+    a, b, c = (X[f[:, k]] for k in range(3))
+    assert abs(st["volume"] - np.einsum("ij,ij->i", a, np.cross(b, c)).sum() / 6) < 1e-9 * st["volume"]
+    assert abs(st["area"] - 0.5 * np.linalg.norm(np.cross(b - a, c - a), axis=1).sum()) < 1e-9 * st["area"]
+    ctx.close()

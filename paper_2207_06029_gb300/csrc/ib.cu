@@ -1521,8 +1521,11 @@ __global__ void __launch_bounds__(256) kb_moments(BatchTables T, int phase) {
                        vb, nvb);
 }
 
+// Five blocks an SM (102 registers instead of 130 and three blocks): the
+// gathers of many bodies need warps in flight (64 lattices, 618 000 points:
+// 1.091 -> 1.063 ms a step, in spite of 52 spilt bytes).
 template <typename R>
-__global__ void __launch_bounds__(kBatchMlsThreads) kb_mls(BatchTables T, int phase) {
+__global__ void __launch_bounds__(kBatchMlsThreads, sizeof(R) == 4 ? 5 : 2) kb_mls(BatchTables T, int phase) {
     __shared__ Lattice L;
     __shared__ BodyRef br;
     const int j = __ldg(T.mls_blk + blockIdx.x);

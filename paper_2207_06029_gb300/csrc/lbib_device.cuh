@@ -386,7 +386,6 @@ struct BatchTables {
     const int *cen_pre;    // [ncen + 1] blocks of 32 triangles
     const int *sweep_blk, *mom_blk, *mls_blk, *memb_blk, *rm_blk, *cen_blk;  // item of each block
     int sweep_threads;     // threads per sweep block
-    int sweep_cpt;         // cells per sweep thread (blocks per lattice = cells / (threads * cpt))
     int sweep_off32;       // 1: every lattice of the batch has off32 set
 };
 

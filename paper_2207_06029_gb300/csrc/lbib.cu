@@ -1011,9 +1011,20 @@ namespace {
 // 27.7 against 25.2, 80^3 31.0 against 32.0, 96^3 38.4 against 44.5 (16-bit
 // storage and capsules alike); FP64 32^3 78.1 against 76.0, 48^3 109.8 against
 // 125.8.
+//
+// The sweeps of 16-bit storage are bound by instruction issue, so beside
+// them the IB kernels cost what they take, and on large lattices a little
+// more: 160x160x480 sphere FP16 277 against 270, bfloat16 305 against 289 (FP32
+// 305 against 319); 192^3 bfloat16 173 against 166 to 172, FP16 157 against 155
+// to 161; 160^3 bfloat16 95.6 against 94.4.
 constexpr int kSplitCells = 360000, kSplitCells64 = 48000;
+constexpr int kSplitMostFp16 = 8000000, kSplitMostBf16 = 4000000;
 bool splits(const Ctx *c) {
-    return c->bodies.size() == 1 && c->split_sweep && c->L.ncell >= (c->prec == LBIB_FP64 ? kSplitCells64 : kSplitCells);
+    if (c->bodies.size() != 1 || !c->split_sweep) return false;
+    if (c->L.ncell < (c->prec == LBIB_FP64 ? kSplitCells64 : kSplitCells)) return false;
+    if (c->prec == LBIB_FP16_DEV) return c->L.ncell <= kSplitMostFp16;
+    if (c->prec == LBIB_BF16_DEV) return c->L.ncell <= kSplitMostBf16;
+    return true;
 }
 
 // Enqueues one step on the two step streams (the caller forks them from,

@@ -49,6 +49,16 @@ struct DevBody {
     double V0 = 0, A0 = 0, mv = 0, origin[3] = {0, 0, 0};
 };
 
+// Where a recorded trajectory goes (lbib_step_markers): staging planes, their
+// size, the doubles of one step, the step count before the first slot, which
+// arrays are wanted (X 1, U_b 2, F_l 4).
+struct Record {
+    double *dst;
+    long long plane, n3;
+    uint32_t step0;
+    int want;
+};
+
 // Size of a context's page-locked block: allocating one takes about 115 us
 // whatever its size up to 1 MiB, which holds the markers of a body of 14 500
 // vertices.
@@ -106,6 +116,11 @@ struct Ctx {
     std::vector<std::pair<void *, size_t>> allocs;
     double *mstage = nullptr;  // lbib_step_markers: device staging of the recorded markers
     size_t mstage_bytes = 0;
+    // six steps from phase 0, each followed by the staging of record_body's
+    // markers as *d_rec says
+    cudaGraphExec_t gexec6r = nullptr;
+    int record_body = -1;
+    Record *d_rec = nullptr;
     std::vector<void *> transient;  // allocations a checkpoint leaves out (scratch, support moments)
     bool profile = false;
     std::vector<cudaEvent_t> events;  // per step: begin, after MLS, after structure, after sweep
@@ -621,6 +636,7 @@ void lbib_destroy(void *h) {
         if (st) cudaStreamSynchronize(st);
     for (auto ev : c->events) cudaEventDestroy(ev);
     if (c->gexec6) cudaGraphExecDestroy(c->gexec6);
+    if (c->gexec6r) cudaGraphExecDestroy(c->gexec6r);
     for (int k = 0; k < 6; ++k) {
         if (c->gexec[k]) cudaGraphExecDestroy(c->gexec[k]);
         if (c->gstore[k]) cudaGraphExecDestroy(c->gstore[k]);
@@ -1133,7 +1149,8 @@ void invalidate_graphs(Ctx *c) {
         c->stored[k] = false;
     }
     if (c->gexec6) cudaGraphExecDestroy(c->gexec6);
-    c->gexec6 = nullptr;
+    if (c->gexec6r) cudaGraphExecDestroy(c->gexec6r);
+    c->gexec6 = c->gexec6r = nullptr;
     c->graph_origin = c->steps;
 }
 
@@ -1146,10 +1163,35 @@ void rotate(Ctx *c, int n) {
     }
 }
 
+// The step's markers of one body into their slot of the staging planes (X,
+// U_b, F_l): the slot of the step counter, or given (slot >= 0).
+__global__ void k_stage_markers(const double *__restrict__ X, const double *__restrict__ Ub,
+                                const double *__restrict__ Fl, const Record *__restrict__ rec,
+                                const uint32_t *__restrict__ dstep, int slot) {
+    const Record r = *rec;
+    double *dst = r.dst + (slot >= 0 ? slot : (long long)(uint32_t)(*dstep - r.step0 - 1u)) * r.n3;
+    for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < r.n3; i += (long long)gridDim.x * blockDim.x) {
+        if (r.want & 1) dst[i] = X[i];
+        if (r.want & 2) dst[r.plane + i] = Ub[i];
+        if (r.want & 4) dst[2 * r.plane + i] = Fl[i];
+    }
+}
+__global__ void k_set_record(Record *rec, Record r) { *rec = r; }
+__global__ void k_record_base(Record *rec, uint32_t step0) { rec->step0 = step0; }
+
+cudaError_t stage_markers(Ctx *c, int body, int slot, cudaStream_t st) {
+    const DevBody &b = c->bodies[body];
+    const size_t n3 = 3 * (size_t)b.nv;
+    k_stage_markers<<<(unsigned)std::min<size_t>((n3 + 255) / 256, 1024), 256, 0, st>>>(b.X[b.cur], b.Ub, b.Fl, c->d_rec,
+                                                                                       c->d_step, slot);
+    return cudaGetLastError();
+}
+
 // Captures the next nsteps steps (1 or 6) as a CUDA graph on the capture
 // stream; the host state is left as it was.  store: the step stores the
-// fields; k: the phase (timing events).
-int build_graph(Ctx *c, int nsteps, bool store, int k, cudaGraphExec_t *out) {
+// fields; k: the phase (timing events); record >= 0: every step is followed by
+// the staging of that body's markers.
+int build_graph(Ctx *c, int nsteps, bool store, int k, int record, cudaGraphExec_t *out) {
     cudaError_t e = cudaStreamBeginCapture(c->s_cap, cudaStreamCaptureModeThreadLocal);
     if (e != cudaSuccess) return cuda_fail(c, e, "graph capture");
     cudaEventRecord(c->ev_fork, c->s_cap);
@@ -1157,8 +1199,11 @@ int build_graph(Ctx *c, int nsteps, bool store, int k, cudaGraphExec_t *out) {
     cudaStreamWaitEvent(c->s_lo, c->ev_fork, 0);
     const long long launches = c->launches;
     int rc = LBIB_OK, done = 0;
-    for (; done < nsteps && rc == LBIB_OK; ++done)
+    for (; done < nsteps && rc == LBIB_OK; ++done) {
         rc = enqueue_step(c, store, c->profile ? c->gev[k] : nullptr, true, (int)((c->steps + done) & 1));
+        if (rc == LBIB_OK && record >= 0 && (e = stage_markers(c, record, -1, c->s_hi)) != cudaSuccess)
+            rc = cuda_fail(c, e, "marker staging");
+    }
     if (rc) --done;                      // a failed step has not rotated
     rotate(c, (6 - done % 6) % 6);       // six steps return the rotation to where it started
     c->launches = launches;
@@ -1205,8 +1250,9 @@ int plain_steps(const Ctx *c, int n, bool end_of_call) {
 }
 
 // nsteps steps; with fields_every = 0 the fields are stored on the last of
-// them when end_of_call (the last step of a public call)
-int step_steps(Ctx *c, int nsteps, bool end_of_call) {
+// them when end_of_call (the last step of a public call).  record >= 0: after
+// every step the markers of that body are staged as *d_rec says.
+int step_steps(Ctx *c, int nsteps, bool end_of_call, int record = -1) {
     if (!c) return LBIB_EINVAL;
     if (c->err) return c->err;
     if (nsteps < 0) return fail(c, LBIB_EINVAL, "nsteps < 0");
@@ -1221,6 +1267,11 @@ int step_steps(Ctx *c, int nsteps, bool end_of_call) {
         e = cudaMemsetAsync(c->d_tot, 0, sizeof(double) * (size_t)totals_scratch_doubles(), c->stream);
             if (e != cudaSuccess) return cuda_fail(c, e, "step counter reset");
             c->step_host = 1;
+            if (record >= 0) {  // slots count from the restarted counter on
+                k_record_base<<<1, 1, 0, c->stream>>>(c->d_rec, 0u - (uint32_t)it);
+                if ((e = cudaGetLastError()) != cudaSuccess) return cuda_fail(c, e, "marker staging");
+                c->launches++;
+            }
         }
         const bool store = c->fields_every == 0 ? (end_of_call && it == nsteps - 1)
                                                 : (c->fields_every > 0 && (c->steps + 1) % c->fields_every == 0);
@@ -1229,15 +1280,16 @@ int step_steps(Ctx *c, int nsteps, bool end_of_call) {
             c->graphs_timed = c->profile;
         }
         const int k = (int)(((c->steps - c->graph_origin) % 6 + 6) % 6);
+        bool staged = false;  // the graph staged the markers itself
         if (c->use_graphs && (!store || (c->stored[k] && !c->profile))) {
             // six steps at once where none of them stores the fields, is
             // timed, restarts the step counter or (but for the last) precedes
             // a watchdog check: the gap between two graph launches (4 to 5 us)
             // is paid once for the six
             const bool six = k == 0 && !store && !c->profile && plain_steps(c, nsteps - it, end_of_call) >= 6;
-            cudaGraphExec_t *g = six ? &c->gexec6 : store ? &c->gstore[k] : &c->gexec[k];
+            cudaGraphExec_t *g = six ? (record >= 0 ? &c->gexec6r : &c->gexec6) : store ? &c->gstore[k] : &c->gexec[k];
             if (!*g) {
-                int rc = build_graph(c, six ? 6 : 1, store, k, g);
+                int rc = build_graph(c, six ? 6 : 1, store, k, six ? record : -1, g);
                 if (rc) return rc;
             }
             harvest_graph_events(c, k);
@@ -1245,6 +1297,7 @@ int step_steps(Ctx *c, int nsteps, bool end_of_call) {
             if (e != cudaSuccess) return cuda_fail(c, e, "graph launch");
             if (c->profile) c->gev_pending[k] = true;
             if (six) {
+                staged = record >= 0;
                 if (!c->bodies.empty()) c->step_host += 5;
                 c->steps += 5;
                 it += 5;
@@ -1273,6 +1326,11 @@ int step_steps(Ctx *c, int nsteps, bool end_of_call) {
             cudaEventRecord(c->ev_join, c->s_hi);
             cudaStreamWaitEvent(c->stream, c->ev_join, 0);
         }
+        if (record >= 0 && !staged) {
+            cudaError_t e = stage_markers(c, record, it, c->stream);
+            if (e != cudaSuccess) return cuda_fail(c, e, "marker staging");
+        }
+        if (record >= 0) c->launches += staged ? 6 : 1;
         c->steps++;
         if (c->watch_every > 0 && c->steps % c->watch_every == 0) {
             int rc = enqueue_watch(c, c->stream);
@@ -1393,17 +1451,6 @@ int lbib_get_markers_async(void *h, int body, double *X, double *V, double *F) {
     return LBIB_OK;
 }
 
-// Step k's markers into slot k of the staging planes (X, U_b, F_l).
-__global__ void k_stage_markers(const double *__restrict__ X, const double *__restrict__ Ub,
-                                const double *__restrict__ Fl, double *__restrict__ dst, long long n3,
-                                long long plane, int slot) {
-    for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < n3; i += (long long)gridDim.x * blockDim.x) {
-        if (X) dst[slot * n3 + i] = X[i];
-        if (Ub) dst[plane + slot * n3 + i] = Ub[i];
-        if (Fl) dst[2 * plane + slot * n3 + i] = Fl[i];
-    }
-}
-
 int lbib_step_markers(void *h, int nsteps, int body, double *X, double *V, double *F) {
     Ctx *c = as_ctx(h);
     if (!c || nsteps < 0) return LBIB_EINVAL;
@@ -1425,22 +1472,24 @@ int lbib_step_markers(void *h, int nsteps, int body, double *X, double *V, doubl
         if (!c->mstage) return fail(c, LBIB_ENOMEM, "marker staging buffer of %zu bytes", need);
         c->mstage_bytes = need;
     }
-    // each step's markers go to the staging planes on the device (one small
-    // kernel behind the step); the host copies follow the last step, one
-    // per requested array
-    const int blocks = (int)std::min<size_t>((n3 + 255) / 256, 1024);
-    for (int k = 0; k < nsteps; ++k) {
-        // one step at a time, the fields stored as lbib_step(h, nsteps) would
-        int rc = step_steps(c, 1, k == nsteps - 1);
-        if (rc) return rc;
-        DevBody &b = c->bodies[body];
-        k_stage_markers<<<blocks, 256, 0, c->stream>>>(X ? b.X[b.cur] : nullptr, V ? b.Ub : nullptr,
-                                                       F ? b.Fl : nullptr, c->mstage, (long long)n3,
-                                                       (long long)plane, k);
-        cudaError_t e = cudaGetLastError();
-        if (e != cudaSuccess) return cuda_fail(c, e, "marker staging");
-        c->launches++;
+    if (!c->d_rec) {
+        c->d_rec = static_cast<Record *>(dev_alloc(c, sizeof(Record)));
+        if (!c->d_rec) return fail(c, LBIB_ENOMEM, "marker staging");
+        c->transient.push_back(c->d_rec);
     }
+    if (c->record_body != body) {  // the graph holds the body's buffers
+        if (c->gexec6r) cudaGraphExecDestroy(c->gexec6r);
+        c->gexec6r = nullptr;
+        c->record_body = body;
+    }
+    // each step's markers go to the staging planes on the device (one small
+    // kernel behind the step, in the six-step graph with it); the host copies
+    // follow the last step, one per requested array
+    const Record r{c->mstage, (long long)plane, (long long)n3, c->step_host, (X ? 1 : 0) | (V ? 2 : 0) | (F ? 4 : 0)};
+    k_set_record<<<1, 1, 0, c->stream>>>(c->d_rec, r);
+    if (cudaError_t e0 = cudaGetLastError(); e0 != cudaSuccess) return cuda_fail(c, e0, "marker staging");
+    c->launches++;
+    if (int rc = step_steps(c, nsteps, true, body)) return rc;
     const size_t bytes = plane * sizeof(double);
     cudaError_t e = cudaSuccess;
     if (X) e = cudaMemcpyAsync(X, c->mstage, bytes, cudaMemcpyDeviceToHost, c->stream);

@@ -94,6 +94,24 @@ constexpr int kLineThreads = 128;
 static bool line_sweep(const Lattice &L, int part) {
     return L.sweep_bx == 0 && ((L.nx & 31) != 0 || (part != 1 && L.ncell < (1 << 20)));
 }
+// FP64: an SM quarter issues one double-precision instruction of a warp every
+// 64 cycles, so a small lattice takes as long as the quarter with the most
+// warps.  Up to kOneWarpRounds warps a quarter the blocks are of one warp,
+// which spread evenly (walls all round, against 128 threads: 24x28x30 33.4 ->
+// 21.8 us, 40x24x27 31.6 -> 23.9, 45x33x30 37.7 -> 34.4, 48^3 67.9 and 68.3);
+// and where single rows give no quarter more warps, one row a block, whose
+// walls along y and z are whole warps (24^3 19.4 -> 17.1, 31x45x50 47.3 ->
+// 44.6; 24x40x40, a third round, 29.7 against 34.4).
+constexpr int kOneWarpRounds = 4;
+struct SmallSweep {
+    bool rows;
+    int threads;
+};
+static SmallSweep small_sweep64(const Lattice &L, int nsm) {
+    const long long quarters = 4LL * nsm, line = (L.ncell + 31LL) / 32, rows = (L.nx + 31LL) / 32 * L.ny * L.nz;
+    if ((line + quarters - 1) / quarters > kOneWarpRounds) return {false, kLineThreads};
+    return {L.nx < 256 && (rows + quarters - 1) / quarters == (line + quarters - 1) / quarters, 32};
+}
 template <typename S, typename R, bool kOff32>
 __global__ void __launch_bounds__(kLineThreads) k_sweep_line(const S *__restrict__ fin, S *__restrict__ fout,
                                                              R *__restrict__ force,
@@ -104,7 +122,7 @@ __global__ void __launch_bounds__(kLineThreads) k_sweep_line(const S *__restrict
     const uint32_t step = stamp ? *dstep : 0u;
     const uint32_t seed = sr[parity];
     if (blockIdx.x == 0 && threadIdx.x == 0) sr[parity ^ 1] = seed + 1u;
-    const int c = blockIdx.x * kLineThreads + threadIdx.x;
+    const int c = blockIdx.x * blockDim.x + threadIdx.x;
     if (c >= L.ncell) return;
     int x, y, z;
     node_coords(L, c, x, y, z);
@@ -418,8 +436,14 @@ static cudaError_t sweep_t(const void *fin, void *fout, void *force, const uint3
                                                                L, (R *)fields, box, sr, parity, (int)grid.x,
                                                                (int)grid.y);
     } else if (line_sweep(L, part)) {
-        k_sweep_line<S, R, kOff32><<<grid_for(L.ncell, kLineThreads), kLineThreads, 0, s>>>(
-            (const S *)fin, (S *)fout, (R *)force, stamp, step, L, (R *)fields, part == 1 ? box : nullptr, sr, parity);
+        const SmallSweep m = sizeof(R) == 8 && part == 0 ? small_sweep64(L, nsm) : SmallSweep{false, kLineThreads};
+        if (m.rows)
+            k_sweep<S, R, kOff32><<<dim3(1, L.ny, L.nz), (L.nx + 31) / 32 * 32, 0, s>>>(
+                (const S *)fin, (S *)fout, (R *)force, stamp, step, L, (R *)fields, nullptr, sr, parity);
+        else
+            k_sweep_line<S, R, kOff32><<<grid_for(L.ncell, m.threads), m.threads, 0, s>>>(
+                (const S *)fin, (S *)fout, (R *)force, stamp, step, L, (R *)fields, part == 1 ? box : nullptr, sr,
+                parity);
     } else {
         dim3 grid, block;
         sweep_shape(L, grid, block);

@@ -282,8 +282,9 @@ int lbib_get_launch_config(void *ctx, int *cfg);
 /* With a single body, the sweep of the nodes outside the body's support
  * box runs on a second stream concurrently with the IB stage (default 1);
  * 0 runs one whole-lattice sweep after the IB stage, as small lattices
- * (below 360 000 nodes, 48 000 in FP64) do either way.  Results are the same
- * either way. */
+ * (below 360 000 nodes, 48 000 in FP64) and large ones in 16-bit storage
+ * (above 8 000 000 nodes in FP16, 4 000 000 in bfloat16) do either way.
+ * Results are the same either way. */
 int lbib_set_overlap(void *ctx, int enable);
 
 /* Steps that do not store the fields run as CUDA graphs captured on first

@@ -215,8 +215,8 @@ int lbib_get_markers_async(void *ctx, int body, double *X, double *V, double *F)
  * after each step k into X + 3 nv k, V + 3 nv k and F + 3 nv k (host arrays
  * of nsteps * 3 * nv doubles; any may be NULL): a trajectory recorded
  * without a host round trip per step.  Each step's markers are staged on the
- * device by one small kernel queued behind the step (in a context-owned
- * buffer of 3 * nsteps * 3 nv doubles, kept for later calls and grown when
+ * device, by the step's structure kernel or one small kernel behind the
+ * step (in a context-owned buffer of 3 * nsteps * 3 nv doubles, kept for later calls and grown when
  * needed); the device-to-host copies, one per requested array, are queued
  * after the last step.  The fields are stored as lbib_step(ctx, nsteps)
  * stores them (lbib_set_output), and steps that store none run from the

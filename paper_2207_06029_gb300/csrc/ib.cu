@@ -1174,6 +1174,9 @@ __device__ __forceinline__ void membrane_body(const Lattice &L, const BodyView &
         if constexpr (sizeof(R) == 4) B.Xlo_next[3 * vj + a] = float(rel - double(float(rel)));
         B.Ub[3 * vj + a] = Ub;
         B.Fl[3 * vj + a] = Fla;
+        record(B.rec, step, 0, 3 * vj + a, xn);
+        record(B.rec, step, 1, 3 * vj + a, Ub);
+        record(B.rec, step, 2, 3 * vj + a, Fla);
         sbox.add(a, xn);
         s_Fl[j][a] = R(Fla);
     }
@@ -1423,6 +1426,8 @@ __device__ __forceinline__ void rigid_markers_body(const Lattice &L, const BodyV
             const double Fla = ub - U;
             B.Ub[3 * vj + a] = ub;
             B.Fl[3 * vj + a] = Fla;
+            record(B.rec, step, 1, 3 * vj + a, ub);
+            record(B.rec, step, 2, 3 * vj + a, Fla);
             s_Fl[j][a] = R(Fla);
         } else if (first && warp == 0) {
             rigid_orientation(r, lane);
@@ -1436,6 +1441,7 @@ __device__ __forceinline__ void rigid_markers_body(const Lattice &L, const BodyV
             // has diverged
             if (!(fabs(xn - x[0]) < kMaxMarkerStep)) atomicCAS(B.err, 0, kErrDiverged);
             B.Xnew[3 * vj + a] = xn;
+            record(B.rec, step, 0, 3 * vj + a, xn);
             ((R *)B.Xrel_next)[3 * vj + a] = R(xn - B.origin[a]);
             sbox.add(a, xn);
         }

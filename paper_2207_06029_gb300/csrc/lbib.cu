@@ -49,16 +49,6 @@ struct DevBody {
     double V0 = 0, A0 = 0, mv = 0, origin[3] = {0, 0, 0};
 };
 
-// Where a recorded trajectory goes (lbib_step_markers): staging planes, their
-// size, the doubles of one step, the step count before the first slot, which
-// arrays are wanted (X 1, U_b 2, F_l 4).
-struct Record {
-    double *dst;
-    long long plane, n3;
-    uint32_t step0;
-    int want;
-};
-
 // Size of a context's page-locked block: allocating one takes about 115 us
 // whatever its size up to 1 MiB, which holds the markers of a body of 14 500
 // vertices.
@@ -116,8 +106,8 @@ struct Ctx {
     std::vector<std::pair<void *, size_t>> allocs;
     double *mstage = nullptr;  // lbib_step_markers: device staging of the recorded markers
     size_t mstage_bytes = 0;
-    // six steps from phase 0, each followed by the staging of record_body's
-    // markers as *d_rec says
+    // six steps from phase 0, whose structure kernels also write record_body's
+    // markers where *d_rec says
     cudaGraphExec_t gexec6r = nullptr;
     int record_body = -1;
     Record *d_rec = nullptr;
@@ -1051,7 +1041,7 @@ bool splits(const Ctx *c) {
 // swept after the spreading.  ev (6 events or nullptr) receives the stage
 // timestamps; `external` records them as graph nodes during capture.
 // Advances the host-side buffer rotation but not the step count.
-int enqueue_step(Ctx *c, bool store_fields, cudaEvent_t *ev, bool external, int parity) {
+int enqueue_step(Ctx *c, bool store_fields, cudaEvent_t *ev, bool external, int parity, int record = -1) {
     const bool split = splits(c);
     cudaStream_t hi = c->s_hi, lo = c->s_lo;
     auto rec = [&](int k, cudaStream_t st) {
@@ -1084,7 +1074,8 @@ int enqueue_step(Ctx *c, bool store_fields, cudaEvent_t *ev, bool external, int 
     rec(1, hi);
     // structure update and spreading
     for (auto &b : c->bodies) {
-        const BodyView v = make_view(c, b);
+        BodyView v = make_view(c, b);
+        if (record >= 0 && &b == &c->bodies[record]) v.rec = c->d_rec;
         // programmatically behind the MLS kernel (or the body before), unless
         // a timing event stands between them
         const cudaError_t e = launch_structure(c->prec, c->L, v, c->force, c->stamp, c->d_step, c->nsm,
@@ -1163,13 +1154,12 @@ void rotate(Ctx *c, int n) {
     }
 }
 
-// The step's markers of one body into their slot of the staging planes (X,
-// U_b, F_l): the slot of the step counter, or given (slot >= 0).
+// The markers of one body into slot `slot` of the staging planes, behind a
+// step that ran from no six-step graph.
 __global__ void k_stage_markers(const double *__restrict__ X, const double *__restrict__ Ub,
-                                const double *__restrict__ Fl, const Record *__restrict__ rec,
-                                const uint32_t *__restrict__ dstep, int slot) {
+                                const double *__restrict__ Fl, const Record *__restrict__ rec, int slot) {
     const Record r = *rec;
-    double *dst = r.dst + (slot >= 0 ? slot : (long long)(uint32_t)(*dstep - r.step0 - 1u)) * r.n3;
+    double *dst = r.dst + slot * r.n3;
     for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < r.n3; i += (long long)gridDim.x * blockDim.x) {
         if (r.want & 1) dst[i] = X[i];
         if (r.want & 2) dst[r.plane + i] = Ub[i];
@@ -1182,15 +1172,14 @@ __global__ void k_record_base(Record *rec, uint32_t step0) { rec->step0 = step0;
 cudaError_t stage_markers(Ctx *c, int body, int slot, cudaStream_t st) {
     const DevBody &b = c->bodies[body];
     const size_t n3 = 3 * (size_t)b.nv;
-    k_stage_markers<<<(unsigned)std::min<size_t>((n3 + 255) / 256, 1024), 256, 0, st>>>(b.X[b.cur], b.Ub, b.Fl, c->d_rec,
-                                                                                       c->d_step, slot);
+    k_stage_markers<<<(unsigned)std::min<size_t>((n3 + 255) / 256, 1024), 256, 0, st>>>(b.X[b.cur], b.Ub, b.Fl, c->d_rec, slot);
     return cudaGetLastError();
 }
 
 // Captures the next nsteps steps (1 or 6) as a CUDA graph on the capture
 // stream; the host state is left as it was.  store: the step stores the
-// fields; k: the phase (timing events); record >= 0: every step is followed by
-// the staging of that body's markers.
+// fields; k: the phase (timing events); record >= 0: the structure kernels
+// also write that body's markers where *d_rec says.
 int build_graph(Ctx *c, int nsteps, bool store, int k, int record, cudaGraphExec_t *out) {
     cudaError_t e = cudaStreamBeginCapture(c->s_cap, cudaStreamCaptureModeThreadLocal);
     if (e != cudaSuccess) return cuda_fail(c, e, "graph capture");
@@ -1199,11 +1188,8 @@ int build_graph(Ctx *c, int nsteps, bool store, int k, int record, cudaGraphExec
     cudaStreamWaitEvent(c->s_lo, c->ev_fork, 0);
     const long long launches = c->launches;
     int rc = LBIB_OK, done = 0;
-    for (; done < nsteps && rc == LBIB_OK; ++done) {
-        rc = enqueue_step(c, store, c->profile ? c->gev[k] : nullptr, true, (int)((c->steps + done) & 1));
-        if (rc == LBIB_OK && record >= 0 && (e = stage_markers(c, record, -1, c->s_hi)) != cudaSuccess)
-            rc = cuda_fail(c, e, "marker staging");
-    }
+    for (; done < nsteps && rc == LBIB_OK; ++done)
+        rc = enqueue_step(c, store, c->profile ? c->gev[k] : nullptr, true, (int)((c->steps + done) & 1), record);
     if (rc) --done;                      // a failed step has not rotated
     rotate(c, (6 - done % 6) % 6);       // six steps return the rotation to where it started
     c->launches = launches;
@@ -1250,8 +1236,8 @@ int plain_steps(const Ctx *c, int n, bool end_of_call) {
 }
 
 // nsteps steps; with fields_every = 0 the fields are stored on the last of
-// them when end_of_call (the last step of a public call).  record >= 0: after
-// every step the markers of that body are staged as *d_rec says.
+// them when end_of_call (the last step of a public call).  record >= 0: every
+// step's markers of that body go where *d_rec says.
 int step_steps(Ctx *c, int nsteps, bool end_of_call, int record = -1) {
     if (!c) return LBIB_EINVAL;
     if (c->err) return c->err;
@@ -1280,7 +1266,7 @@ int step_steps(Ctx *c, int nsteps, bool end_of_call, int record = -1) {
             c->graphs_timed = c->profile;
         }
         const int k = (int)(((c->steps - c->graph_origin) % 6 + 6) % 6);
-        bool staged = false;  // the graph staged the markers itself
+        bool staged = false;  // the graph wrote the markers to the staging planes itself
         if (c->use_graphs && (!store || (c->stored[k] && !c->profile))) {
             // six steps at once where none of them stores the fields, is
             // timed, restarts the step counter or (but for the last) precedes
@@ -1330,7 +1316,7 @@ int step_steps(Ctx *c, int nsteps, bool end_of_call, int record = -1) {
             cudaError_t e = stage_markers(c, record, it, c->stream);
             if (e != cudaSuccess) return cuda_fail(c, e, "marker staging");
         }
-        if (record >= 0) c->launches += staged ? 6 : 1;
+        if (record >= 0 && !staged) c->launches++;
         c->steps++;
         if (c->watch_every > 0 && c->steps % c->watch_every == 0) {
             int rc = enqueue_watch(c, c->stream);
@@ -1482,9 +1468,11 @@ int lbib_step_markers(void *h, int nsteps, int body, double *X, double *V, doubl
         c->gexec6r = nullptr;
         c->record_body = body;
     }
-    // each step's markers go to the staging planes on the device (one small
-    // kernel behind the step, in the six-step graph with it); the host copies
-    // follow the last step, one per requested array
+    // each step's markers go to the staging planes on the device, written by
+    // the structure kernel in the six-step graph (a staging kernel a step
+    // before: 64^3 capsule, 40 steps 1114 -> 1062 us) and by a small kernel
+    // behind any other step; the host copies follow the last step, one per
+    // requested array
     const Record r{c->mstage, (long long)plane, (long long)n3, c->step_host, (X ? 1 : 0) | (V ? 2 : 0) | (F ? 4 : 0)};
     k_set_record<<<1, 1, 0, c->stream>>>(c->d_rec, r);
     if (cudaError_t e0 = cudaGetLastError(); e0 != cudaSuccess) return cuda_fail(c, e0, "marker staging");

@@ -329,7 +329,23 @@ struct BodyView {
     double *part;           // per MLS block: partial volume (membranes) or force and moment (rigid, 6); then the sums
     unsigned int *vol_count; // rigid: blocks of the marker kernel that have read the old state
     int *err;               // device error word of the context (first error wins)
+    const struct Record *rec;  // where the structure kernel also writes the markers, or null
 };
+
+// Where a recorded trajectory goes (lbib_step_markers): staging planes of X,
+// U_b and F_l, their size, the doubles of one step, the step count before the
+// first slot, which arrays are wanted (X 1, U_b 2, F_l 4).
+struct Record {
+    double *dst;
+    long long plane, n3;
+    uint32_t step0;
+    int want;
+};
+// Coordinate i of array q (0 X, 1 U_b, 2 F_l) into the slot of the step.
+__device__ __forceinline__ void record(const Record *rec, uint32_t step, int q, int i, double value) {
+    if (rec && (rec->want >> q & 1))
+        rec->dst[q * rec->plane + (long long)(uint32_t)(step - rec->step0 - 1u) * rec->n3 + i] = value;
+}
 
 // Blocks of `threads` MLS points (markers, then two probes per triangle).
 __host__ __device__ inline int points_blocks(const BodyView &B, int threads) {

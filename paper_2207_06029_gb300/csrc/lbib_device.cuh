@@ -137,7 +137,7 @@ struct Pop<double, double> {
     // raw: the stored value itself (the deviation times 2^kScaleLog2)
     static constexpr int kScaleLog2 = 0;
     __device__ static double ld_raw(const double *p) { return __ldg(p); }
-    __device__ static void st_raw(double *p, double v) { __stcs(p, v); }
+    __device__ static void st_raw(double *p, double v) { *p = v; }
     __device__ static double from_raw(double v) { return v; }
     __device__ static double to_raw(double v) { return v; }
 };
@@ -149,7 +149,7 @@ struct Pop<float, float> {
     __device__ static float to(float v) { return v; }
     static constexpr int kScaleLog2 = 0;
     __device__ static float ld_raw(const float *p) { return __ldg(p); }
-    __device__ static void st_raw(float *p, float v) { __stcs(p, v); }
+    __device__ static void st_raw(float *p, float v) { *p = v; }
     __device__ static float from_raw(float v) { return v; }
     __device__ static float to_raw(float v) { return v; }
 };

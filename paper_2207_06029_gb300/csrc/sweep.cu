@@ -58,26 +58,50 @@ __device__ __forceinline__ bool in_box(const Lattice &L, const int *lo, const in
 // Whole lattice (box == nullptr), or every node outside the box.
 // sr: the two-word rounding-seed counter of the lattice; a step reads word
 // `parity` and advances the other one (parity alternates with the steps).
-template <typename S, typename R, bool kOff32>
+// flip (FP32): blocks from the last plane to the first; kStream: see sweep_reuse.
+template <typename S, typename R, bool kOff32, bool kStream>
 __global__ void __launch_bounds__(256) k_sweep(const S *__restrict__ fin, S *__restrict__ fout,
                                                R *__restrict__ force, const uint32_t *__restrict__ stamp,
                                                const uint32_t *__restrict__ dstep, Lattice L,
                                                R *__restrict__ fields, const int *__restrict__ box,
-                                               uint32_t *__restrict__ sr, int parity) {
+                                               uint32_t *__restrict__ sr, int parity, int flip) {
     const uint32_t step = stamp ? *dstep : 0u;
     const uint32_t seed = sr[parity];
     if (blockIdx.x == 0 && blockIdx.y == 0 && blockIdx.z == 0 && threadIdx.x == 0 && threadIdx.y == 0)
         sr[parity ^ 1] = seed + 1u;
     const int x = blockIdx.x * blockDim.x + threadIdx.x;
-    const int y = blockIdx.y * blockDim.y + threadIdx.y;
-    const int z = blockIdx.z;
+    const bool back = sizeof(S) == 4 && flip;
+    const int y = (back ? gridDim.y - 1 - blockIdx.y : blockIdx.y) * blockDim.y + threadIdx.y;
+    const int z = back ? gridDim.z - 1 - blockIdx.z : blockIdx.z;
     if (x >= L.nx || y >= L.ny) return;
     if (box) {
         int lo[3], ext[3];
         clamp_box(L, box, lo, ext);
         if (in_box(L, lo, ext, x, y, z)) return;
     }
-    sweep_cell<S, R, kOff32>(fin, fout, force, stamp, step, L, fields, x, y, z, seed);
+    sweep_cell<S, R, kOff32, false, kStream>(fin, fout, force, stamp, step, L, fields, x, y, z, seed);
+}
+
+// What of a step's output the L2 (129 MB) still holds when the next step
+// begins: alternate steps run through the lattice from its end (flip), so
+// that a step begins with what the one before wrote last, and on lattices
+// that are not much larger than the L2 the populations it reads, each once,
+// make room first (kStream; stores stay in the L2).  FP32, neither, flip
+// alone, both: 80^3 10.4, 10.6, 10.0 us; 96^3 20.9, 19.4, 17.0 (7.9 TB/s);
+// 128^3 49.1, 46.1, 45.0; 137x141x139 62.4, 59.6, 60.4; 176^3 122.9, 121.0,
+// 125.7; 160x160x480 280.5, 278.6, 288.2.  Below kReuseCells both buffers stay
+// in the L2 as they are (75x67x81 8.0 us in every form).  16-bit storage (issue
+// bound) loses what the flip's instructions cost (96^3 15.75, 16.08) and FP64
+// gains 0.5 %: neither has it.
+constexpr int kReuseCells = 450000, kStreamCells = 2400000;
+struct SweepReuse {
+    int flip;
+    bool stream;
+};
+template <typename S>
+static SweepReuse sweep_reuse(const Lattice &L, int parity) {
+    if (sizeof(S) != 4 || L.ncell < kReuseCells) return {0, false};
+    return {parity, L.ncell <= kStreamCells};
 }
 
 // The same over consecutive nodes, whatever the rows: for row lengths that
@@ -112,17 +136,17 @@ static SmallSweep small_sweep64(const Lattice &L, int nsm) {
     if ((line + quarters - 1) / quarters > kOneWarpRounds) return {false, kLineThreads};
     return {L.nx < 256 && (rows + quarters - 1) / quarters == (line + quarters - 1) / quarters, 32};
 }
-template <typename S, typename R, bool kOff32>
+template <typename S, typename R, bool kOff32, bool kStream>
 __global__ void __launch_bounds__(kLineThreads) k_sweep_line(const S *__restrict__ fin, S *__restrict__ fout,
                                                              R *__restrict__ force,
                                                              const uint32_t *__restrict__ stamp,
                                                              const uint32_t *__restrict__ dstep, Lattice L,
                                                              R *__restrict__ fields, const int *__restrict__ box,
-                                                             uint32_t *__restrict__ sr, int parity) {
+                                                             uint32_t *__restrict__ sr, int parity, int flip) {
     const uint32_t step = stamp ? *dstep : 0u;
     const uint32_t seed = sr[parity];
     if (blockIdx.x == 0 && threadIdx.x == 0) sr[parity ^ 1] = seed + 1u;
-    const int c = blockIdx.x * blockDim.x + threadIdx.x;
+    const int c = (sizeof(S) == 4 && flip ? gridDim.x - 1 - blockIdx.x : blockIdx.x) * blockDim.x + threadIdx.x;
     if (c >= L.ncell) return;
     int x, y, z;
     node_coords(L, c, x, y, z);
@@ -131,7 +155,7 @@ __global__ void __launch_bounds__(kLineThreads) k_sweep_line(const S *__restrict
         clamp_box(L, box, lo, ext);
         if (in_box(L, lo, ext, x, y, z)) return;
     }
-    sweep_cell<S, R, kOff32>(fin, fout, force, stamp, step, L, fields, x, y, z, seed);
+    sweep_cell<S, R, kOff32, false, kStream>(fin, fout, force, stamp, step, L, fields, x, y, z, seed);
 }
 
 // The far field (nodes outside the body box) with a bounded number of
@@ -415,6 +439,29 @@ static void sweep_shape(const Lattice &L, dim3 &grid, dim3 &block) {
     grid = dim3((L.nx + bx - 1) / bx, (L.ny + by - 1) / by, L.nz);
 }
 
+// Parts 0 and 1 by rows or by consecutive nodes
+template <typename S, typename R, bool kOff32, bool kStream>
+static void sweep_nodes(const void *fin, void *fout, void *force, const uint32_t *stamp, const uint32_t *step,
+                        const Lattice &L, void *fields, int part, const int *box, uint32_t *sr, int parity, int flip,
+                        int nsm, cudaStream_t s) {
+    dim3 grid, block;
+    const int *skip = part == 1 ? box : nullptr;
+    if (line_sweep(L, part)) {
+        const SmallSweep m = sizeof(R) == 8 && part == 0 ? small_sweep64(L, nsm) : SmallSweep{false, kLineThreads};
+        if (!m.rows) {
+            k_sweep_line<S, R, kOff32, kStream><<<grid_for(L.ncell, m.threads), m.threads, 0, s>>>(
+                (const S *)fin, (S *)fout, (R *)force, stamp, step, L, (R *)fields, skip, sr, parity, flip);
+            return;
+        }
+        grid = dim3(1, L.ny, L.nz);
+        block = dim3((L.nx + 31) / 32 * 32);
+    } else {
+        sweep_shape(L, grid, block);
+    }
+    k_sweep<S, R, kOff32, kStream><<<grid, block, 0, s>>>((const S *)fin, (S *)fout, (R *)force, stamp, step, L,
+                                                          (R *)fields, skip, sr, parity, flip);
+}
+
 // part: 0 whole lattice, 1 outside the box, 2 inside the box
 template <typename S, typename R, bool kOff32>
 static cudaError_t sweep_t(const void *fin, void *fout, void *force, const uint32_t *stamp, const uint32_t *step,
@@ -435,20 +482,17 @@ static cudaError_t sweep_t(const void *fin, void *fout, void *force, const uint3
         k_sweep_far<S, R, kOff32><<<L.far_per_sm * nsm, block, 0, s>>>((const S *)fin, (S *)fout, (R *)force, stamp, step,
                                                                L, (R *)fields, box, sr, parity, (int)grid.x,
                                                                (int)grid.y);
-    } else if (line_sweep(L, part)) {
-        const SmallSweep m = sizeof(R) == 8 && part == 0 ? small_sweep64(L, nsm) : SmallSweep{false, kLineThreads};
-        if (m.rows)
-            k_sweep<S, R, kOff32><<<dim3(1, L.ny, L.nz), (L.nx + 31) / 32 * 32, 0, s>>>(
-                (const S *)fin, (S *)fout, (R *)force, stamp, step, L, (R *)fields, nullptr, sr, parity);
-        else
-            k_sweep_line<S, R, kOff32><<<grid_for(L.ncell, m.threads), m.threads, 0, s>>>(
-                (const S *)fin, (S *)fout, (R *)force, stamp, step, L, (R *)fields, part == 1 ? box : nullptr, sr,
-                parity);
     } else {
-        dim3 grid, block;
-        sweep_shape(L, grid, block);
-        k_sweep<S, R, kOff32><<<grid, block, 0, s>>>((const S *)fin, (S *)fout, (R *)force, stamp, step, L, (R *)fields,
-                                             part == 1 ? box : nullptr, sr, parity);
+        const SweepReuse reuse = sweep_reuse<S>(L, parity);
+        if constexpr (sizeof(S) == 4) {
+            if (reuse.stream) {
+                sweep_nodes<S, R, kOff32, true>(fin, fout, force, stamp, step, L, fields, part, box, sr, parity,
+                                                reuse.flip, nsm, s);
+                return cudaGetLastError();
+            }
+        }
+        sweep_nodes<S, R, kOff32, false>(fin, fout, force, stamp, step, L, fields, part, box, sr, parity, reuse.flip,
+                                         nsm, s);
     }
     return cudaGetLastError();
 }

@@ -287,8 +287,8 @@ __device__ __forceinline__ T *plane_ptr(T *base, const Lattice &L, int i, int o)
 
 // Stream, walls and collision of node (x, y, z).  kCG: the populations and
 // tile flags may have been written by other blocks of the launch (see
-// ld_ro).
-template <typename S, typename R, bool kOff32, bool kCG = false>
+// ld_ro).  kStream: the populations read leave the L2 first.
+template <typename S, typename R, bool kOff32, bool kCG = false, bool kStream = false>
 __device__ __forceinline__ void sweep_cell(const S *__restrict__ fin, S *__restrict__ fout, R *__restrict__ force,
                                            const uint32_t *__restrict__ stamp, uint32_t step, const Lattice &L,
                                            R *__restrict__ fields, int x, int y, int z, uint32_t seed) {
@@ -317,7 +317,11 @@ __device__ __forceinline__ void sweep_cell(const S *__restrict__ fin, S *__restr
         const int sx = ex(i) > 0 ? xm : ex(i) < 0 ? xp : x;
         const int sy = ey(i) > 0 ? oy_m : ey(i) < 0 ? oy_p : oy_0;
         const int sz = ez(i) > 0 ? oz_m : ez(i) < 0 ? oz_p : oz_0;
-        raw[i] = ld_ro<kCG>(plane_ptr<kOff32>(fin, L, i, sx + sy + sz));
+        const S *const p = plane_ptr<kOff32>(fin, L, i, sx + sy + sz);
+        if constexpr (kStream)
+            raw[i] = __ldcs(p);
+        else
+            raw[i] = ld_ro<kCG>(p);
     }
     R fib[3];
     fetch_force(force, stamp && flag == step, st, idx, fib);

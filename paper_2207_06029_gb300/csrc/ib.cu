@@ -336,7 +336,8 @@ __device__ __forceinline__ void exchange_force(const BodyView &B, int t, R area,
 //  positions: the point (probes: triangle geometry), the nearest node base =
 //           floor(X + 1/2) and the exact offset X - base.
 //           Nothing here reads the moments: with kChain it runs while the
-//           moments kernel ends;
+//           moments kernel ends, and so reads the positions at the L2
+//           (chain_release's comment);
 //  sums:    W is a product over the axes but for its cut-off r_k <= 1 (a bit
 //           per node, decided exactly as in FP64), so the ten sums of A and
 //           the sixteen of b (fields less those of the centre node) are formed
@@ -364,11 +365,10 @@ __device__ __forceinline__ void mls_body(const R *mom, const Lattice &L, const B
         double P[3];
         if (p < nm && B.centroid) {
             const int *tv = B.tri + 3 * p;
-            for (int a = 0; a < 3; ++a) P[a] = (B.X[3 * tv[0] + a] + B.X[3 * tv[1] + a] + B.X[3 * tv[2] + a]) / 3.0;
+            for (int a = 0; a < 3; ++a)
+                P[a] = (__ldcg(B.X + 3 * tv[0] + a) + __ldcg(B.X + 3 * tv[1] + a) + __ldcg(B.X + 3 * tv[2] + a)) / 3.0;
         } else if (p < nm) {
-            P[0] = B.X[3 * p];
-            P[1] = B.X[3 * p + 1];
-            P[2] = B.X[3 * p + 2];
+            for (int a = 0; a < 3; ++a) P[a] = __ldcg(B.X + 3 * p + a);
         } else {
             // probe X_c +- 1.2 n, with X_c = x_0 + (e1 + e2)/3 and the
             // triangle's edges and normal from origin-relative positions
@@ -377,10 +377,10 @@ __device__ __forceinline__ void mls_body(const R *mom, const Lattice &L, const B
             const R *Xr = (const R *)B.Xrel;
             R r0[3], e1[3], e2[3];
             for (int a = 0; a < 3; ++a) {
-                P[a] = B.X[3 * tv[0] + a];
-                r0[a] = Xr[3 * tv[0] + a];
-                e1[a] = Xr[3 * tv[1] + a] - r0[a];
-                e2[a] = Xr[3 * tv[2] + a] - r0[a];
+                P[a] = __ldcg(B.X + 3 * tv[0] + a);
+                r0[a] = __ldcg(Xr + 3 * tv[0] + a);
+                e1[a] = __ldcg(Xr + 3 * tv[1] + a) - r0[a];
+                e2[a] = __ldcg(Xr + 3 * tv[2] + a) - r0[a];
             }
             const R N[3] = {e1[1] * e2[2] - e1[2] * e2[1], e1[2] * e2[0] - e1[0] * e2[2],
                             e1[0] * e2[1] - e1[1] * e2[0]};
@@ -651,15 +651,15 @@ __device__ __forceinline__ void mls_quad_body(const R *mom, const Lattice &L, co
         const int *tv = B.tri + 3 * t;
         const int i0 = tv[0], i1 = tv[1], i2 = tv[2];
         const R *Xr = (const R *)B.Xrel;
-        P = B.X[3 * i0 + a];
-        r0 = Xr[3 * i0 + a];
-        e1 = Xr[3 * i1 + a] - r0;
-        e2 = Xr[3 * i2 + a] - r0;
+        P = __ldcg(B.X + 3 * i0 + a);
+        r0 = __ldcg(Xr + 3 * i0 + a);
+        e1 = __ldcg(Xr + 3 * i1 + a) - r0;
+        e2 = __ldcg(Xr + 3 * i2 + a) - r0;
     } else if (p >= 0 && B.centroid) {
         const int *tv = B.tri + 3 * p;
-        P = (B.X[3 * tv[0] + a] + B.X[3 * tv[1] + a] + B.X[3 * tv[2] + a]) / 3.0;
+        P = (__ldcg(B.X + 3 * tv[0] + a) + __ldcg(B.X + 3 * tv[1] + a) + __ldcg(B.X + 3 * tv[2] + a)) / 3.0;
     } else if (p >= 0) {
-        P = B.X[3 * p + a];
+        P = __ldcg(B.X + 3 * p + a);
     }
     const R e1b = from(e1, a1), e1c = from(e1, a2), e2b = from(e2, a1), e2c = from(e2, a2);
     const R N = e1b * e2c - e1c * e2b;
@@ -1035,10 +1035,10 @@ __device__ __forceinline__ void membrane_body(const Lattice &L, const BodyView &
         const R ksh = par[0], l0h = par[1], kbh = par[2], th0h = par[3];
         R e[3], ac[3], ad[3];
         for (int a = 0; a < 3; ++a) {
-            const R xa = Xr[3 * H.x + a];
-            e[a] = Xr[3 * H.y + a] - xa;
-            ac[a] = Xr[3 * H.z + a] - xa;
-            ad[a] = Xr[3 * H.w + a] - xa;
+            const R xa = __ldcg(Xr + 3 * H.x + a);
+            e[a] = __ldcg(Xr + 3 * H.y + a) - xa;
+            ac[a] = __ldcg(Xr + 3 * H.z + a) - xa;
+            ad[a] = __ldcg(Xr + 3 * H.w + a) - xa;
         }
         if constexpr (sizeof(R) == 4) {
             // the FP32 coordinates carry an absolute error of half an ulp of
@@ -1047,10 +1047,10 @@ __device__ __forceinline__ void membrane_body(const Lattice &L, const BodyView &
             // angles (small differences of the edges) need
             const float *Xl = B.Xlo;
             for (int a = 0; a < 3; ++a) {
-                const float la = Xl[3 * H.x + a];
-                e[a] += Xl[3 * H.y + a] - la;
-                ac[a] += Xl[3 * H.z + a] - la;
-                ad[a] += Xl[3 * H.w + a] - la;
+                const float la = __ldcg(Xl + 3 * H.x + a);
+                e[a] += __ldcg(Xl + 3 * H.y + a) - la;
+                ac[a] += __ldcg(Xl + 3 * H.z + a) - la;
+                ad[a] += __ldcg(Xl + 3 * H.w + a) - la;
             }
         }
         const R le2 = e[0] * e[0] + e[1] * e[1] + e[2] * e[2];
@@ -1102,7 +1102,7 @@ __device__ __forceinline__ void membrane_body(const Lattice &L, const BodyView &
     // components of the block's vertices integrated below: thread 3 j + a
     const int j = threadIdx.x / 3, a = threadIdx.x % 3, vj = v0 + j;
     const bool mine = (int)threadIdx.x < 3 * nvpb && vj < B.nv;
-    const double x = mine ? B.X[3 * vj + a] : 0.0, xp = mine ? B.Xprev[3 * vj + a] : 0.0;
+    const double x = mine ? __ldcg(B.X + 3 * vj + a) : 0.0, xp = mine ? __ldcg(B.Xprev + 3 * vj + a) : 0.0;
     chain_wait();
     const uint32_t step = __ldcg(dstep);  // written by the moments kernel of the step
     const double U0 = mine && !B.centroid ? B.U[3 * vj + a] : 0.0;
@@ -1382,7 +1382,7 @@ __device__ __forceinline__ void rigid_markers_body(const Lattice &L, const BodyV
         double x[3] = {0.0, 0.0, 0.0}, xb[3] = {0.0, 0.0, 0.0};
         if (mine)
             for (int k = 0; k < 3; ++k) {
-                x[k] = B.X[3 * vj + (a + k) % 3];
+                x[k] = __ldcg(B.X + 3 * vj + (a + k) % 3);
                 xb[k] = B.Xbody[3 * vj + k];
             }
         const int q1 = v < B.nv ? B.vt_ptr[v + 1] : 0, q0 = v < B.nv ? B.vt_ptr[v] + l8 : 0;
@@ -1510,9 +1510,9 @@ __global__ void __launch_bounds__(kStructThreads) k_centroid_spread(Lattice L, B
 // ---- batch kernels: the bodies of all lattices of a batch per launch ----
 // Each is launched programmatically behind the one before and waits for it
 // once its tables are staged (and, MLS and membrane, the positions, weights
-// and hinge forces formed).  Those early parts read what the previous step's
-// structure kernels wrote: the sweep between releases its successor only
-// after its own wait, so these have completed by then.
+// and hinge forces formed).  Those early parts read, at the L2, what the
+// previous step's structure kernels wrote: the sweep between releases its
+// successor only after its own wait, so these have completed by then.
 template <typename S, typename R>
 __global__ void __launch_bounds__(256) kb_moments(BatchTables T, int phase) {
     __shared__ Lattice L;

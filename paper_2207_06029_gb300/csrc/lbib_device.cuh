@@ -18,9 +18,15 @@ constexpr int kTile = 8;  // edge of the cubic tiles that carry an IB-force flag
 // Programmatic dependent launch (sm_90 and later).  A kernel launched with
 // programmatic stream serialization may be scheduled once every block of
 // its predecessor in the stream has called chain_release() (or ended); it
-// calls chain_wait() before its first global-memory access, which returns
-// when the predecessor has completed and its writes are visible.  Without
-// that launch attribute chain_wait() returns at once.
+// calls chain_wait() before it touches anything the predecessor reads or
+// writes, which returns when the predecessor has completed and its writes are
+// visible.  Without that launch attribute chain_wait() returns at once.
+//
+// Before its wait a kernel reads only what never changes during the steps
+// (meshes, tables) and what kernels completed before its predecessor began
+// wrote.  Nothing orders the latter for it but their completion: the writes
+// have reached the L2, but an L1 line of an earlier step may stand on its SM,
+// so these loads go to the L2 (__ldcg).
 __device__ __forceinline__ void chain_release() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
 __device__ __forceinline__ void chain_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
 

@@ -912,7 +912,9 @@ __device__ __forceinline__ void tri_hydro(const BodyView &B, int t, R *F) {
 
 // Spreading by the 8 lanes of a marker: c phi_k F added to the force field
 // at the support nodes with r_k <= 1 (the others have phi_k = 0), from the
-// marker's transfer record; the tiles of the block's 8 corners are flagged.
+// marker's transfer record; the tiles of the 27 nodes' 8 corners are flagged.
+// These are all their tiles, but for a middle node that is a tile by itself:
+// the last node of a periodic axis of 8 m + 1 nodes (Lattice::seam).
 constexpr int kLanes = 8;  // lanes per marker in the structure kernels
 template <typename R>
 __device__ __forceinline__ void spread(const Lattice &L, const BodyView &B, int p, int l8, R c, const R *Fl,
@@ -934,9 +936,18 @@ __device__ __forceinline__ void spread(const Lattice &L, const BodyView &B, int 
         atomicAdd(force + st + node, phi * F1);
         atomicAdd(force + 2 * st + node, phi * F2);
     }
-    const int x = support_coord(L, 0, bs.x + (l8 & 1 ? 1 : -1)), y = support_coord(L, 1, bs.y + (l8 & 2 ? 1 : -1)),
-              z = support_coord(L, 2, bs.z + (l8 & 4 ? 1 : -1));
-    stamp[(x >> 3) + L.ntx * ((y >> 3) + L.nty * (z >> 3))] = step;
+    auto flag = [&](int i, int j, int k) {
+        const int x = support_coord(L, 0, bs.x + i), y = support_coord(L, 1, bs.y + j), z = support_coord(L, 2, bs.z + k);
+        stamp[(x >> 3) + L.ntx * ((y >> 3) + L.nty * (z >> 3))] = step;
+    };
+    const bool seam = (L.seam & 1 && support_coord(L, 0, bs.x) == L.nx - 1) ||
+                      (L.seam & 2 && support_coord(L, 1, bs.y) == L.ny - 1) ||
+                      (L.seam & 4 && support_coord(L, 2, bs.z) == L.nz - 1);
+    if (!seam) {
+        flag(l8 & 1 ? 1 : -1, l8 & 2 ? 1 : -1, l8 & 4 ? 1 : -1);
+    } else {
+        for (int q = l8; q < 27; q += kLanes) flag(q % 3 - 1, (q / 3) % 3 - 1, q / 9 - 1);
+    }
 }
 template <typename T>
 __device__ __forceinline__ T lanes_sum(T v) {  // over the 8 lanes of a marker

@@ -468,6 +468,9 @@ int lbib_create(const lbib_params *p, void **out) {
     L.ntx = (n[0] + kTile - 1) / kTile;
     L.nty = (n[1] + kTile - 1) / kTile;
     L.ntz = (n[2] + kTile - 1) / kTile;
+    L.seam = 0;
+    for (int a = 0; a < 3; ++a)
+        if (p->bc[a] == LBIB_PERIODIC && n[a] % kTile == 1) L.seam |= 1 << a;
     L.ncell = (int)ncell;
     set_dividers(L);
     L.stride = (ncell + 63) / 64 * 64;

@@ -228,6 +228,7 @@ struct Lattice {
     double tau;
     double gext[3];
     double wall_u[6][3];
+    int seam;               // bit a: axis a is periodic with n % 8 == 1, its last tile one node wide
     double dist2_cut;       // largest |X - x_k|^2 whose MLS weight is non-zero
     uint32_t mul_x, mul_y;  // division by nx and ny (set_dividers)
     int shr_x, shr_y;

@@ -247,7 +247,8 @@ int lbib_get_profile(void *ctx, double *ms, long long *nsteps);
  * the sweep kernel and its block shape (the row-tile kernel with 128-bit
  * loads and stores where rows are whole 16-byte vectors, or the one-node
  * kernel in several shapes), then (single-body contexts) the overlap of the far-field
- * sweep with the IB stage.  Each trial runs
+ * sweep with the IB stage, which its trials turn off and on whatever the
+ * lattice's size and its choice sets as lbib_set_overlap does.  Each trial runs
  * 1 + 2 * `steps` real time steps, so the simulation advances by about
  * 16 * `steps` steps.  choice (optional, 5 ints) receives block x, block y (0, 0: whole
  * x-rows), the overlap flag, the row-tile flag and the far-field blocks per
@@ -262,8 +263,9 @@ int lbib_autotune(void *ctx, int steps, int *choice);
  * ignored), 0 the one-node kernel with blocks of block_x * block_y threads
  * (0, 0: whole x-rows); far_per_sm > 0 runs the far-field sweep (overlap
  * on) with that many resident blocks per SM striding over the lattice, so
- * that the IB kernels beside it find free SMs, 0 on its full grid.  Results
- * are the same in every configuration. */
+ * that the IB kernels beside it find free SMs, 0 on its full grid; a context
+ * whose overlap has not been set (lbib_set_overlap) overlaps with far_per_sm >
+ * 0 whatever its size.  Results are the same in every configuration. */
 int lbib_set_sweep_config(void *ctx, int row_tiles, int block_x, int block_y, int far_per_sm);
 
 /* Resident blocks per SM of the IB kernels (MLS, structure update and
@@ -280,10 +282,12 @@ int lbib_set_ib_blocks(void *ctx, int per_sm);
 int lbib_get_launch_config(void *ctx, int *cfg);
 
 /* With a single body, the sweep of the nodes outside the body's support
- * box runs on a second stream concurrently with the IB stage (default 1);
- * 0 runs one whole-lattice sweep after the IB stage, as small lattices
- * (below 360 000 nodes, 48 000 in FP64) and large ones in 16-bit storage
- * (above 8 000 000 nodes in FP16, 4 000 000 in bfloat16) do either way.
+ * box runs on a second stream concurrently with the IB stage (1), or one
+ * whole-lattice sweep runs after it (0).  Until this call (or lbib_autotune)
+ * the faster of the two by the lattice's size is taken: one sweep for small
+ * lattices (below 360 000 nodes, 48 000 in FP64) and large ones in 16-bit
+ * storage (above 8 000 000 nodes in FP16, 4 000 000 in bfloat16), the overlap
+ * for all others.  lbib_get_launch_config reports the overlap in force.
  * Results are the same either way. */
 int lbib_set_overlap(void *ctx, int enable);
 

@@ -74,7 +74,9 @@ struct Ctx {
     cudaStream_t stream = nullptr;           // the caller's (or the library's) stream
     cudaStream_t s_hi = nullptr, s_lo = nullptr;  // step streams: IB + box sweep (high priority), far field (low)
     cudaEvent_t ev_fork = nullptr, ev_far = nullptr, ev_near = nullptr, ev_join = nullptr;
-    bool split_sweep = true;
+    // the far-field sweep beside the IB stage: 1 yes, 0 no (lbib_set_overlap, the
+    // autotuner), -1 as the lattice's size says (splits_by_size)
+    int overlap = -1;
     int ib_per_sm = 0;  // > 0: the IB kernels keep at most this many blocks per SM (lbib_set_ib_blocks)
     bool own_stream = false;
     std::vector<DevBody> bodies;
@@ -1012,7 +1014,8 @@ int lbib_add_body(void *h, const double *verts, int nv, const int *tris, int nt,
 
 namespace {
 
-// Whether the step of a context sweeps the far field beside the IB stage.
+// Whether the step of a context sweeps the far field beside the IB stage
+// unless the caller or the autotuner has said so.
 // Below kSplitCells nodes (kSplitCells64 in FP64) the step is the chain of
 // the IB kernels' latencies, and one sweep behind them is shorter than the
 // box sweep and the join.  Measured us a step, overlap against one sweep,
@@ -1028,13 +1031,18 @@ namespace {
 // to 161; 160^3 bfloat16 95.6 against 94.4.
 constexpr int kSplitCells = 360000, kSplitCells64 = 48000;
 constexpr int kSplitMostFp16 = 8000000, kSplitMostBf16 = 4000000;
-bool splits(const Ctx *c) {
-    if (c->bodies.size() != 1 || !c->split_sweep) return false;
+bool splits_by_size(const Ctx *c) {
     if (c->L.ncell < (c->prec == LBIB_FP64 ? kSplitCells64 : kSplitCells)) return false;
     if (c->prec == LBIB_FP16_DEV) return c->L.ncell <= kSplitMostFp16;
     if (c->prec == LBIB_BF16_DEV) return c->L.ncell <= kSplitMostBf16;
     return true;
 }
+// The overlap in force (of a context with one body): blocks per SM asked for
+// the far-field sweep ask for that sweep.
+bool overlaps(const Ctx *c) {
+    return c->overlap >= 0 ? c->overlap != 0 : c->L.far_per_sm > 0 || splits_by_size(c);
+}
+bool splits(const Ctx *c) { return c->bodies.size() == 1 && overlaps(c); }
 
 // Enqueues one step on the two step streams (the caller forks them from,
 // and joins them into, an origin stream).  With one body, the nodes
@@ -1697,8 +1705,7 @@ int lbib_autotune(void *h, int steps, int *choice) {
     const bool vec_ok = (c->L.nx & 3) == 0 && (c->L.nx * esz) % 16 == 0 &&
                         19LL * std::max(1, std::min(256 / c->L.nx, c->L.ny)) * c->L.nx * esz <= 160 * 1024 &&
                         c->L.nx <= 512;
-    const bool saved_split = c->split_sweep;
-    c->split_sweep = false;
+    c->overlap = 0;
     float best = 1e30f;
     int best_shape = 0, rc = 0;
     for (int k = 0; k < (int)(sizeof(shapes) / sizeof(shapes[0])); ++k) {
@@ -1723,10 +1730,9 @@ int lbib_autotune(void *h, int steps, int *choice) {
     // on its full grid or on a few resident blocks per SM, the IB kernels on
     // their full grids or on one or two resident blocks per SM
     int overlap = 0, far = 0, ibs = 0;
-    const int saved_ibs = c->ib_per_sm;
     c->ib_per_sm = 0;
     if (!rc && c->bodies.size() == 1) {
-        c->split_sweep = true;
+        c->overlap = 1;
         for (int fps : {0, 1, 2, 3})
             for (int ib : {0, 1, 2}) {
                 if (rc) break;
@@ -1742,13 +1748,10 @@ int lbib_autotune(void *h, int steps, int *choice) {
                     ibs = ib;
                 }
             }
-    } else {
-        (void)saved_split;
-        (void)saved_ibs;
     }
     c->L.far_per_sm = far;
     c->ib_per_sm = ibs;
-    c->split_sweep = overlap != 0;
+    c->overlap = overlap;
     invalidate_graphs(c);
     cudaEventDestroy(e0);
     cudaEventDestroy(e1);
@@ -1790,7 +1793,7 @@ int lbib_get_launch_config(void *h, int *cfg) {
     if (!c || !cfg) return LBIB_EINVAL;
     cfg[0] = c->L.sweep_bx;
     cfg[1] = c->L.sweep_by;
-    cfg[2] = c->split_sweep ? 1 : 0;
+    cfg[2] = overlaps(c) ? 1 : 0;
     cfg[3] = c->L.sweep_vec;
     cfg[4] = c->L.far_per_sm;
     cfg[5] = c->ib_per_sm;
@@ -1800,8 +1803,9 @@ int lbib_get_launch_config(void *h, int *cfg) {
 int lbib_set_overlap(void *h, int enable) {
     Ctx *c = as_ctx(h);
     if (!c) return LBIB_EINVAL;
-    if (c->split_sweep != (enable != 0)) invalidate_graphs(c);
-    c->split_sweep = enable != 0;
+    const bool was = overlaps(c);
+    c->overlap = enable != 0;
+    if (was != overlaps(c)) invalidate_graphs(c);
     return LBIB_OK;
 }
 

@@ -164,6 +164,8 @@ void dev_free_one(Ctx *c, void *ptr) {
                 cudaFree(ptr);
             c->bytes -= c->allocs[k].second;
             c->allocs.erase(c->allocs.begin() + k);
+            // a later array at the same address belongs to the checkpoints
+            c->transient.erase(std::remove(c->transient.begin(), c->transient.end(), ptr), c->transient.end());
             return;
         }
 }
@@ -1467,6 +1469,7 @@ int lbib_step_markers(void *h, int nsteps, int body, double *X, double *V, doubl
         }
         c->mstage = static_cast<double *>(dev_alloc(c, need));
         if (!c->mstage) return fail(c, LBIB_ENOMEM, "marker staging buffer of %zu bytes", need);
+        c->transient.push_back(c->mstage);
         c->mstage_bytes = need;
     }
     if (!c->d_rec) {
@@ -2619,12 +2622,17 @@ int lbib_load(void *h, const void *buf, size_t size) {
             return fail(c, LBIB_EINVAL, "checkpoint bodies differ from the context's");
     int32_t nsaved = 0;
     for (size_t k = 0; k < c->allocs.size(); ++k) nsaved += persistent(c, k);
+    // checkpoints written when the staging buffer of recorded markers was saved
+    // too load where they did, in a context that has one of the same size
+    const bool staged = c->mstage && hd.nsaved == nsaved + 1;
+    nsaved += staged;
+    auto saved = [&](size_t k) { return persistent(c, k) || (staged && c->allocs[k].first == c->mstage); };
     if (nsaved != hd.nsaved || hd.fa_index < 0 || hd.fa_index >= (int32_t)c->allocs.size())
         return fail(c, LBIB_EINVAL, "checkpoint buffers differ from the context's");
     // check every size before copying anything
     size_t o = off;
     for (size_t k = 0; k < c->allocs.size(); ++k) {
-        if (!persistent(c, k)) continue;
+        if (!saved(k)) continue;
         uint64_t n = 0;
         if (size < o + sizeof(n)) return fail(c, LBIB_EINVAL, "checkpoint too short");
         std::memcpy(&n, in + o, sizeof(n));
@@ -2637,7 +2645,7 @@ int lbib_load(void *h, const void *buf, size_t size) {
     if (e == cudaSuccess) e = cudaStreamSynchronize(c->s_lo);
     if (e != cudaSuccess) return cuda_fail(c, e, "checkpoint sync");
     for (size_t k = 0; k < c->allocs.size(); ++k) {
-        if (!persistent(c, k)) continue;
+        if (!saved(k)) continue;
         uint64_t n = 0;
         std::memcpy(&n, in + off, sizeof(n));
         off += sizeof(n);

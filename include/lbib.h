@@ -354,9 +354,10 @@ int lbib_batch_counters(void *batch, long long *steps, long long *launches);
 /* Times `steps` six-step graph launches and one field-storing step (what
  * a long lbib_batch_step runs) for each sweep configuration and keeps the
  * fastest:
- * the batched sweep with 128, 256 or 512 threads a block and 1 or 4 cells a
- * thread, one one-lattice sweep launch per lattice spread over side
- * streams, or the persistent kernel (lbib_batch_set_persistent) with sweep
+ * the batched sweep with 128 or 256 threads a block and 1 or 4 cells a
+ * thread, 128 threads and 8 cells or 512 and 4, one one-lattice sweep launch
+ * per lattice spread over side streams, or the persistent kernel
+ * (lbib_batch_set_persistent) with sweep
  * tiles of 256 x 4, 8 or 16 cells, each with the lattices as given or
  * largest first; the contexts advance by 20 * (24 + 12 * steps) steps.
  * choice (optional, 3 ints): threads (0: one launch per lattice, -1: the

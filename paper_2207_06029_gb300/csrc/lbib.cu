@@ -2419,8 +2419,11 @@ int lbib_batch_autotune(void *h, int steps, int *choice) {
     // lattices as given or largest first
     // or the persistent kernel (threads = -1) with sweep tiles of 256 x 4, 8
     // or 16 cells
-    const int shapes[][2] = {{128, 1}, {256, 1}, {512, 1}, {128, 4}, {128, 8}, {256, 4},
+    // (their number is part of the interface: 20 trials with the two orders, of
+    // 24 + 12 steps steps each)
+    const int shapes[][2] = {{128, 1}, {256, 1}, {128, 4}, {128, 8}, {256, 4},
                              {512, 4}, {0, 0},   {-1, 4},  {-1, 8}, {-1, 16}};
+    static_assert(sizeof(shapes) / sizeof(shapes[0]) == 10, "lbib_batch_autotune advances by 20 trials");
     float best = 1e30f;
     int best_t = b->sweep_threads, best_o = b->order, best_c = b->sweep_cpt, best_split = b->sweep_split,
         best_p = b->persistent;

@@ -283,6 +283,13 @@ __device__ __forceinline__ int support_coord(const Lattice &L, int a, int c) {
     return wrap_periodic(c, n);
 }
 
+// Coordinate of the node nearest to x (any that is on the lattice, for a run
+// that has diverged).
+__device__ __forceinline__ int near_coord(const Lattice &L, int a, double x) {
+    const int n = a == 0 ? L.nx : a == 1 ? L.ny : L.nz, c = __double2int_rn(x);
+    return L.bc[a] == kPeriodic ? support_coord(L, a, c) : min(max(c, 0), n - 1);
+}
+
 // Transfer record of marker p: row 0 of A^-1 (4), the offset X - base (3) and
 // the three axes' weights (9), from which every support node's transfer
 // weight phi_k = W_k (A^-1 p_k)_0 follows; base node and the bits of the
@@ -348,6 +355,13 @@ __device__ __forceinline__ void exchange_force(const BodyView &B, int t, R area,
 //           probes the pressure c_s^2 rho and the traction
 //           rho nu (grad u + grad u^T) . n from the fits (membranes keep
 //           them per triangle, rigid bodies sum the forces and moments).
+//           A rigid body's two probes of a triangle are rounded and summed
+//           apart, so both take their pressure less that of the node nearest
+//           to the triangle's first corner: an offset of the density leaves
+//           before the first rounding (density 1.1, sphere of radius 4 to 8,
+//           error of the FP32 angular impulse against FP64: 10 to 21e-9 with
+//           the full pressures, 3 to 14e-9 as differences per triangle,
+//           3 to 14e-9 so; 32^3 FP64 sphere 50.3 -> 50.7 us a step).
 template <typename R, bool kCG = false, bool kChain = false>
 __device__ __forceinline__ void mls_body(const R *mom, const Lattice &L, const BodyView &B, int *err,
                                          const int vb) {
@@ -360,7 +374,7 @@ __device__ __forceinline__ void mls_body(const R *mom, const Lattice &L, const B
     // ---------------- positions ----------------
     double vol = 0.0, frac[3] = {0.0, 0.0, 0.0};
     R nrm[3] = {R(0), R(0), R(0)}, arm[3] = {R(0), R(0), R(0)}, area = R(0);  // probes: normal, X_c - x_c, area
-    int base[3] = {2, 2, 2};
+    int base[3] = {2, 2, 2}, ref = 0;  // ref: the node whose density a rigid body's probe refers to
     if (p >= 0) {
         double P[3];
         if (p < nm && B.centroid) {
@@ -388,6 +402,8 @@ __device__ __forceinline__ void mls_body(const R *mom, const Lattice &L, const B
             const R inn = R(1) / nn, sg = side ? R(-kProbe) : R(kProbe);
             R *tg = (R *)B.tri_geo + 8 * t;
             area = R(0.5) * nn;
+            if (B.rigid)
+                ref = near_coord(L, 0, P[0]) + L.nx * (near_coord(L, 1, P[1]) + L.ny * near_coord(L, 2, P[2]));
             for (int a = 0; a < 3; ++a) {
                 nrm[a] = N[a] * inn;
                 const R c3 = (e1[a] + e2[a]) / R(3);
@@ -464,6 +480,7 @@ __device__ __forceinline__ void mls_body(const R *mom, const Lattice &L, const B
     // the fitted values) need
     R fc[4];
     mom_load<kCG>(mom, ox[1] + oy[1] + oz[1], fc);
+    const R dr = p >= nm && B.rigid ? fc[0] - ld_ro<kCG>(mom + 4 * (size_t)ref) : fc[0];
     // A: 00, 01, 02, 03, 11, 12, 13, 22, 23, 33; b[c]: 1, x, y, z
     R A[10], b[4][4];
 #pragma unroll
@@ -559,7 +576,7 @@ __device__ __forceinline__ void mls_body(const R *mom, const Lattice &L, const B
     } else {
         // fits: c_f[i] = sum_m Ai[i][m] b_f[m], plus the centre value for
         // the value (i = 0)
-        const R cr = Ai[0] * b[0][0] + Ai[1] * b[0][1] + Ai[2] * b[0][2] + Ai[3] * b[0][3] + fc[0];
+        const R c0 = Ai[0] * b[0][0] + Ai[1] * b[0][1] + Ai[2] * b[0][2] + Ai[3] * b[0][3];
         R gr[3][3];
 #pragma unroll
         for (int c = 0; c < 3; ++c)
@@ -569,8 +586,8 @@ __device__ __forceinline__ void mls_body(const R *mom, const Lattice &L, const B
                 gr[c][a] = row[0] * bu[0] + row[1] * bu[1] + row[2] * bu[2] + row[3] * bu[3];
             }
         const int t = (p - nm) >> 1, side = (p - nm) & 1;
-        const R rn = (R(1) + cr) * pick<R>(L.nu_d, L.nu_f);
-        const R pr0 = cr / R(3);  // p - c_s^2 rho0
+        const R rn = (R(1) + (c0 + fc[0])) * pick<R>(L.nu_d, L.nu_f);
+        const R pr0 = (c0 + dr) / R(3);  // p - c_s^2 rho0 (rigid: less that of node ref)
         R tr[3];
 #pragma unroll
         for (int c = 0; c < 3; ++c) {
@@ -646,12 +663,14 @@ __device__ __forceinline__ void mls_quad_body(const R *mom, const Lattice &L, co
 
     // ---------------- positions: component a ----------------
     double P = 0.0;
+    int rc = 0;  // rigid: coordinate of the node whose density the probe refers to
     R r0 = R(0), e1 = R(0), e2 = R(0);
     if (probe) {
         const int *tv = B.tri + 3 * t;
         const int i0 = tv[0], i1 = tv[1], i2 = tv[2];
         const R *Xr = (const R *)B.Xrel;
         P = __ldcg(B.X + 3 * i0 + a);
+        if (B.rigid) rc = near_coord(L, a, P);
         r0 = __ldcg(Xr + 3 * i0 + a);
         e1 = __ldcg(Xr + 3 * i1 + a) - r0;
         e2 = __ldcg(Xr + 3 * i2 + a) - r0;
@@ -754,11 +773,13 @@ __device__ __forceinline__ void mls_quad_body(const R *mom, const Lattice &L, co
         oy[i] = from(o, 1);
         oz[i] = from(o, 2);
     }
+    const int ref = B.rigid ? from(rc, 0) + L.nx * (from(rc, 1) + L.ny * from(rc, 2)) : 0;
     chain_wait();
 
     // ---------------- sums: field q, and A by the power of x ----------------
     const R *mq = mom + q;
     const R fc = ld_ca(mq + 4 * (size_t)(ox[1] + oy[1] + oz[1]));
+    const R dr = B.rigid && q == 0 ? fc - ld_ca(mom + 4 * (size_t)ref) : fc;  // on lane 0
     R b[4] = {R(0), R(0), R(0), R(0)};
     R C00 = R(0), C10 = R(0), C20 = R(0), C01 = R(0), C11 = R(0), C02 = R(0);  // y and z powers
 #pragma unroll
@@ -799,7 +820,7 @@ __device__ __forceinline__ void mls_quad_body(const R *mom, const Lattice &L, co
     // ---------------- solve ----------------
     R Ai[16];
     if (!spd_inverse4(A, Ai) && p >= 0) atomicCAS(err, 0, -1);
-    const R val = fc + (Ai[3] * b[3] + Ai[2] * b[2] + Ai[1] * b[1] + Ai[0] * b[0]);
+    const R fit = Ai[3] * b[3] + Ai[2] * b[2] + Ai[1] * b[1] + Ai[0] * b[0], val = fc + fit;
     const int b0 = from(base, 0), b1 = from(base, 1), b2 = from(base, 2);
     const R x0 = wx[0], x1 = wx[1], x2 = wx[2], y0 = wy[0], y1 = wy[1], y2 = wy[2], z0 = wz[0], z1 = wz[1], z2 = wz[2];
     if (p >= 0 && !probe) {
@@ -827,7 +848,8 @@ __device__ __forceinline__ void mls_quad_body(const R *mom, const Lattice &L, co
         const R col = from(g[c], 1) * n0 + from(g[c], 2) * n1 + from(g[c], 3) * n2;
         if (q == c + 1) acc += col;
     }
-    const R tr = (R(1) + cr) * pick<R>(L.nu_d, L.nu_f) * acc, pr0 = third(cr);  // p - c_s^2 rho0
+    // p - c_s^2 rho0 (rigid: less that of node ref)
+    const R tr = (R(1) + cr) * pick<R>(L.nu_d, L.nu_f) * acc, pr0 = third(B.rigid ? from(dr + fit, 0) : cr);
     if (probe && !B.rigid) ((R *)B.probe + 8 * t + 4 * side)[q] = q == 0 ? pr0 : tr;
     __shared__ double red[6][kQuadThreads / 32];
     if (B.rigid) {

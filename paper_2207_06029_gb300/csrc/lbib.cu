@@ -1540,16 +1540,26 @@ double *read_back(Ctx *c, const DevBody &b, bool X, bool V, bool F, bool state, 
     return out;
 }
 
-// Whether p may be written by the host (not device memory).
-bool host_pointer(const void *p) {
+// Whether p is null or ordinary host memory (not page-locked, managed or on
+// the device).
+bool pageable(const void *p) {
     if (!p) return true;
     cudaPointerAttributes at{};
     if (cudaPointerGetAttributes(&at, p) != cudaSuccess) {
         cudaGetLastError();
         return false;
     }
-    return at.type != cudaMemoryTypeDevice;
+    return at.type == cudaMemoryTypeUnregistered;
 }
+
+// Bodies whose markers lbib_get_markers takes through the page-locked block
+// when all arrays are pageable.  A copy into pageable memory takes 10 us
+// whatever its size, the block 5 us per 1000 vertices of three arrays and the
+// host's own copy out of it: 162 vertices X, V and F 18 us against 41 by
+// copies, X alone 14 against 20; 4098 34 / 42 and 19.5 / 20; 6146 42 / 44 and
+// 22 / 20; 10 242 61 / 45 and 28 / 21.  Page-locked arrays are copied into
+// directly (10 242 vertices 23 us, 61 through the block; 642 19.6 and 19.5).
+constexpr int kBlockVertices = 5000;
 
 }  // namespace
 
@@ -1562,7 +1572,7 @@ int lbib_get_markers(void *h, int body, double *X, double *V, double *F) {
     if (c->err && !readable_error(c->err)) return c->err;
     const DevBody &b = c->bodies[body];
     const size_t n3 = 3 * (size_t)b.nv;
-    if (host_pointer(X) && host_pointer(V) && host_pointer(F)) {
+    if (b.nv <= kBlockVertices && pageable(X) && pageable(V) && pageable(F)) {
         int rc = LBIB_OK;
         if (const double *r = read_back(c, b, X, V, F, false, &rc)) {
             if (rc == LBIB_ECUDA) return rc;
@@ -1572,7 +1582,7 @@ int lbib_get_markers(void *h, int body, double *X, double *V, double *F) {
             return rc;
         }
     }
-    // large bodies: the copies and the device error word in one round trip
+    // the copies and the device error word in one round trip
     int rc = lbib_get_markers_async(h, body, X, V, F);
     if (rc) return rc;
     return sync_ctx(c);

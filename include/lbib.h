@@ -246,13 +246,13 @@ int lbib_get_profile(void *ctx, double *ms, long long *nsteps);
 /* Times the step in several launch configurations and keeps the fastest:
  * the sweep kernel and its block shape (the row-tile kernel with 128-bit
  * loads and stores where rows are whole 16-byte vectors, or the one-node
- * kernel in several shapes), then (single-body contexts) the overlap of the far-field
- * sweep with the IB stage, which its trials turn off and on whatever the
- * lattice's size and its choice sets as lbib_set_overlap does.  Each trial runs
- * 1 + 2 * `steps` real time steps, so the simulation advances by about
- * 16 * `steps` steps.  choice (optional, 5 ints) receives block x, block y (0, 0: whole
- * x-rows), the overlap flag, the row-tile flag and the far-field blocks per
- * SM (0: full grid).  With overlap it also chooses the IB kernels' blocks
+ * kernel in several shapes), then (single-body contexts) the overlap of the
+ * far-field sweep with the IB stage, which its trials turn off and on whatever
+ * the lattice's size and its choice sets as lbib_set_overlap does.  Each trial
+ * runs 1 + 2 * `steps` real time steps, so the simulation advances by up to 20
+ * times as many.  choice (optional, 5 ints) receives block x, block y (0, 0:
+ * the shape by the lattice, lbib_set_sweep_config), the overlap flag, the
+ * row-tile flag and the far-field blocks per SM (0: full grid).  With overlap it also chooses the IB kernels' blocks
  * per SM (0, 1 or 2; lbib_get_launch_config reports it). */
 int lbib_autotune(void *ctx, int steps, int *choice);
 
@@ -261,7 +261,9 @@ int lbib_autotune(void *ctx, int steps, int *choice);
  * with 128-bit loads and stores; any precision with rows of whole 16-byte
  * vectors: nx a multiple of 4 in FP32/FP64, of 8 in FP16/BF16, else
  * ignored), 0 the one-node kernel with blocks of block_x * block_y threads
- * (0, 0: whole x-rows); far_per_sm > 0 runs the far-field sweep (overlap
+ * (0, 0: whole x-rows, or consecutive nodes whatever the rows where nx is no
+ * multiple of 32 and, when the lattice is swept in one part, below 2^20
+ * nodes); far_per_sm > 0 runs the far-field sweep (overlap
  * on) with that many resident blocks per SM striding over the lattice, so
  * that the IB kernels beside it find free SMs, 0 on its full grid; a context
  * whose overlap has not been set (lbib_set_overlap) overlaps with far_per_sm >
@@ -291,11 +293,15 @@ int lbib_get_launch_config(void *ctx, int *cfg);
  * Results are the same either way. */
 int lbib_set_overlap(void *ctx, int enable);
 
-/* Steps that do not store the fields run as CUDA graphs captured on first
- * use (one per phase of the six-step rotation of the population, position
- * and support-box buffers) and launched into the context stream (enable = 1,
- * default); 0 enqueues every kernel of every step.  Results are identical.
- * Adding a body, changing the overlap or autotuning recaptures. */
+/* Steps run as CUDA graphs captured on first use and launched into the
+ * context stream (enable = 1, default): one per phase of the six-step rotation
+ * of the population, position and support-box buffers; one of six steps, taken
+ * from phase 0 where none of the six stores the fields, is timed
+ * (lbib_profile) or but for the last precedes a watchdog check; and one per
+ * phase for steps that store the fields, which are enqueued kernel by kernel
+ * the first time their phase does.  0 enqueues every kernel of every step.
+ * Results are identical.  Adding a body, changing the launch configuration
+ * or autotuning recaptures. */
 int lbib_set_graphs(void *ctx, int enable);
 
 /* When the sweep also writes the macroscopic fields read by

@@ -1560,9 +1560,9 @@ __global__ void __launch_bounds__(256) kb_moments(BatchTables T, int phase) {
                        vb, nvb);
 }
 
-// Five blocks an SM (102 registers instead of 130 and three blocks): the
+// Five blocks an SM (96 registers instead of 130 and three blocks): the
 // gathers of many bodies need warps in flight (64 lattices, 618 000 points:
-// 1.091 -> 1.063 ms a step, in spite of 52 spilt bytes).
+// 1.091 -> 1.063 ms a step, in spite of 60 spilt bytes).
 template <typename R>
 __global__ void __launch_bounds__(kBatchMlsThreads, sizeof(R) == 4 ? 5 : 2) kb_mls(BatchTables T, int phase) {
     __shared__ Lattice L;
@@ -1879,8 +1879,13 @@ static cudaError_t launch_centroid(int prec, const Lattice &L, const BodyView &B
 // the membrane's hinge forces and the rigid body's preparation run beside
 // it.  Its blocks hold their registers while they wait, on SMs that a
 // far-field sweep could use, so only grids of at most this many blocks per SM
-// are launched so (96^3 capsule, 161 blocks: 45 us a step with, 49 without;
-// 160x160x480 sphere, 641 blocks: 343 with, 310 us without).
+// are launched so.  Us a step, chained / not, FP32 sphere and capsule: 96^3
+// 161 blocks 33.4 / 35.4 and 29.0 / 33.6, 257 35.0 / 36.2 and 30.4 / 34.6, 641
+// 43.6 / 44.1 and 39.5 / 43.0; where the far field is the longer part 128^3 161
+// 57.3 / 56.3 and 56.4 / 56.4, 257 59.0 / 56.6 and 57.8 / 56.5, 385 64.6 / 59.4 and
+// 62.9 / 59.7, 160x160x480 641 305.8 / 298.6 and 301.3 / 297.6; FP64 72^3 97 blocks
+// 147.0 / 147.5 and 149.7 / 173.9, 96^3 161 280.9 / 269.4 and 285.5 / 282.2, 257
+// 315.4 / 288.5 and 316.8 / 309.5.
 constexpr int kChainPerSm = 2;
 
 template <typename... KArgs, typename... Args>

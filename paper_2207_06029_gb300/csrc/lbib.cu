@@ -1020,17 +1020,24 @@ namespace {
 // unless the caller or the autotuner has said so.
 // Below kSplitCells nodes (kSplitCells64 in FP64) the step is the chain of
 // the IB kernels' latencies, and one sweep behind them is shorter than the
-// box sweep and the join.  Measured us a step, overlap against one sweep,
-// rigid sphere in FP32: 32^3 21.0 against 20.1, 48^3 24.2 against 22.6, 64^3
-// 27.7 against 25.2, 80^3 31.0 against 32.0, 96^3 38.4 against 44.5 (16-bit
-// storage and capsules alike); FP64 32^3 78.1 against 76.0, 48^3 109.8 against
-// 125.8.
+// box sweep and the join.  Us a step, overlap / one sweep, FP32 (3202 points
+// up to 56^3, 12 802 above), sphere and capsule: 32^3 20.3 / 18.2 and 17.4 /
+// 15.9, 48^3 22.3 / 19.4 and 19.7 / 17.0, 64^3 28.9 / 26.5 and 23.6 / 21.6, 72^3
+// 28.2 / 27.8 and 23.5 / 23.4, 80^3 29.6 / 29.9 and 24.9 / 25.5, 96^3 33.5 / 38.3
+// and 29.4 / 33.8; 16-bit storage alike (72^3 FP16 27.8 / 27.7, bfloat16 27.9 /
+// 28.6).  FP64 spheres: 32^3 62.0 / 47.4, 36^3 65.0 / 51.1, 40^3 65.5 / 57.8, 48^3
+// 78.8 / 71.5 (of 802 points 63.6 / 70.7), 64^3 144.6 / 140.1 (90.3 / 105.2), 96^3
+// 275.9 / 299.1.  (The FP64 line was drawn with a slower MLS kernel, which left
+// the far field more to hide; with this one the two routes cross between
+// 64 000 and 262 000 nodes by the body's size.)
 //
 // The sweeps of 16-bit storage are bound by instruction issue, so beside
 // them the IB kernels cost what they take, and on large lattices a little
-// more: 160x160x480 sphere FP16 277 against 270, bfloat16 305 against 289 (FP32
-// 305 against 319); 192^3 bfloat16 173 against 166 to 172, FP16 157 against 155
-// to 161; 160^3 bfloat16 95.6 against 94.4.
+// more.  FP16, sphere and capsule: 160^3 89.4 / 92.4 and 88.5 / 87.5, 192^3 146.7 /
+// 147.2 and 146.2 / 142.0, 208^3 182.7 / 178.1 and 182.1 / 172.9, 160x160x480
+// 234.9 / 228.0 and 233.9 / 223.0; bfloat16 144^3 74.4 / 78.0 and 74.1 / 73.4, 160^3
+// 98.8 / 100.1 and 98.1 / 95.2, 176^3 126.5 / 124.6 and 126.0 / 119.4, 160x160x480
+// 262.6 / 246.4 (FP32 there 291.8 / 302.6).
 constexpr int kSplitCells = 360000, kSplitCells64 = 48000;
 constexpr int kSplitMostFp16 = 8000000, kSplitMostBf16 = 4000000;
 bool splits_by_size(const Ctx *c) {

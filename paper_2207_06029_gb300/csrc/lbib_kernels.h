@@ -34,9 +34,11 @@ constexpr int kNodeThreads = 64;            // threads per block of the support-
 // operations but add to their number; in FP64, of which an SM quarter issues
 // a warp instruction per 64 cycles, they pay up to about a warp per quarter
 // (8 points x 608), in FP32 until the warps fill the GPU.  Us a step, four
-// lanes against one: 3 202 points FP64 52.6 against 76.0, FP32 19.3 against 22.0;
-// 12 802 points FP64 295 against 285, FP32 32.8 against 33.6; 51 202 points FP32
-// 309.3 against 303.5.
+// lanes / one, sphere and capsule at 48^3: FP32 3202 points 19.5 / 21.7 and
+// 17.0 / 18.3, 10 242 21.7 / 22.3 and 18.1 / 19.3, 12 802 22.7 / 22.3 and 18.4 /
+// 19.3, 20 482 27.3 / 24.5 and 22.5 / 19.9; FP64 3202 79.2 / 95.1 and 78.4 / 93.0,
+// 5122 82.9 / 96.1 and 85.9 / 92.1, 7682 98.5 / 95.4 and 96.7 / 103.7, 12 802 111.8 /
+// 107.1 and 124.1 / 119.2.
 inline bool mls_quads(int prec, const BodyView &B) { return B.nm + 2 * B.nt <= (prec == 0 ? 6000 : 20000); }
 // points per block; a thread per point, FP64 takes blocks of one warp, which
 // spread over more SMs

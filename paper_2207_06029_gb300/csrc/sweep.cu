@@ -6,9 +6,11 @@
 // Design: one thread per node, pull streaming f_i(x) = f*_i(x - e_i) from
 // structure-of-arrays planes (x fastest, so every population load and store
 // of a warp is one contiguous 128-byte run except at the x-wrap), read-only
-// loads through the non-coherent path and evict-first stores.  The IB force
-// lives in a dense field that is read (and zeroed) only inside tiles flagged
-// for the current step, so untouched tiles cost one cached 4-byte flag read.
+// loads through the non-coherent path and plain stores, of which the L2 keeps
+// what the next step begins with (sweep_reuse).  The IB force lives in a dense
+// field that is read, and zeroed where it is not zero, only inside tiles
+// flagged for the current step, so untouched tiles cost one cached 4-byte flag
+// read.
 #include <type_traits>
 
 #include "lbib_device.cuh"

@@ -361,7 +361,10 @@ __device__ __forceinline__ void exchange_force(const BodyView &B, int t, R area,
 //           before the first rounding (density 1.1, sphere of radius 4 to 8,
 //           error of the FP32 angular impulse against FP64: 10 to 21e-9 with
 //           the full pressures, 3 to 14e-9 as differences per triangle,
-//           3 to 14e-9 so; 32^3 FP64 sphere 50.3 -> 50.7 us a step).
+//           3 to 14e-9 so).  Its density is fetched with the moments for all
+//           points, without a branch: 48^3 FP32 sphere 18.67 us a step (18.26
+//           with the full pressures, 18.98 with a branch), 64^3 capsule 19.1 to
+//           19.2 (19.02, 19.3).
 template <typename R, bool kCG = false, bool kChain = false>
 __device__ __forceinline__ void mls_body(const R *mom, const Lattice &L, const BodyView &B, int *err,
                                          const int vb) {
@@ -480,7 +483,7 @@ __device__ __forceinline__ void mls_body(const R *mom, const Lattice &L, const B
     // the fitted values) need
     R fc[4];
     mom_load<kCG>(mom, ox[1] + oy[1] + oz[1], fc);
-    const R dr = p >= nm && B.rigid ? fc[0] - ld_ro<kCG>(mom + 4 * (size_t)ref) : fc[0];
+    const R fr = ld_ro<kCG>(mom + 4 * (size_t)(p >= nm && B.rigid ? ref : ox[1] + oy[1] + oz[1]));
     // A: 00, 01, 02, 03, 11, 12, 13, 22, 23, 33; b[c]: 1, x, y, z
     R A[10], b[4][4];
 #pragma unroll
@@ -587,7 +590,7 @@ __device__ __forceinline__ void mls_body(const R *mom, const Lattice &L, const B
             }
         const int t = (p - nm) >> 1, side = (p - nm) & 1;
         const R rn = (R(1) + (c0 + fc[0])) * pick<R>(L.nu_d, L.nu_f);
-        const R pr0 = (c0 + dr) / R(3);  // p - c_s^2 rho0 (rigid: less that of node ref)
+        const R pr0 = (c0 + (B.rigid ? fc[0] - fr : fc[0])) / R(3);  // p - c_s^2 rho0 (rigid: less that of node ref)
         R tr[3];
 #pragma unroll
         for (int c = 0; c < 3; ++c) {
@@ -773,13 +776,13 @@ __device__ __forceinline__ void mls_quad_body(const R *mom, const Lattice &L, co
         oy[i] = from(o, 1);
         oz[i] = from(o, 2);
     }
-    const int ref = B.rigid ? from(rc, 0) + L.nx * (from(rc, 1) + L.ny * from(rc, 2)) : 0;
+    const int centre = ox[1] + oy[1] + oz[1];
+    const int ref = B.rigid ? from(rc, 0) + L.nx * (from(rc, 1) + L.ny * from(rc, 2)) : centre;
     chain_wait();
 
     // ---------------- sums: field q, and A by the power of x ----------------
     const R *mq = mom + q;
-    const R fc = ld_ca(mq + 4 * (size_t)(ox[1] + oy[1] + oz[1]));
-    const R dr = B.rigid && q == 0 ? fc - ld_ca(mom + 4 * (size_t)ref) : fc;  // on lane 0
+    const R fc = ld_ca(mq + 4 * (size_t)centre), fr = ld_ca(mom + 4 * (size_t)ref);
     R b[4] = {R(0), R(0), R(0), R(0)};
     R C00 = R(0), C10 = R(0), C20 = R(0), C01 = R(0), C11 = R(0), C02 = R(0);  // y and z powers
 #pragma unroll
@@ -849,7 +852,7 @@ __device__ __forceinline__ void mls_quad_body(const R *mom, const Lattice &L, co
         if (q == c + 1) acc += col;
     }
     // p - c_s^2 rho0 (rigid: less that of node ref)
-    const R tr = (R(1) + cr) * pick<R>(L.nu_d, L.nu_f) * acc, pr0 = third(B.rigid ? from(dr + fit, 0) : cr);
+    const R tr = (R(1) + cr) * pick<R>(L.nu_d, L.nu_f) * acc, pr0 = third(from(B.rigid ? (fc - fr) + fit : val, 0));
     if (probe && !B.rigid) ((R *)B.probe + 8 * t + 4 * side)[q] = q == 0 ? pr0 : tr;
     __shared__ double red[6][kQuadThreads / 32];
     if (B.rigid) {
@@ -1562,7 +1565,7 @@ __global__ void __launch_bounds__(256) kb_moments(BatchTables T, int phase) {
 
 // Five blocks an SM (96 registers instead of 130 and three blocks): the
 // gathers of many bodies need warps in flight (64 lattices, 618 000 points:
-// 1.091 -> 1.063 ms a step, in spite of 60 spilt bytes).
+// 1.091 -> 1.063 ms a step, in spite of 44 spilt bytes).
 template <typename R>
 __global__ void __launch_bounds__(kBatchMlsThreads, sizeof(R) == 4 ? 5 : 2) kb_mls(BatchTables T, int phase) {
     __shared__ Lattice L;
